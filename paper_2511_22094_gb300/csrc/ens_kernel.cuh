@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(kEnsBlock, 4) ens_kernel(const ModelConst mc, 
         const int64_t left = ra.n_vox - v0;
         const int nv = left < VB ? static_cast<int>(left) : VB;
         __syncthreads();
-        model_smem_load<KIND>(mc);
+        model_smem_load<KIND, 1>(mc);
         {
             const float *src = ra.data + v0 * M;
             for (int e = tid; e < nv * M; e += blockDim.x) {
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kEnsBlock, 4) ens_kernel(const ModelConst mc, 
                 R th[P];
 #pragma unroll
                 for (int p = 0; p < P; ++p) th[p] = xk[p];
-                LL[lv * L + k] = loglik_any<KIND, PREC>(th, y, inv_s2, mc);
+                LL[lv * L + k] = loglik_any<KIND, PREC, 1>(th, y, inv_s2, mc);
 #pragma unroll
                 for (int p = 0; p < P; ++p) {
                     wf_mean[p * nw + lv * L + k] = W(0);
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(kEnsBlock, 4) ens_kernel(const ModelConst mc, 
                     R Lp = R(0);
                     bool acc = false;
                     if (inside) {
-                        Lp = loglik_any<KIND, PREC>(prop, y, inv_s2, mc);
+                        Lp = loglik_any<KIND, PREC, 1>(prop, y, inv_s2, mc);
                         n_bad[h] += !isfinite(Lp);
                         // log u < (P - 1) log z + L(Y) - L(X_k): the z factor
                         // enters as an offset of the likelihood difference

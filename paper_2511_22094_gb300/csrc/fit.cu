@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(kFitBlock, fit_min_blocks(PREC)) fit_step_kern
     // completed and its writes are visible
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (*fa.stop) return;  // the same for every thread
-    model_smem_load<KIND>(mc);
+    model_smem_load<KIND, 1>(mc);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int M = mc.n_meas;

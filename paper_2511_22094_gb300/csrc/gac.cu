@@ -701,6 +701,9 @@ gac_status gac_model_register(const gac_model_desc *d, int *model_id) {
         }
         const gac_status st = build_g_table(xmin, xmax, &mc);
         if (st != GAC_OK) return st;
+        mc.smt_b0 = mc.acq_f[0] == 0.0f;
+        for (int k = 1; k < mc.n_acq; ++k)
+            if (mc.acq_f[k] == 0.0f) mc.smt_b0 = 0;
     }
     if (d->kind == GAC_MODEL_AXCAL_SMT) {
         gac_status st = build_axcal(d, &mc);

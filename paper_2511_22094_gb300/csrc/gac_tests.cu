@@ -15,7 +15,7 @@ template <int KIND, int PREC>
 __global__ void forward_kernel(const ModelConst mc, const double *theta, int64_t n, double *s) {
     constexpr int P = model_n_par(KIND);
     const int M = mc.n_meas;
-    model_smem_load<KIND>(mc);
+    model_smem_load<KIND, 1>(mc);
     __syncthreads();
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -31,9 +31,9 @@ __global__ void forward_kernel(const ModelConst mc, const double *theta, int64_t
             float th[P];
             for (int p = 0; p < P; ++p) th[p] = static_cast<float>(theta[i * P + p]);
             if constexpr (model_complex(KIND))
-                eval_f<KIND>(th, mc, [&](int k, float re, float im) { out[2 * k] = re; out[2 * k + 1] = im; });
+                eval_f<KIND, 1>(th, mc, [&](int k, float re, float im) { out[2 * k] = re; out[2 * k + 1] = im; });
             else
-                eval_f<KIND>(th, mc, [&](int k, float v) { out[k] = v; });
+                eval_f<KIND, 1>(th, mc, [&](int k, float v) { out[k] = v; });
         }
     }
 }
@@ -44,14 +44,14 @@ __global__ void loglik_kernel(const ModelConst mc, const double *theta, int64_t 
     constexpr int P = model_n_par(KIND);
     using R = typename PrecTraits<PREC>::R;
     const int M = mc.n_meas;
-    model_smem_load<KIND>(mc);
+    model_smem_load<KIND, 1>(mc);
     __syncthreads();
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         R th[P];
         for (int p = 0; p < P; ++p) th[p] = static_cast<R>(theta[i * P + p]);
         const R sg = static_cast<R>(sigma[i]);
-        L[i] = static_cast<double>(loglik_any<KIND, PREC>(th, y + i * M, R(1) / (sg * sg), mc));
+        L[i] = static_cast<double>(loglik_any<KIND, PREC, 1>(th, y + i * M, R(1) / (sg * sg), mc));
     }
 }
 

@@ -51,11 +51,13 @@ namespace gac {
 constexpr int kBlock = 256;
 // Blocks per SM each kernel is compiled for (a register cap): the 3-pool
 // model needs ~118 registers (2 blocks of 256); AxCaliberSMT spills under the
-// 3-block cap of 80 registers and runs 8% faster at 2 blocks; SMT and the
-// lighter models fit 3 blocks; FP64 paths are left uncapped.
+// 3-block cap of 80 registers and runs 8% faster at 2 blocks; SMT, whose six
+// unrolled b-values would take 80 registers, runs 3% faster at 4 blocks and 64
+// (22.3 -> 21.6 ms for 150,000 voxels x 4 x 2,500); the lighter models fit 3
+// blocks; FP64 paths are left uncapped.
 template <int KIND, int PREC>
 constexpr int mh_min_blocks() {
-    return PREC == GAC_PREC_FP64 ? 1 : ((KIND == GAC_MODEL_MWI3 || KIND == GAC_MODEL_AXCAL_SMT) ? 2 : 3);
+    return PREC == GAC_PREC_FP64 ? 1 : ((KIND == GAC_MODEL_MWI3 || KIND == GAC_MODEL_AXCAL_SMT) ? 2 : (KIND == GAC_MODEL_SMT ? 4 : 3));
 }
 
 // The one-launch kernel's own block size and blocks per SM (the serving and
@@ -193,12 +195,12 @@ struct PrecTraits<GAC_PREC_FP64> {
     using Acc = PlainSumD;
 };
 
-template <int KIND, int PREC>
+template <int KIND, int PREC, int REP = gtab_copies(KIND)>
 __device__ __forceinline__ typename PrecTraits<PREC>::R loglik_any(
     const typename PrecTraits<PREC>::R *th, const float *y, typename PrecTraits<PREC>::R inv_s2,
     const ModelConst &mc) {
     if constexpr (PREC == GAC_PREC_FP64) return loglik_d<KIND>(th, y, inv_s2, mc);
-    else return loglik_f<KIND, typename PrecTraits<PREC>::Acc>(th, y, inv_s2, mc);
+    else return loglik_f<KIND, typename PrecTraits<PREC>::Acc, REP>(th, y, inv_s2, mc);
 }
 
 // MIXED acceptance, FP64 semantics at FP32 cost, from lu32 = __logf(u01_f(w)).

@@ -107,6 +107,7 @@ struct ModelConst {
     int gtab_n;
     int gtab_tail;
     float gtab_tail_x;
+    int smt_b0;  // SMT: the first b-value is 0 and no other
     AxConst ax;  // GAC_MODEL_AXCAL_SMT only
 };
 
@@ -128,25 +129,39 @@ constexpr double kSqrtPiHalfD = 0.886226925452758014;
 // ---------------------------------------------------------------- g(x) ----
 // The g(x) table of the block's model, copied from ModelConst by
 // model_smem_load before the first evaluation (the lookups of a warp go to
-// different intervals, which the constant bank would serialise).
+// different intervals, which the constant bank would serialise).  REP = 8: eight
+// copies side by side.  A 16-byte load is served eight lanes at a time, and with
+// lane l reading copy l % 8 no two of them meet in a bank.  The AxCaliberSMT MH
+// kernels, bound by shared-memory wavefronts (64 such loads an evaluation; 346
+// wavefronts of a warp's 425 cycles an SM, 71 of them conflicts) and holding 2
+// blocks an SM by registers, take it: 23.9 -> 23.5 ms for 25,001 voxels x 4 x
+// 5,000.  SMT (12 loads) gained 0.5% and keeps one copy, and so do the ensemble
+// kernels, whose walkers need the shared memory (64 walkers with moments over
+// every state lost a block an SM to the copies: 7.7 -> 8.1 ms).
+__host__ __device__ constexpr int gtab_copies(int kind) { return kind == GAC_MODEL_AXCAL_SMT ? 8 : 1; }
 static __shared__ float4 smt_gtab_s[2 * kGTabMax];
+static __shared__ float4 smt_gtab_r[2 * kGTabMax * 8];
 
-// The AxCaliberSMT series table and per-measurement constants of the
-// block's model (FP32 path).
+// The AxCaliberSMT series table of the block's model (FP32 path).
 static __shared__ float4 ax_tab_s[kAxMaxTiming * 2 * kAxTabMax];
-static __shared__ float4 ax_meas_s[kAxMaxMeas * 2];
 
-template <int KIND>
+template <int KIND, int REP = gtab_copies(KIND)>
 __device__ __forceinline__ void model_smem_load(const ModelConst &mc) {
     if constexpr (KIND == GAC_MODEL_SMT || KIND == GAC_MODEL_AXCAL_SMT) {
-        float *dst = reinterpret_cast<float *>(smt_gtab_s);
-        for (int e = threadIdx.x; e < 2 * kGTabMax * 4; e += blockDim.x) dst[e] = mc.gtab[e];
+        const float4 *src = reinterpret_cast<const float4 *>(mc.gtab);
+        for (int e = threadIdx.x; e < 2 * kGTabMax; e += blockDim.x) {
+            const float4 q = src[e];
+            if constexpr (REP == 1) {
+                smt_gtab_s[e] = q;
+            } else {
+#pragma unroll
+                for (int r = 0; r < REP; ++r) smt_gtab_r[e * REP + ((r + e) & (REP - 1))] = q;
+            }
+        }
     }
     if constexpr (KIND == GAC_MODEL_AXCAL_SMT) {
         float *dst = reinterpret_cast<float *>(ax_tab_s);
         for (int e = threadIdx.x; e < kAxMaxTiming * 2 * kAxTabMax * 4; e += blockDim.x) dst[e] = mc.ax.tab[e];
-        float *dm = reinterpret_cast<float *>(ax_meas_s);
-        for (int e = threadIdx.x; e < kAxMaxMeas * 2 * 4; e += blockDim.x) dm[e] = mc.ax.meas[e];
     }
 }
 
@@ -164,7 +179,7 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // gtab_tail_x takes the asymptote sqrt(pi)/2 x^-1/2 instead (relative error
 // below erfc(4)); without it the table covers every argument the bounds
 // allow.  The clamped index keeps every load inside the table for any x.
-template <bool TAIL>
+template <bool TAIL, int REP>
 __device__ __forceinline__ float smt_g_f(float x, const ModelConst &mc) {
     constexpr float kRound = 12582912.0f;  // 1.5 * 2^23
     const float t = fmaf(x, 2.0f, kRound);
@@ -173,8 +188,9 @@ __device__ __forceinline__ float smt_g_f(float x, const ModelConst &mc) {
     // to a large unsigned value)
     const int i = static_cast<int>(min(static_cast<unsigned>(__float_as_int(t) - __float_as_int(kRound) - mc.gtab_lo),
                                        static_cast<unsigned>(mc.gtab_n - 1)));
-    const float4 lo = smt_gtab_s[i];
-    const float4 hi = smt_gtab_s[kGTabMax + i];
+    const float4 *tab = REP == 1 ? smt_gtab_s : smt_gtab_r + (threadIdx.x & (REP - 1));
+    const float4 lo = tab[i * REP];
+    const float4 hi = tab[(kGTabMax + i) * REP];
     float p = fmaf(hi.y, d, hi.x);
     p = fmaf(p, d, lo.w);
     p = fmaf(p, d, lo.z);
@@ -638,33 +654,56 @@ __device__ __forceinline__ void eval_mwi3_f(const float *th, const ModelConst &m
     }
 }
 
-template <bool TAIL, class V>
-__device__ __forceinline__ void eval_smt_f(const float *th, const ModelConst &mc, V &&visit) {
+// S(b = 0) = S0 = 1 exactly.  SEL: any measurement may be b = 0 (a select, no
+// branch); otherwise only the first one is, and its two lookups are left out
+// (registration sets smt_b0 for such protocols; of the benchmark's six b-values
+// it saves a sixth of the evaluation).
+template <bool TAIL, bool SEL, class V>
+__device__ __forceinline__ void eval_smt_blocks_f(const float *th, const ModelConst &mc, V &visit) {
     const float f = th[0], da = th[1], dpar = th[2], dperp = th[3];
     const float ddiff = dpar - dperp;
     const int n = mc.n_acq;
-    // S(b = 0) = S0 = 1 exactly, by a select (no branch); blocks of kAnchor
-    // b-values unrolled, and a protocol of at most kAnchor b-values (one
-    // block, the same for every thread) reads them at fixed offsets
     auto one = [&](int k) {
         const float b = mc.acq_f[k];
-        const float intra = smt_g_f<TAIL>(b * da, mc);
-        const float extra = ex2_approx(-mc.acq_l2e_f[k] * dperp) * smt_g_f<TAIL>(b * ddiff, mc);
-        visit(k, b == 0.0f ? 1.0f : fmaf(f, intra, (1.0f - f) * extra));
+        const float intra = smt_g_f<TAIL, 1>(b * da, mc);
+        const float extra = ex2_approx(-mc.acq_l2e_f[k] * dperp) * smt_g_f<TAIL, 1>(b * ddiff, mc);
+        const float s = fmaf(f, intra, (1.0f - f) * extra);
+        visit(k, SEL && b == 0.0f ? 1.0f : s);
     };
-    if (n <= kAnchor) {
+    auto first = [&](int k) {
+        if (!SEL && k == 0) visit(0, 1.0f);  // the same branch for every thread
+        else one(k);
+    };
+    // a full block has no test between its b-values, so their table lookups
+    // overlap; a protocol of one block reads them at fixed offsets; only a
+    // last, partial block tests
+    if (n == kAnchor) {
+        first(0);
 #pragma unroll
-        for (int k = 0; k < kAnchor; ++k)
-            if (k < n) one(k);
+        for (int k = 1; k < kAnchor; ++k) one(k);
         end_block(visit, 0);
         return;
     }
-    for (int k0 = 0; k0 < n; k0 += kAnchor) {
+    int k0 = 0;
+    for (; k0 + kAnchor <= n; k0 += kAnchor) {
+        first(k0);
 #pragma unroll
-        for (int i = 0; i < kAnchor; ++i)
+        for (int i = 1; i < kAnchor; ++i) one(k0 + i);
+        end_block(visit, 0);
+    }
+    if (k0 < n) {
+        first(k0);
+#pragma unroll
+        for (int i = 1; i < kAnchor; ++i)
             if (k0 + i < n) one(k0 + i);
         end_block(visit, 0);
     }
+}
+
+template <bool TAIL, class V>
+__device__ __forceinline__ void eval_smt_f(const float *th, const ModelConst &mc, V &&visit) {
+    if (mc.smt_b0) eval_smt_blocks_f<TAIL, false>(th, mc, visit);  // the same branch for every thread
+    else eval_smt_blocks_f<TAIL, true>(th, mc, visit);
 }
 
 // The cylinder's Gaussian-phase attenuation (Neuman 1974; van Gelderen et al.
@@ -748,9 +787,12 @@ __device__ __forceinline__ void ax_phi_table_f(float R, const AxConst &ax, float
 }
 
 // Measurements in timing order, so that the timing's attenuation phi_j is a
-// loop constant; per measurement two 16-byte shared-memory loads bring
-// b Da, g2, g2 log2 e, b log2 e, b, e^{-b D_csf} and the measurement's index.
-template <bool TAIL, class V>
+// loop constant; per measurement b Da, g2, g2 log2 e, b log2 e, b, e^{-b D_csf}
+// and the measurement's index come from the kernel parameters (the same address
+// for every thread: no shared-memory wavefronts, of which the table lookups
+// leave few; 24.6 -> 23.5 ms for 25,001 voxels x 4 x 5,000).  A full block's
+// lookups overlap, and so do those of a pair of the rest.
+template <bool TAIL, int REP, class V>
 __device__ __forceinline__ void eval_axcal_f(const float *th, const ModelConst &mc, V &&visit) {
     const AxConst &ax = mc.ax;
     const float R = 0.5f * th[0], fn = th[1], fcsf = th[2], der = th[3];
@@ -763,14 +805,25 @@ __device__ __forceinline__ void eval_axcal_f(const float *th, const ModelConst &
         const int end = ax.first[j + 1];
         for (int i0 = ax.first[j]; i0 < end; i0 += kAnchor) {
             const int i1 = min(i0 + kAnchor, end);
-            for (int i = i0; i < i1; ++i) {
-                const float4 A = ax_meas_s[2 * i], B = ax_meas_s[2 * i + 1];
+            auto one = [&](int i) {
+                const float4 A = reinterpret_cast<const float4 *>(ax.meas)[2 * i], B = reinterpret_cast<const float4 *>(ax.meas)[2 * i + 1];
                 // restricted: e^{-kappa} g(b Da - kappa), kappa = g2 phi_j
-                const float sr = ex2_approx(A.z * nph) * smt_g_f<TAIL>(fmaf(A.y, nph, A.x), mc);
+                const float sr = ex2_approx(A.z * nph) * smt_g_f<TAIL, REP>(fmaf(A.y, nph, A.x), mc);
                 // hindered: e^{-b De_R} g(b (De_par - De_R))
-                const float sh = ex2_approx(-A.w * der) * smt_g_f<TAIL>(B.x * dh, mc);
+                const float sh = ex2_approx(-A.w * der) * smt_g_f<TAIL, REP>(B.x * dh, mc);
                 visit(__float_as_int(B.z), fmaf(w_r, sr, fmaf(w_h, sh, fcsf * B.y)));
+            };
+            int i = i0;
+            if (i + kAnchor == i1) {
+#pragma unroll
+                for (int k = 0; k < kAnchor; ++k) one(i0 + k);
+                i = i1;
             }
+            for (; i + 1 < i1; i += 2) {
+                one(i);
+                one(i + 1);
+            }
+            if (i < i1) one(i);
             end_block(visit, 0);
         }
     }
@@ -859,7 +912,7 @@ __device__ __forceinline__ void eval_linear_d(const double *th, const ModelConst
 }
 
 // --------------------------------------------------------- dispatch by kind
-template <int KIND, class V>
+template <int KIND, int REP = gtab_copies(KIND), class V>
 __device__ __forceinline__ void eval_f(const float *th, const ModelConst &mc, V &&visit) {
     if constexpr (KIND == GAC_MODEL_MONOEXP) eval_monoexp_f(th, mc, visit);
     else if constexpr (KIND == GAC_MODEL_MWI3) eval_mwi3_f(th, mc, visit);
@@ -867,8 +920,8 @@ __device__ __forceinline__ void eval_f(const float *th, const ModelConst &mc, V 
         if (mc.gtab_tail) eval_smt_f<true>(th, mc, visit);  // the same branch for every thread
         else eval_smt_f<false>(th, mc, visit);
     } else if constexpr (KIND == GAC_MODEL_AXCAL_SMT) {
-        if (mc.gtab_tail) eval_axcal_f<true>(th, mc, visit);
-        else eval_axcal_f<false>(th, mc, visit);
+        if (mc.gtab_tail) eval_axcal_f<true, REP>(th, mc, visit);
+        else eval_axcal_f<false, REP>(th, mc, visit);
     }
     else eval_linear_f(th, mc, visit);
 }
@@ -936,11 +989,11 @@ struct ResidualVisitor {
     __device__ __forceinline__ void block_end() const { acc.block_end(); }
 };
 
-template <int KIND, class ACC>
+template <int KIND, class ACC, int REP = gtab_copies(KIND)>
 __device__ __forceinline__ float loglik_f(const float *th, const float *y, float inv_s2,
                                           const ModelConst &mc) {
     ACC acc;
-    eval_f<KIND>(th, mc, ResidualVisitor<ACC>{acc, y});
+    eval_f<KIND, REP>(th, mc, ResidualVisitor<ACC>{acc, y});
     return -0.5f * acc.value() * inv_s2;
 }
 
