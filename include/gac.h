@@ -133,7 +133,10 @@ typedef struct {
                             GAC_ERR_INVALID_ARG otherwise).  Results do not
                             depend on it, bit for bit; the library uses lanes
                             when the chains are too few to give every SM
-                            sub-partition a warp. */
+                            sub-partition a warp: as here, or, for any model,
+                            4 to 32 lanes a chain that evaluate the proposals
+                            of its next 2 to 5 iterations at once, one for
+                            every outcome of the decisions between them. */
 } gac_mcmc_opts;
 
 /* Step adaptation during burn-in (an extension; the paper has no

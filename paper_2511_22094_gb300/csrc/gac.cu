@@ -14,7 +14,7 @@
 #include "gac.h"
 #include "gac_internal.h"
 #include "launch.h"
-#include "mh_split.cuh"
+#include "mh_spec.cuh"
 
 namespace gac {
 
@@ -575,6 +575,95 @@ static gac_status plan_split(const ModelConst &mc, int G, int C, int64_t n_vox, 
     return GAC_OK;
 }
 
+static const void *mh_spec_ptr(int kind, int depth, bool all) {
+    switch (kind) {
+    case GAC_MODEL_MONOEXP: return mh_spec_ptr_monoexp(depth, all);
+    case GAC_MODEL_MWI3: return mh_spec_ptr_mwi3(depth, all);
+    case GAC_MODEL_SMT: return mh_spec_ptr_smt(depth, all);
+    case GAC_MODEL_AXCAL_SMT: return mh_spec_ptr_axcal(depth, all);
+    default: return nullptr;
+    }
+}
+
+// Blocks of a speculative launch: the warps spread evenly over the SMs in
+// blocks of whole voxels.
+struct SpecShape {
+    int threads, vb;
+    int64_t n_tiles;
+    int64_t warps() const { return n_tiles * (threads / 32); }
+};
+static SpecShape spec_shape(int depth, int C, int64_t n_vox) {
+    const int G = 1 << depth, sms = sm_count();
+    const int64_t warps_per_sm = ((n_vox * C * G + 31) / 32 + sms - 1) / sms;
+    const int64_t blocks_per_sm = (warps_per_sm * 32 + kSpecBlock - 1) / kSpecBlock;
+    SpecShape sh;
+    sh.threads = static_cast<int>(32 * ((warps_per_sm + blocks_per_sm - 1) / blocks_per_sm));
+    sh.threads = std::max(sh.threads, 32 * ((C * G + 31) / 32));  // at least one voxel
+    sh.vb = std::max(1, sh.threads / (C * G));
+    sh.n_tiles = (n_vox + sh.vb - 1) / sh.vb;
+    return sh;
+}
+
+// Depth of the speculation tree (mh_spec.cuh) for a gac_mcmc_run, 0 for none:
+// the deepest tree whose warps find idle schedulers.  Measured on GB300 (ms
+// per 1,000 iterations, 1 chain a voxel):
+//   chains           200    1,200  2,400  4,800  9,600  14,400  19,200
+//   3-pool    one    1.14   1.21   1.21   1.22   1.22   1.71    1.72
+//             spec   0.31   0.37   0.47   0.67   0.96   1.31    1.61
+//             depth  5      4      3      2      2      2       2
+//   SMT       one    0.58   0.59   0.59   0.60   0.60   0.60    0.61
+//             spec   0.15   0.18   0.22   0.28   0.41   0.52    0.63
+//             depth  5      4      3      3      2      2       -
+//   AxCaliber one    1.58   1.60   1.60   1.61   1.61   2.00    1.99
+//             spec   0.40   0.49   0.62   0.77   1.10   1.41    1.68
+//             depth  5      4      3      3      2      2       2
+//   mono-exp  split  0.19   0.20   0.20   0.20   0.19   0.26    0.26
+//             spec   0.14   0.17   -      -      -      -       -
+// A round of the trees of depth 3 and more takes as long with a second warp on
+// its scheduler only where it waits on table lookups (SMT, AxCaliberSMT); the
+// 3-pool round issues paired multiply-adds for most of its cycles.  Depth 2
+// doubles the work per iteration and halves the serial path: it pays up to
+// four warps a scheduler, for SMT (whose one-thread kernel keeps 32 warps an SM)
+// up to three.  The mono-exponential round is short enough that the lane-split
+// kernel's shorter path wins where it applies (`split`) once two warps share
+// a scheduler.
+static int choose_depth(const ModelConst &mc, const gac_mcmc_opts *o, int64_t n_vox, bool split) {
+    if (o->precision != GAC_PREC_MIXED || o->trace_n_vox != 0 || o->lanes_per_chain != 0 ||
+        !mh_spec_ptr(mc.kind, 2, false))
+        return 0;
+    const int C = o->n_chains;
+    const int64_t schedulers = static_cast<int64_t>(sm_count()) * 4;
+    const bool mwi3 = mc.kind == GAC_MODEL_MWI3, mono = mc.kind == GAC_MODEL_MONOEXP;
+    for (int depth = 5; depth >= 2; --depth) {
+        if (C << depth > kSpecBlock || n_vox * C > (schedulers * 32 * 4 >> depth)) continue;
+        const int per = depth >= 4 ? 1 : depth == 3 ? (mwi3 || mono ? 1 : 2) : mc.kind == GAC_MODEL_SMT ? 3 : 4;
+        if (depth < 4 && mono && split) return 0;
+        if (spec_shape(depth, C, n_vox).warps() <= per * schedulers) return depth;
+    }
+    return 0;
+}
+
+static gac_status plan_spec(const ModelConst &mc, int depth, int C, int64_t n_vox, int moments_mode, LaunchCfg *cfg,
+                            int64_t *n_tiles, int *vb) {
+    const bool all = moments_mode == GAC_MOMENTS_ALL_POSTBURNIN;
+    const void *fn = mh_spec_ptr(mc.kind, depth, all);
+    if (!fn) return fail(GAC_ERR_INVALID_ARG, "no speculative kernel for kind %d of depth %d", mc.kind, depth);
+    const SpecShape sh = spec_shape(depth, C, n_vox);
+    const size_t smem = spec_smem_bytes(mc.n_par, 1 << depth, sh.threads, sh.vb, row_stride_for(mc.kind, mc.n_meas), all);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    int per_sm = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, sh.threads, smem);
+    if (e != cudaSuccess) return cuda_fail(e, "speculative kernel occupancy");
+    if (per_sm < 1) return fail(GAC_ERR_INVALID_ARG, "speculative kernel does not fit on an SM (smem %zu)", smem);
+    *vb = sh.vb;
+    *n_tiles = sh.n_tiles;
+    cfg->grid = static_cast<int>(std::min<int64_t>(sh.n_tiles, static_cast<int64_t>(per_sm) * sm_count()));
+    cfg->smem = smem;
+    cfg->block = sh.threads;
+    return GAC_OK;
+}
+
 }  // namespace gac
 
 using namespace gac;
@@ -804,7 +893,10 @@ gac_status gac_mcmc_run(int model_id, const void *data, int64_t n_vox, const flo
     LaunchCfg cfg;
     int64_t n_tiles = 0;
     int vb = 0;
-    st = lanes > 1 ? plan_split(mc, lanes, C, n_vox, o->moments_mode, &cfg, &n_tiles, &vb)
+    const int depth = choose_depth(mc, o, n_vox, lanes > 1);
+    const bool all = o->moments_mode == GAC_MOMENTS_ALL_POSTBURNIN;
+    st = depth > 0 ? plan_spec(mc, depth, C, n_vox, o->moments_mode, &cfg, &n_tiles, &vb)
+       : lanes > 1 ? plan_split(mc, lanes, C, n_vox, o->moments_mode, &cfg, &n_tiles, &vb)
                    : plan_launch(mc, o->precision, trace, C, n_vox, o->moments_mode, &cfg, &n_tiles, &vb);
     if (st != GAC_OK) return st;
     cfg.stream = s;
@@ -840,10 +932,12 @@ gac_status gac_mcmc_run(int model_id, const void *data, int64_t n_vox, const flo
     ra.rhat = static_cast<double *>(d_rhat.ptr);
     ra.step_scale = static_cast<float *>(d_scale.ptr);
 
-    cudaError_t e = lanes == 1 ? launch_mh(mc.kind, o->precision, trace, mc, ra, cfg)
+    void *args[] = {&mc, &ra};
+    cudaError_t e = depth > 0 ? cudaLaunchKernel(mh_spec_ptr(mc.kind, depth, all), dim3(cfg.grid), dim3(cfg.block), args, cfg.smem, s)
+                    : lanes == 1 ? launch_mh(mc.kind, o->precision, trace, mc, ra, cfg)
                     : mc.kind == GAC_MODEL_MONOEXP
-                        ? launch_mh_split_monoexp(lanes, o->moments_mode == GAC_MOMENTS_ALL_POSTBURNIN, mc, ra, cfg)
-                        : launch_mh_split_mwi3(lanes, o->moments_mode == GAC_MOMENTS_ALL_POSTBURNIN, mc, ra, cfg);
+                        ? launch_mh_split_monoexp(lanes, all, mc, ra, cfg)
+                        : launch_mh_split_mwi3(lanes, all, mc, ra, cfg);
     if (e != cudaSuccess) return cuda_fail(e, "MH kernel launch");
     for (DevBuf *b : {&d_mean, &d_std, &d_samples, &d_acc, &d_bad, &d_trace, &d_rhat, &d_scale})
         if ((st = b->copy_out()) != GAC_OK) return st;

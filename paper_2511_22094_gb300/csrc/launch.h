@@ -31,6 +31,12 @@ const void *mh_split_ptr_monoexp(int G, bool all);
 const void *mh_split_ptr_mwi3(int G, bool all);
 cudaError_t launch_mh_split_monoexp(int G, bool all, const ModelConst &mc, const RunArgs &ra, const LaunchCfg &cfg);
 cudaError_t launch_mh_split_mwi3(int G, bool all, const ModelConst &mc, const RunArgs &ra, const LaunchCfg &cfg);
+// Speculative kernels (mh_spec.cuh): trees of depth 2..5, MIXED; launched with
+// cudaLaunchKernel(ptr, ..., {&mc, &ra}).
+const void *mh_spec_ptr_monoexp(int depth, bool all);
+const void *mh_spec_ptr_mwi3(int depth, bool all);
+const void *mh_spec_ptr_smt(int depth, bool all);
+const void *mh_spec_ptr_axcal(int depth, bool all);
 cudaError_t launch_mh_monoexp(int prec, bool trace, const ModelConst &mc, const RunArgs &ra, const LaunchCfg &cfg);
 cudaError_t launch_mh_mwi3(int prec, bool trace, const ModelConst &mc, const RunArgs &ra, const LaunchCfg &cfg);
 cudaError_t launch_mh_smt(int prec, bool trace, const ModelConst &mc, const RunArgs &ra, const LaunchCfg &cfg);
