@@ -3,6 +3,7 @@
 // same device functions as the sampler.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 
 #include "gac.h"
@@ -11,30 +12,76 @@
 
 namespace gac {
 
-template <int KIND, int PREC>
-__global__ void forward_kernel(const ModelConst mc, const double *theta, int64_t n, double *s) {
+// FP64: a thread per parameter vector, which writes its row as it evaluates.
+template <int KIND>
+__global__ void forward_d_kernel(const ModelConst mc, const double *theta, int64_t n, double *s) {
     constexpr int P = model_n_par(KIND);
     const int M = mc.n_meas;
-    model_smem_load<KIND, 1>(mc);
-    __syncthreads();
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         double *out = s + i * M;
-        if constexpr (PREC == GAC_PREC_FP64) {
-            double th[P];
-            for (int p = 0; p < P; ++p) th[p] = theta[i * P + p];
-            if constexpr (model_complex(KIND))
-                eval_d<KIND>(th, mc, [&](int k, double re, double im) { out[2 * k] = re; out[2 * k + 1] = im; });
-            else
-                eval_d<KIND>(th, mc, [&](int k, double v) { out[k] = v; });
-        } else {
-            float th[P];
-            for (int p = 0; p < P; ++p) th[p] = static_cast<float>(theta[i * P + p]);
-            if constexpr (model_complex(KIND))
-                eval_f<KIND, 1>(th, mc, [&](int k, float re, float im) { out[2 * k] = re; out[2 * k + 1] = im; });
-            else
-                eval_f<KIND, 1>(th, mc, [&](int k, float v) { out[k] = v; });
+        double th[P];
+        for (int p = 0; p < P; ++p) th[p] = theta[i * P + p];
+        if constexpr (model_complex(KIND))
+            eval_d<KIND>(th, mc, [&](int k, double re, double im) { out[2 * k] = re; out[2 * k + 1] = im; });
+        else
+            eval_d<KIND>(th, mc, [&](int k, double v) { out[k] = v; });
+    }
+}
+
+// FP32 arithmetic (the MIXED and FP32 paths share the forward model): bound by
+// the bytes of its rows, so they cross shared memory.  A warp takes 32
+// consecutive parameter vectors: it reads them as one contiguous piece, each
+// lane evaluates one of them into its row of the warp's tile, and the warp
+// writes the 32 rows as one contiguous piece.  (A thread writing its own row
+// touched 32 lines with every store: 3-pool, 24 echoes, 500,000 vectors took
+// 292 us a call, 73 so, of which about 20 are the launch and the wait of any
+// call; their 228 MB cross HBM in 34.)
+constexpr int kFwdBlock = 128;
+template <int KIND>
+__global__ void __launch_bounds__(kFwdBlock) forward_f_kernel(const ModelConst mc, const double *theta, int64_t n,
+                                                              double *s, int row_stride) {
+    constexpr int P = model_n_par(KIND);
+    extern __shared__ __align__(16) float fwd_rows[];
+    const int M = mc.n_meas;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float *tile = fwd_rows + warp * 32 * row_stride;
+    model_smem_load<KIND, 1>(mc);
+    __syncthreads();
+    const int64_t tiles = (n + 31) / 32;
+    for (int64_t t = blockIdx.x * static_cast<int64_t>(kFwdBlock / 32) + warp; t < tiles;
+         t += static_cast<int64_t>(gridDim.x) * (kFwdBlock / 32)) {
+        const int64_t left = n - t * 32;
+        const int rows = left < 32 ? static_cast<int>(left) : 32;
+        const double *src = theta + t * 32 * P;
+        float th[P];
+#pragma unroll
+        for (int p = 0; p < P; ++p)  // row_stride >= P (the host sees to it)
+            if (lane + 32 * p < rows * P) tile[lane + 32 * p] = static_cast<float>(src[lane + 32 * p]);
+        __syncwarp();
+        const int r = min(lane, rows - 1);  // a lane without a vector repeats the last
+#pragma unroll
+        for (int p = 0; p < P; ++p) th[p] = tile[r * P + p];
+        __syncwarp();
+        float *row = tile + lane * row_stride;
+        if constexpr (model_complex(KIND))
+            eval_f<KIND, 1>(th, mc, [&](int k, float re, float im) { reinterpret_cast<float2 *>(row)[k] = make_float2(re, im); });
+        else
+            eval_f<KIND, 1>(th, mc, [&](int k, float v) { row[k] = v; });
+        __syncwarp();
+        double *out = s + t * 32 * M;
+        int q = lane / M, col = lane - q * M;  // element e = lane + 32 i of the rows as one piece
+        const int dq = 32 / M, dc = 32 - dq * M;
+        for (int e = lane; e < rows * M; e += 32) {
+            out[e] = static_cast<double>(tile[q * row_stride + col]);
+            q += dq;
+            col += dc;
+            if (col >= M) {
+                col -= M;
+                ++q;
+            }
         }
+        __syncwarp();
     }
 }
 
@@ -99,11 +146,20 @@ static int grid_for(int64_t n) {
 template <int KIND>
 static cudaError_t launch_forward(int prec, const ModelConst &mc, const double *th, int64_t n, double *s,
                                   cudaStream_t st) {
-    switch (prec) {
-    case GAC_PREC_MIXED: forward_kernel<KIND, GAC_PREC_MIXED><<<grid_for(n), 256, 0, st>>>(mc, th, n, s); break;
-    case GAC_PREC_FP32: forward_kernel<KIND, GAC_PREC_FP32><<<grid_for(n), 256, 0, st>>>(mc, th, n, s); break;
-    default: forward_kernel<KIND, GAC_PREC_FP64><<<grid_for(n), 256, 0, st>>>(mc, th, n, s); break;
+    if (prec == GAC_PREC_FP64) {
+        forward_d_kernel<KIND><<<grid_for(n), 256, 0, st>>>(mc, th, n, s);
+        return cudaGetLastError();
     }
+    const int row_stride = row_stride_for(KIND, std::max(mc.n_meas, mc.n_par));
+    const size_t smem = static_cast<size_t>(kFwdBlock) * row_stride * sizeof(float);
+    if (smem > 44 * 1024) {  // beside the model's tables, past the default 48 KB
+        const cudaError_t e = cudaFuncSetAttribute(forward_f_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   static_cast<int>(smem));
+        if (e != cudaSuccess) return e;
+    }
+    const int64_t blocks = (n + kFwdBlock - 1) / kFwdBlock;
+    const int grid = static_cast<int>(std::min<int64_t>(blocks, 152 * 8));  // 8 blocks on each SM: one wave
+    forward_f_kernel<KIND><<<grid, kFwdBlock, smem, st>>>(mc, th, n, s, row_stride);
     return cudaGetLastError();
 }
 

@@ -41,3 +41,31 @@ def test_blocks_of_measurements(gac, orc, w, name, acq):
     L = gac.loglik_host(mid, th, y, sig)
     L64 = -0.5 * (((y.astype(np.float64) - want) / sig[:, None].astype(np.float64)) ** 2).sum(1)
     assert (np.abs(L - L64) <= 1e-3 + 5e-5 * np.abs(L64)).all()
+
+
+@pytest.mark.parametrize("kind", ["monoexp", "mwi3", "linear"])
+@pytest.mark.parametrize("n_acq", [1, 2, 7, 33, 64])
+def test_forward_rows(gac, orc, kind, n_acq):
+    """Forward rows written by warps of 32 vectors: ragged counts, and rows shorter and longer
+    than a warp, against the oracle (1e-5 relative norm) and against one vector at a time (equal)."""
+    w = {"monoexp": W.MONOEXP_4K, "mwi3": W.MWI3_1M}.get(kind)
+    acq = 2.0 + 0.7 * np.arange(n_acq)
+    k, lb, ub = (W.LINEAR, (-2.0, -3.0), (2.0, 3.0)) if w is None else (w.kind, w.lb, w.ub)
+    mid = gac.gac_model_register(k, acq, lb, ub, np.ones(len(lb)))
+    rng = np.random.default_rng(n_acq)
+    for n in (1, 31, 33, 1000):
+        th = rng.uniform(lb, ub, (n, len(lb))).astype(np.float32).astype(np.float64)
+        want, got = orc.forward(k, acq, th), gac.forward_host(mid, th)
+        scale = np.linalg.norm(want, axis=1) if k != W.LINEAR else 4.0 + 3.0 * np.abs(acq).max()
+        assert (np.linalg.norm(got - want, axis=1) <= 1e-5 * scale).all()
+        for i in {0, n // 2, n - 1}:
+            np.testing.assert_array_equal(gac.forward_host(mid, th[i])[0], got[i])
+
+
+def test_forward_more_vectors_than_a_wave(gac, orc):
+    w = W.MONOEXP_4K
+    mid = gac.gac_model_register(w.kind, w.acq[:3], w.lb, w.ub, w.step)
+    n = 200_001
+    th = W.truths(w.with_(n_vox=n), 0, n).astype(np.float32).astype(np.float64)
+    want, got = orc.forward(w.kind, w.acq[:3], th), gac.forward_host(mid, th)
+    assert (np.linalg.norm(got - want, axis=1) <= 1e-5 * np.linalg.norm(want, axis=1)).all()
