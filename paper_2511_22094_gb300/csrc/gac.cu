@@ -410,93 +410,102 @@ int row_stride_for(int kind, int M) {
     return M | 1;
 }
 
-template <int KIND>
-static int block_of(int prec) {
-    switch (prec) {
-    case GAC_PREC_MIXED: return mh_block<KIND, GAC_PREC_MIXED>();
-    case GAC_PREC_FP32: return mh_block<KIND, GAC_PREC_FP32>();
-    default: return mh_block<KIND, GAC_PREC_FP64>();
-    }
-}
-
-// Threads per block of the one-launch kernel for (kind, precision).
-int mh_block_size(int kind, int prec) {
-    switch (kind) {
-    case GAC_MODEL_MONOEXP: return block_of<GAC_MODEL_MONOEXP>(prec);
-    case GAC_MODEL_MWI3: return block_of<GAC_MODEL_MWI3>(prec);
-    case GAC_MODEL_SMT: return block_of<GAC_MODEL_SMT>(prec);
-    case GAC_MODEL_AXCAL_SMT: return block_of<GAC_MODEL_AXCAL_SMT>(prec);
-    default: return block_of<GAC_MODEL_LINEAR_TEST>(prec);
-    }
-}
-
-size_t smem_bytes_for(int kind, int prec, int C, int M, int moments_mode) {
+static size_t smem_bytes_for(int kind, int prec, int C, int M, int moments_mode, int block) {
     const size_t w = (prec == GAC_PREC_FP32) ? sizeof(float) : sizeof(double);
     const bool blocked = prec == GAC_PREC_MIXED && moments_mode == GAC_MOMENTS_ALL_POSTBURNIN;
-    const int block = mh_block_size(kind, prec);
     return tile_smem_bytes(model_n_par(kind), w, block / C, row_stride_for(kind, M), true, blocked, block);
 }
 
-const void *mh_kernel_ptr(int kind, int prec, bool trace) {
+static const void *mh_kernel_ptr(int kind, int prec, bool trace, int block) {
     switch (kind) {
-    case GAC_MODEL_MONOEXP: return mh_ptr_monoexp(prec, trace);
-    case GAC_MODEL_MWI3: return mh_ptr_mwi3(prec, trace);
-    case GAC_MODEL_SMT: return mh_ptr_smt(prec, trace);
-    case GAC_MODEL_AXCAL_SMT: return mh_ptr_axcal(prec, trace);
-    case GAC_MODEL_LINEAR_TEST: return mh_ptr_linear(prec, trace);
+    case GAC_MODEL_MONOEXP: return mh_ptr_monoexp(prec, trace, block);
+    case GAC_MODEL_MWI3: return mh_ptr_mwi3(prec, trace, block);
+    case GAC_MODEL_SMT: return mh_ptr_smt(prec, trace, block);
+    case GAC_MODEL_AXCAL_SMT: return mh_ptr_axcal(prec, trace, block);
+    case GAC_MODEL_LINEAR_TEST: return mh_ptr_linear(prec, trace, block);
     default: return nullptr;
     }
 }
 
-cudaError_t launch_mh(int kind, int prec, bool trace, const ModelConst &mc, const RunArgs &ra,
-                      const LaunchCfg &cfg) {
-    switch (kind) {
-    case GAC_MODEL_MONOEXP: return launch_mh_monoexp(prec, trace, mc, ra, cfg);
-    case GAC_MODEL_MWI3: return launch_mh_mwi3(prec, trace, mc, ra, cfg);
-    case GAC_MODEL_SMT: return launch_mh_smt(prec, trace, mc, ra, cfg);
-    case GAC_MODEL_AXCAL_SMT: return launch_mh_axcal(prec, trace, mc, ra, cfg);
-    case GAC_MODEL_LINEAR_TEST: return launch_mh_linear(prec, trace, mc, ra, cfg);
-    default: return cudaErrorInvalidValue;
-    }
-}
-
-// Grid: one block per tile of voxels, capped at the number of blocks that
-// are resident at once (the kernel strides over the remaining tiles).
-gac_status plan_launch(const ModelConst &mc, int prec, bool trace, int C, int64_t n_vox, int moments_mode,
-                       LaunchCfg *cfg, int64_t *n_tiles, int *vb) {
-    const void *fn = mh_kernel_ptr(mc.kind, prec, trace);
-    if (!fn) return fail(GAC_ERR_INVALID_ARG, "no kernel for kind %d precision %d", mc.kind, prec);
-    const size_t smem = smem_bytes_for(mc.kind, prec, C, mc.n_meas, moments_mode);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
+// Resident blocks of `block` threads per SM of the one-launch kernel, with its
+// attributes set.
+static gac_status mh_resident(const ModelConst &mc, int prec, bool trace, int C, int moments_mode, int block,
+                              LaunchCfg *cfg, int *per_sm) {
+    cfg->fn = mh_kernel_ptr(mc.kind, prec, trace, block);
+    if (!cfg->fn) return fail(GAC_ERR_INVALID_ARG, "no kernel for kind %d precision %d", mc.kind, prec);
+    cfg->block = block;
+    cfg->smem = smem_bytes_for(mc.kind, prec, C, mc.n_meas, moments_mode, block);
+    cudaError_t e = cudaFuncSetAttribute(cfg->fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(cfg->smem));
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
     // prefer the largest shared-memory carveout: the tile and Welford
     // accumulators, not L1, decide how many blocks fit
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    e = cudaFuncSetAttribute(cfg->fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(carveout)");
-    int per_sm = 0;
-    const int block = mh_block_size(mc.kind, prec);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, cfg->fn, block, cfg->smem);
     if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
-    if (per_sm < 1) return fail(GAC_ERR_INVALID_ARG, "kernel does not fit on an SM (smem %zu)", smem);
-    // Voxels per tile: a full block's worth, unless the problem is too small
-    // to give every resident block a full tile; then tiles shrink (in whole
-    // warps of chains) so that the chains spread over all SMs instead of
-    // crowding a few -- a small problem is bound by the latency of one
-    // iteration, which a warp alone on its SM sub-partition runs fastest.
-    // The block's remaining threads stay idle; results do not depend on the
-    // tiling (random numbers are keyed by voxel, chain and iteration).
-    const int64_t resident = static_cast<int64_t>(per_sm) * sm_count();
+    if (*per_sm < 1) return fail(GAC_ERR_INVALID_ARG, "kernel does not fit on an SM (smem %zu)", cfg->smem);
+    return GAC_OK;
+}
+
+// Time of a launch of `tiles` full blocks in units of a full wave: whole waves,
+// and a last one in which the fullest SM holds r of its `per_sm` blocks.  An SM
+// with few warps waits out their latency, so the last wave costs 1/4 + 3/4 r /
+// per_sm of a full one (3-pool, blocks of 128: 0.42, 0.58, 0.80 and 1 measured
+// for r = 1..4).
+static double waves(int64_t tiles, int per_sm) {
+    const int64_t slots = static_cast<int64_t>(per_sm) * sm_count();
+    const int64_t rest = tiles % slots;
+    if (rest == 0) return static_cast<double>(tiles / slots);
+    const int64_t r = (rest + sm_count() - 1) / sm_count();
+    return static_cast<double>(tiles / slots) + 0.25 + 0.75 * static_cast<double>(r) / per_sm;
+}
+
+// Grid: one block per tile of voxels, capped at the number of blocks that
+// are resident at once (the kernel strides over the remaining tiles).  The
+// random numbers are keyed by voxel, chain and iteration, so results do not
+// depend on the tiling.
+static gac_status plan_launch(const ModelConst &mc, int prec, bool trace, int C, int64_t n_vox, int moments_mode,
+                              LaunchCfg *cfg, int64_t *n_tiles, int *vb) {
     const int64_t chains = n_vox * C;
-    int threads = block;
-    if (chains < resident * block) {
+    int per_sm = 0;
+    gac_status st = mh_resident(mc, prec, trace, C, moments_mode, kBlock, cfg, &per_sm);
+    if (st != GAC_OK) return st;
+    int threads = kBlock;
+    const int64_t resident = static_cast<int64_t>(per_sm) * sm_count();
+    if (!trace && prec != GAC_PREC_FP64) {
+        // Blocks of kHalfBlock where they spread the chains more evenly: a
+        // block's warps go to the SM's four schedulers in turn, so full blocks
+        // of four warps load them evenly, while two blocks of eight with
+        // some idle warps, or a last wave of few large blocks, leave
+        // schedulers with twice the warps of others.  Full waves of half
+        // blocks measured up to 3% slower (1.03).  3-pool, us per iteration,
+        // kBlock -> kHalfBlock: 14,400 chains 1.79 -> 1.31, 49,380 3.12 ->
+        // 2.51, 120,000 6.09 -> 5.24, 200,000 9.01 -> 8.05.  Below one block
+        // an SM, tiles shrink in whole warps of chains: each scheduler gets at
+        // most one warp.
+        LaunchCfg half;
+        int half_per_sm = 0;
+        if ((st = mh_resident(mc, prec, trace, C, moments_mode, kHalfBlock, &half, &half_per_sm)) != GAC_OK) return st;
+        half_per_sm = std::min(half_per_sm, 2 * per_sm);  // as many warps: 20 instead of 16 ran 2% slower (3-pool)
+        const int vb1 = std::max(1, kBlock / C), vb2 = std::max(1, kHalfBlock / C);
+        const double t1 = waves((n_vox + vb1 - 1) / vb1, per_sm);
+        const double t2 = 1.03 * waves((n_vox + vb2 - 1) / vb2, half_per_sm);
+        const int64_t want = (chains + sm_count() - 1) / sm_count();  // chains an SM
+        if (t2 < t1 || want <= kHalfBlock) {
+            *cfg = half;
+            per_sm = half_per_sm;
+            threads = static_cast<int>(std::min<int64_t>(kHalfBlock, (want + 31) / 32 * 32));
+        }
+    } else if (chains < resident * kBlock) {
+        // too few chains for a full tile per resident block: tiles shrink in
+        // whole warps of chains, so that the chains spread over all SMs
         const int64_t want = (chains + resident - 1) / resident;  // chains per block
-        threads = static_cast<int>(std::min<int64_t>(block, std::max<int64_t>(32, (want + 31) / 32 * 32)));
+        threads = static_cast<int>(std::min<int64_t>(kBlock, std::max<int64_t>(32, (want + 31) / 32 * 32)));
     }
     *vb = std::max(1, threads / C);
     *n_tiles = (n_vox + *vb - 1) / *vb;
-    cfg->grid = static_cast<int>(std::min<int64_t>(*n_tiles, resident));
-    cfg->smem = smem;
+    cfg->grid = static_cast<int>(std::min<int64_t>(*n_tiles, static_cast<int64_t>(per_sm) * sm_count()));
     return GAC_OK;
 }
 
@@ -525,10 +534,12 @@ gac_status validate_opts(const gac_mcmc_opts *o, int64_t n_vox) {
 
 // Lanes per chain of a gac_mcmc_run (1: the one-thread kernel).  The
 // lane-split kernel handles MIXED runs without trace of the mono-exponential
-// and 3-pool models with evenly spaced echoes in 2..4 blocks of kAnchor; the
-// library uses it when the chains would give fewer than one warp per SM
-// sub-partition (there it shortens the latency of an iteration; on larger
-// problems one thread per chain keeps more chains in flight).
+// and 3-pool models with evenly spaced echoes in 2..4 blocks of kAnchor.  The
+// library uses it for the mono-exponential model when the chains would give
+// fewer than one warp per SM sub-partition (there it shortens the latency of an
+// iteration; on larger problems one thread per chain keeps more chains in
+// flight); the 3-pool model runs faster on the speculative kernel or, from
+// about 12,000 chains, one thread per chain (1.30 against 2.35 us an iteration).
 static gac_status choose_lanes(const ModelConst &mc, const gac_mcmc_opts *o, int64_t n_vox, int *lanes) {
     const int nb = (mc.n_acq + kAnchor - 1) / kAnchor;
     const bool eligible = o->precision == GAC_PREC_MIXED && o->trace_n_vox == 0 && mc.even &&
@@ -545,7 +556,7 @@ static gac_status choose_lanes(const ModelConst &mc, const gac_mcmc_opts *o, int
         return GAC_OK;
     }
     const int64_t one_warp_each = static_cast<int64_t>(sm_count()) * 4 * 32;
-    if (eligible && n_vox * o->n_chains < one_warp_each) *lanes = nb <= 2 ? 2 : 4;
+    if (eligible && mc.kind == GAC_MODEL_MONOEXP && n_vox * o->n_chains < one_warp_each) *lanes = nb <= 2 ? 2 : 4;
     return GAC_OK;
 }
 
@@ -570,6 +581,7 @@ static gac_status plan_split(const ModelConst &mc, int G, int C, int64_t n_vox, 
     if (per_sm < 1) return fail(GAC_ERR_INVALID_ARG, "lane-split kernel does not fit on an SM (smem %zu)", smem);
     *n_tiles = (n_vox + *vb - 1) / *vb;
     cfg->grid = static_cast<int>(std::min<int64_t>(*n_tiles, static_cast<int64_t>(per_sm) * sms));
+    cfg->fn = fn;
     cfg->smem = smem;
     cfg->block = threads;
     return GAC_OK;
@@ -608,13 +620,13 @@ static SpecShape spec_shape(int depth, int C, int64_t n_vox) {
 // the deepest tree whose warps find idle schedulers.  Measured on GB300 (ms
 // per 1,000 iterations, 1 chain a voxel):
 //   chains           200    1,200  2,400  4,800  9,600  14,400  19,200
-//   3-pool    one    1.14   1.21   1.21   1.22   1.22   1.71    1.72
+//   3-pool    one    1.14   1.21   1.21   1.22   1.22   1.30    1.30
 //             spec   0.31   0.37   0.47   0.67   0.96   1.31    1.61
-//             depth  5      4      3      2      2      2       2
+//             depth  5      4      3      2      2      -       -
 //   SMT       one    0.58   0.59   0.59   0.60   0.60   0.60    0.61
 //             spec   0.15   0.18   0.22   0.28   0.41   0.52    0.63
 //             depth  5      4      3      3      2      2       -
-//   AxCaliber one    1.58   1.60   1.60   1.61   1.61   2.00    1.99
+//   AxCaliber one    1.58   1.60   1.60   1.61   1.61   1.72    1.77
 //             spec   0.40   0.49   0.62   0.77   1.10   1.41    1.68
 //             depth  5      4      3      3      2      2       2
 //   mono-exp  split  0.19   0.20   0.20   0.20   0.19   0.26    0.26
@@ -623,8 +635,8 @@ static SpecShape spec_shape(int depth, int C, int64_t n_vox) {
 // its scheduler only where it waits on table lookups (SMT, AxCaliberSMT); the
 // 3-pool round issues paired multiply-adds for most of its cycles.  Depth 2
 // doubles the work per iteration and halves the serial path: it pays up to
-// four warps a scheduler, for SMT (whose one-thread kernel keeps 32 warps an SM)
-// up to three.  The mono-exponential round is short enough that the lane-split
+// four warps a scheduler for AxCaliberSMT, three for SMT and two for the 3-pool
+// model, the least latency-bound of the three.  The mono-exponential round is short enough that the lane-split
 // kernel's shorter path wins where it applies (`split`) once two warps share
 // a scheduler.
 static int choose_depth(const ModelConst &mc, const gac_mcmc_opts *o, int64_t n_vox, bool split) {
@@ -636,7 +648,7 @@ static int choose_depth(const ModelConst &mc, const gac_mcmc_opts *o, int64_t n_
     const bool mwi3 = mc.kind == GAC_MODEL_MWI3, mono = mc.kind == GAC_MODEL_MONOEXP;
     for (int depth = 5; depth >= 2; --depth) {
         if (C << depth > kSpecBlock || n_vox * C > (schedulers * 32 * 4 >> depth)) continue;
-        const int per = depth >= 4 ? 1 : depth == 3 ? (mwi3 || mono ? 1 : 2) : mc.kind == GAC_MODEL_SMT ? 3 : 4;
+        const int per = depth >= 4 ? 1 : depth == 3 ? (mwi3 || mono ? 1 : 2) : mwi3 ? 2 : mc.kind == GAC_MODEL_SMT ? 3 : 4;
         if (depth < 4 && mono && split) return 0;
         if (spec_shape(depth, C, n_vox).warps() <= per * schedulers) return depth;
     }
@@ -659,6 +671,7 @@ static gac_status plan_spec(const ModelConst &mc, int depth, int C, int64_t n_vo
     *vb = sh.vb;
     *n_tiles = sh.n_tiles;
     cfg->grid = static_cast<int>(std::min<int64_t>(sh.n_tiles, static_cast<int64_t>(per_sm) * sm_count()));
+    cfg->fn = fn;
     cfg->smem = smem;
     cfg->block = sh.threads;
     return GAC_OK;
@@ -894,12 +907,10 @@ gac_status gac_mcmc_run(int model_id, const void *data, int64_t n_vox, const flo
     int64_t n_tiles = 0;
     int vb = 0;
     const int depth = choose_depth(mc, o, n_vox, lanes > 1);
-    const bool all = o->moments_mode == GAC_MOMENTS_ALL_POSTBURNIN;
     st = depth > 0 ? plan_spec(mc, depth, C, n_vox, o->moments_mode, &cfg, &n_tiles, &vb)
        : lanes > 1 ? plan_split(mc, lanes, C, n_vox, o->moments_mode, &cfg, &n_tiles, &vb)
                    : plan_launch(mc, o->precision, trace, C, n_vox, o->moments_mode, &cfg, &n_tiles, &vb);
     if (st != GAC_OK) return st;
-    cfg.stream = s;
 
     RunArgs ra;
     std::memset(&ra, 0, sizeof ra);
@@ -933,11 +944,7 @@ gac_status gac_mcmc_run(int model_id, const void *data, int64_t n_vox, const flo
     ra.step_scale = static_cast<float *>(d_scale.ptr);
 
     void *args[] = {&mc, &ra};
-    cudaError_t e = depth > 0 ? cudaLaunchKernel(mh_spec_ptr(mc.kind, depth, all), dim3(cfg.grid), dim3(cfg.block), args, cfg.smem, s)
-                    : lanes == 1 ? launch_mh(mc.kind, o->precision, trace, mc, ra, cfg)
-                    : mc.kind == GAC_MODEL_MONOEXP
-                        ? launch_mh_split_monoexp(lanes, all, mc, ra, cfg)
-                        : launch_mh_split_mwi3(lanes, all, mc, ra, cfg);
+    cudaError_t e = cudaLaunchKernel(cfg.fn, dim3(cfg.grid), dim3(cfg.block), args, cfg.smem, s);
     if (e != cudaSuccess) return cuda_fail(e, "MH kernel launch");
     for (DevBuf *b : {&d_mean, &d_std, &d_samples, &d_acc, &d_bad, &d_trace, &d_rhat, &d_scale})
         if ((st = b->copy_out()) != GAC_OK) return st;

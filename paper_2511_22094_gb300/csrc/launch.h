@@ -1,5 +1,7 @@
 // Host-side launch interface between the C ABI (gac.cu) and the kernel
-// translation units (one per model kind, compiled in parallel).
+// translation units (one per model kind, compiled in parallel).  Every kernel
+// takes (const ModelConst, const RunArgs) and is launched with
+// cudaLaunchKernel(ptr, ..., {&mc, &ra}, ...).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -8,39 +10,26 @@
 namespace gac {
 
 struct LaunchCfg {
+    const void *fn;
     int grid;
+    int block;  // threads per block
     size_t smem;
-    cudaStream_t stream;
-    int block = kBlock;  // threads per block (the lane-split kernel sizes its blocks)
 };
 
-// Returns the kernel for (kind, precision, trace) or nullptr.
-const void *mh_kernel_ptr(int kind, int prec, bool trace);
-cudaError_t launch_mh(int kind, int prec, bool trace, const ModelConst &mc, const RunArgs &ra,
-                      const LaunchCfg &cfg);
-
-// Per-kind entry points defined in mh_<kind>.cu
-const void *mh_ptr_monoexp(int prec, bool trace);
-const void *mh_ptr_mwi3(int prec, bool trace);
-const void *mh_ptr_smt(int prec, bool trace);
-const void *mh_ptr_axcal(int prec, bool trace);
-const void *mh_ptr_linear(int prec, bool trace);
+// Per-kind kernels defined in mh_<kind>.cu: (precision, trace, kBlock or kHalfBlock)
+const void *mh_ptr_monoexp(int prec, bool trace, int block);
+const void *mh_ptr_mwi3(int prec, bool trace, int block);
+const void *mh_ptr_smt(int prec, bool trace, int block);
+const void *mh_ptr_axcal(int prec, bool trace, int block);
+const void *mh_ptr_linear(int prec, bool trace, int block);
 // Lane-split kernels (mh_split.cuh): G = 2 or 4 lanes per chain, MIXED; all:
 // moments over every post-burn-in state.
 const void *mh_split_ptr_monoexp(int G, bool all);
 const void *mh_split_ptr_mwi3(int G, bool all);
-cudaError_t launch_mh_split_monoexp(int G, bool all, const ModelConst &mc, const RunArgs &ra, const LaunchCfg &cfg);
-cudaError_t launch_mh_split_mwi3(int G, bool all, const ModelConst &mc, const RunArgs &ra, const LaunchCfg &cfg);
-// Speculative kernels (mh_spec.cuh): trees of depth 2..5, MIXED; launched with
-// cudaLaunchKernel(ptr, ..., {&mc, &ra}).
+// Speculative kernels (mh_spec.cuh): trees of depth 2..5, MIXED.
 const void *mh_spec_ptr_monoexp(int depth, bool all);
 const void *mh_spec_ptr_mwi3(int depth, bool all);
 const void *mh_spec_ptr_smt(int depth, bool all);
 const void *mh_spec_ptr_axcal(int depth, bool all);
-cudaError_t launch_mh_monoexp(int prec, bool trace, const ModelConst &mc, const RunArgs &ra, const LaunchCfg &cfg);
-cudaError_t launch_mh_mwi3(int prec, bool trace, const ModelConst &mc, const RunArgs &ra, const LaunchCfg &cfg);
-cudaError_t launch_mh_smt(int prec, bool trace, const ModelConst &mc, const RunArgs &ra, const LaunchCfg &cfg);
-cudaError_t launch_mh_axcal(int prec, bool trace, const ModelConst &mc, const RunArgs &ra, const LaunchCfg &cfg);
-cudaError_t launch_mh_linear(int prec, bool trace, const ModelConst &mc, const RunArgs &ra, const LaunchCfg &cfg);
 
 }  // namespace gac

@@ -60,18 +60,11 @@ constexpr int mh_min_blocks() {
     return PREC == GAC_PREC_FP64 ? 1 : ((KIND == GAC_MODEL_MWI3 || KIND == GAC_MODEL_AXCAL_SMT) ? 2 : (KIND == GAC_MODEL_SMT ? 4 : 3));
 }
 
-// The one-launch kernel's own block size and blocks per SM (the serving and
-// allocation-free kernels always run blocks of kBlock).  Measured on the
-// 3-pool MIXED kernel: blocks of 128 threads, 5 or 6 per SM (20 or 24 warps),
-// ran 3% slower than 2 blocks of 256, so every kind keeps kBlock.
-template <int KIND, int PREC>
-__host__ __device__ constexpr int mh_block() {
-    return kBlock;
-}
-template <int KIND, int PREC>
-constexpr int mh_launch_min_blocks() {
-    return mh_block<KIND, PREC>() == kBlock ? mh_min_blocks<KIND, PREC>() : 5;
-}
+// The one-launch kernel comes in blocks of kBlock and, for MIXED and FP32
+// without a trace, of kHalfBlock threads (twice as many an SM): plan_launch
+// takes the one that leaves the SMs less idle.  The serving and allocation-free
+// kernels always run blocks of kBlock.
+constexpr int kHalfBlock = kBlock / 2;
 
 struct RunArgs {
     const float *data;   // [N][M]
@@ -596,13 +589,34 @@ __device__ __forceinline__ void run_tile(const ModelConst &mc, const RunArgs &ra
 }
 
 // One job, one launch: every tile runs all I iterations.
-template <int KIND, int PREC, bool TRACE>
-__global__ void __launch_bounds__(mh_block<KIND, PREC>(), mh_launch_min_blocks<KIND, PREC>())
+template <int KIND, int PREC, bool TRACE, int BLK = kBlock>
+__global__ void __launch_bounds__(BLK, mh_min_blocks<KIND, PREC>() * (kBlock / BLK))
     mh_kernel(const ModelConst mc, const RunArgs ra) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SliceState none{};
     for (int64_t tile = blockIdx.x; tile < ra.n_tiles; tile += gridDim.x)
-        run_tile<KIND, PREC, TRACE, false, mh_block<KIND, PREC>()>(mc, ra, none, tile, 0, ra.I, smem_raw);
+        run_tile<KIND, PREC, TRACE, false, BLK>(mc, ra, none, tile, 0, ra.I, smem_raw);
+}
+
+// The kernel of a kind for (precision, trace, threads per block), or nullptr.
+template <int KIND>
+const void *mh_kernel_ptr_of(int prec, bool trace, int block) {
+    const bool half = block == kHalfBlock;
+    if (half && (trace || prec == GAC_PREC_FP64)) return nullptr;
+    switch (prec) {
+    case GAC_PREC_MIXED:
+        return trace  ? reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_MIXED, true>)
+               : half ? reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_MIXED, false, kHalfBlock>)
+                      : reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_MIXED, false>);
+    case GAC_PREC_FP32:
+        return trace  ? reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_FP32, true>)
+               : half ? reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_FP32, false, kHalfBlock>)
+                      : reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_FP32, false>);
+    case GAC_PREC_FP64:
+        return trace ? reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_FP64, true>)
+                     : reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_FP64, false>);
+    default: return nullptr;
+    }
 }
 
 }  // namespace gac

@@ -543,4 +543,12 @@ __global__ void __launch_bounds__(kBlock, 1)
         run_tile_split<KIND, G, ALL>(mc, ra, tile, smem_raw);
 }
 
+// The kernel for 2 or 4 lanes a chain (nullptr otherwise).
+template <int KIND>
+const void *mh_split_kernel_ptr(int G, bool all) {
+    if (G == 2) return all ? reinterpret_cast<const void *>(&mh_split_kernel<KIND, 2, true>) : reinterpret_cast<const void *>(&mh_split_kernel<KIND, 2, false>);
+    if (G == 4) return all ? reinterpret_cast<const void *>(&mh_split_kernel<KIND, 4, true>) : reinterpret_cast<const void *>(&mh_split_kernel<KIND, 4, false>);
+    return nullptr;
+}
+
 }  // namespace gac
