@@ -1,6 +1,8 @@
 // Whole-volume gradient fit (askadam.m, Sec. 2.2.1; Eq. 2, 4, 5): Adam on
 // the L1 or L2 data loss over a masked voxel grid, with an optional total-
-// variation penalty on chosen parameter maps.  One launch per iteration:
+// variation penalty on chosen parameter maps.  Without the penalty no voxel
+// depends on another, and fit_many_kernel takes up to 128 updates a launch (its
+// comment below).  With it, one launch per iteration:
 //   fit_step_kernel   every voxel (one thread each): forward model and its
 //                     analytic Jacobian, the data loss and its gradient, the
 //                     total-variation subgradient from the six (or four)
@@ -261,6 +263,63 @@ __device__ __forceinline__ float mwi3_rec_loss_grad_f(const float *th, const Mod
     return L1 ? aw * loss : wgt * wgt * loss;
 }
 
+// The data loss of one voxel and its gradient (with respect to theta) at the
+// normalised parameters u, against its staged data row y.
+template <int KIND, int PREC, bool L1>
+__device__ __forceinline__ void fit_loss_grad(const ModelConst &mc, const float *y,
+                                              const typename PrecTraits<PREC>::R (&u)[model_n_par(KIND)],
+                                              typename PrecTraits<PREC>::R w, typename PrecTraits<PREC>::R &loss,
+                                              typename PrecTraits<PREC>::R (&g)[model_n_par(KIND)]) {
+    using R = typename PrecTraits<PREC>::R;
+    constexpr int P = model_n_par(KIND);
+    R th[P];
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        const R lo = sizeof(R) == 8 ? R(mc.lb_d[p]) : R(mc.lb_f[p]);
+        const R hi = sizeof(R) == 8 ? R(mc.ub_d[p]) : R(mc.ub_f[p]);
+        th[p] = lo + u[p] * (hi - lo);
+    }
+    // data term: rho(w (y - s)), drho/ds = -w sign(r) (L1) or -2 w r (L2)
+    auto visit = [&](int k, R s, const R *J) {
+        const R r = w * (R(y[k]) - s);
+        R d;
+        if constexpr (L1) {
+            d = -w * sgn(r);
+            loss += fabs(r);
+        } else {
+            d = R(-2) * w * r;
+            loss += r * r;
+        }
+#pragma unroll
+        for (int p = 0; p < P; ++p) g[p] = fma(d, J[p], g[p]);
+    };
+    if constexpr (KIND == GAC_MODEL_MWI3 && PREC == GAC_PREC_FP32) {
+        if (mc.even) loss = mwi3_rec_loss_grad_f<L1>(th, mc, y, w, g);  // same branch for every thread
+        else jacobian<KIND, R>(th, mc, visit);
+    } else {
+        jacobian<KIND, R>(th, mc, visit);
+    }
+}
+
+// One parameter's Adam step: bias-corrected moments a, b (updated), then the
+// box.  FP32: the corrections as the reciprocals c1, c2 carry (1 / (1 -
+// beta^t)), the step's square root and quotient on the special-function unit (a
+// few ulp); FP64: divided, as the oracle does.
+template <class R>
+__device__ __forceinline__ R fit_adam(const FitArgs<R> &fa, R u, R g, R &a, R &b, R c1, R c2) {
+    a = fa.beta1 * a + (R(1) - fa.beta1) * g;
+    b = fa.beta2 * b + (R(1) - fa.beta2) * g * g;
+    R stepu;
+    if constexpr (sizeof(R) == 8) {
+        stepu = fa.lr * (a / c1) / (sqrt(b / c2) + fa.eps);
+    } else {
+        float sq;
+        asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(sq) : "f"(b * c2));
+        stepu = __fdividef(fa.lr * (a * c1), sq + fa.eps);
+    }
+    return fmin(fmax(u - stepu, R(0)), R(1));
+}
+
 // One voxel's update: forward model and Jacobian against its staged data row
 // y, the loss gradient, the total-variation subgradient, Adam and the box.
 // Returns the voxel's share of the loss (0 outside the mask).
@@ -329,34 +388,7 @@ __device__ __forceinline__ void fit_phase_a(const ModelConst &mc, const FitArgs<
     loss = R(0);
 #pragma unroll
     for (int p = 0; p < P; ++p) g[p] = R(0);
-    if (!inside) return;
-    R th[P];
-#pragma unroll
-    for (int p = 0; p < P; ++p) {
-        const R lo = sizeof(R) == 8 ? R(mc.lb_d[p]) : R(mc.lb_f[p]);
-        const R hi = sizeof(R) == 8 ? R(mc.ub_d[p]) : R(mc.ub_f[p]);
-        th[p] = lo + u[p] * (hi - lo);
-    }
-    // data term: rho(w (y - s)), drho/ds = -w sign(r) (L1) or -2 w r (L2)
-    auto visit = [&](int k, R s, const R *J) {
-        const R r = w * (R(y[k]) - s);
-        R d;
-        if constexpr (L1) {
-            d = -w * sgn(r);
-            loss += fabs(r);
-        } else {
-            d = R(-2) * w * r;
-            loss += r * r;
-        }
-#pragma unroll
-        for (int p = 0; p < P; ++p) g[p] = fma(d, J[p], g[p]);
-    };
-    if constexpr (KIND == GAC_MODEL_MWI3 && PREC == GAC_PREC_FP32) {
-        if (mc.even) loss = mwi3_rec_loss_grad_f<L1>(th, mc, y, w, g);  // same branch for every thread
-        else jacobian<KIND, R>(th, mc, visit);
-    } else {
-        jacobian<KIND, R>(th, mc, visit);
-    }
+    if (inside) fit_loss_grad<KIND, PREC, L1>(mc, y, u, w, loss, g);
 }
 
 // Phase B; returns the voxel's share of the loss (0 outside the mask).
@@ -410,25 +442,12 @@ __device__ __forceinline__ typename PrecTraits<PREC>::R fit_phase_b(
             vl += fa.lambda_n * tv_loss;
         }
     }
-    // Adam (bias-corrected moments), then the box.  FP32: the corrections as
-    // the reciprocals c1, c2 carry (1 / (1 - beta^t)), the step's square root
-    // and quotient on the special-function unit (a few ulp); FP64: divided,
-    // as the oracle does
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        const R a = fa.beta1 * mo[p * 32] + (R(1) - fa.beta1) * g[p];
-        const R b = fa.beta2 * mo[(P + p) * 32] + (R(1) - fa.beta2) * g[p] * g[p];
+        R a = mo[p * 32], b = mo[(P + p) * 32];
+        u_out[p * n + v] = fit_adam(fa, u[p], g[p], a, b, c1, c2);
         m1[p * n + v] = a;
         m2[p * n + v] = b;
-        R stepu;
-        if constexpr (sizeof(R) == 8) {
-            stepu = fa.lr * (a / c1) / (sqrt(b / c2) + fa.eps);
-        } else {
-            float sq;
-            asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(sq) : "f"(b * c2));
-            stepu = __fdividef(fa.lr * (a * c1), sq + fa.eps);
-        }
-        u_out[p * n + v] = fmin(fmax(u[p] - stepu, R(0)), R(1));
     }
     return vl;
 }
@@ -452,6 +471,31 @@ __device__ __forceinline__ void cp_async16(float *dst, const float *src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+
+// Copies the measurement rows of `rows` voxels (lane r's voxel v is row r) into
+// the warp's shared memory, 16 bytes a copy where rows are whole float4s.
+template <class FA>
+__device__ __forceinline__ void fit_stage_rows(const FA &fa, int M, int v, int rows, int lane, float *rows_s) {
+    if (fa.vec4) {  // row = floor((e + 1/2) / (M/4)) by one float multiply
+        const int M4 = M >> 2, S4 = fa.row_stride >> 2, total4 = rows * M4;
+#pragma unroll 4
+        for (int e0 = 0; e0 < total4; e0 += 32) {
+            const int e = e0 + lane;
+            const int row = static_cast<int>((static_cast<float>(e) + 0.5f) * fa.inv_m4);
+            const int vr = __shfl_sync(0xffffffffu, v, min(row, rows - 1));
+            if (e < total4)
+                cp_async16(rows_s + 4 * (row * S4 + (e - row * M4)), fa.data + static_cast<int64_t>(vr) * M + 4 * (e - row * M4));
+        }
+    } else {
+        const int total = rows * M;
+        for (int e0 = 0; e0 < total; e0 += 32) {
+            const int e = e0 + lane;
+            const int row = e / M;
+            const int vr = __shfl_sync(0xffffffffu, v, min(row, rows - 1));
+            if (e < total) cp_async4(rows_s + row * fa.row_stride + (e - row * M), fa.data + static_cast<int64_t>(vr) * M + (e - row * M));
+        }
+    }
+}
 
 // Persistent warps over tiles of 32 voxels (warp tile w, w + all warps, ...).
 // Each warp stages its own tile's measurement rows and Adam moments in its
@@ -598,10 +642,31 @@ __global__ void __launch_bounds__(kFitBlock, fit_min_blocks(PREC)) fit_step_kern
     }
 }
 
+// The stopping rules after iteration t, whose loss is hist[t - 1]: loss < tol, or
+// |least-squares slope of the last `window` losses| < conv_value.
+template <class FA>
+__device__ bool fit_halts(const FA &fa, int t) {
+    const double loss = fa.hist[t - 1];
+    if (fa.tol > 0.0 && loss < fa.tol) return true;
+    const int window = fa.window;
+    if (fa.conv_value > 0.0 && window > 1 && t >= window) {
+        const double *yv = fa.hist + t - window;
+        const double xm = 0.5 * (window - 1);
+        double ym = 0.0, sxy = 0.0, sxx = 0.0;
+        for (int i = 0; i < window; ++i) ym += yv[i];
+        ym /= window;
+        for (int i = 0; i < window; ++i) {
+            sxy += (i - xm) * (yv[i] - ym);
+            sxx += (i - xm) * (i - xm);
+        }
+        return fabs(sxy / sxx) < fa.conv_value;
+    }
+    return false;
+}
+
 // Run by the last block of iteration t: sums the block shares (fixed order:
 // thread i the shares i, i + 256, ..., then a tree), records loss t and
-// applies the stopping rules: loss < tol, or |least-squares slope of the
-// last `window` losses| < conv_value.
+// applies the stopping rules.
 template <class FA>
 __device__ void fit_check(const FA &fa, int n_blocks, int t, double *red) {
     double s = 0.0;
@@ -613,24 +678,224 @@ __device__ void fit_check(const FA &fa, int n_blocks, int t, double *red) {
         __syncthreads();
     }
     if (threadIdx.x != 0) return;
-    const double loss = red[0];
-    fa.hist[t - 1] = loss;
+    fa.hist[t - 1] = red[0];
     *fa.done = t;
-    bool halt = fa.tol > 0.0 && loss < fa.tol;
-    const int window = fa.window;
-    if (!halt && fa.conv_value > 0.0 && window > 1 && t >= window) {
-        const double *yv = fa.hist + t - window;
-        const double xm = 0.5 * (window - 1);
-        double ym = 0.0, sxy = 0.0, sxx = 0.0;
-        for (int i = 0; i < window; ++i) ym += yv[i];
-        ym /= window;
-        for (int i = 0; i < window; ++i) {
-            sxy += (i - xm) * (yv[i] - ym);
-            sxx += (i - xm) * (i - xm);
+    if (fit_halts(fa, t)) *fa.stop = 1;
+}
+
+// ------------------------------------------------ fits without coupling ----
+// Without a total-variation term a voxel's updates depend on no other voxel, so
+// one launch takes up to kFitChunk of them: a block of one warp stages the rows
+// of 32 fitted voxels once, keeps their parameters in registers and their Adam
+// moments in registers or shared memory, and iterates.  Bound by issue (and, for
+// a few hundred tiles, by the latency of one update) instead of by the 413 bytes
+// a voxel-update moves when every update is a launch.  Measured, whole calls on
+// a GB300, a launch per update -> this: mono-exponential, 37 x 41 x 9 voxels, 300
+// updates 1.70 -> 0.22 ms; 3-pool, 96 x 96 x 60, 100 updates 5.6 -> 3.3 ms, with
+// a mask of 68% of it 5.7 -> 2.4 ms.  The losses
+// of kFitFlush updates cross the warp through shared memory: two lanes add the 32
+// voxels' shares of one update, in FP32 with the rounding errors carried along
+// (TwoSum; FP64 adds hold the FP64 pipe for 76 cycles each).
+constexpr int kFitChunk = 128, kFitFlush = 16;
+constexpr int kFitLossBlocks = 128;  // blocks of fit_losses_kernel
+
+template <class R>
+struct FitSteps {
+    R c1[kFitChunk], c2[kFitChunk];  // Adam's bias corrections of the launch's updates
+};
+
+template <int KIND>
+__host__ __device__ constexpr bool fit_reg_moments() { return model_n_par(KIND) <= 4; }
+
+template <int KIND, class R>
+__host__ __device__ constexpr size_t fit_many_smem(int row_stride) {
+    return 32 * static_cast<size_t>(row_stride) * sizeof(float) + kFitFlush * 33 * sizeof(R) +
+           (fit_reg_moments<KIND>() ? 0 : 2 * static_cast<size_t>(model_n_par(KIND)) * 32 * sizeof(R));
+}
+
+// Updates t0 .. t0 + count - 1 (t0 = 1: from zero moments) of the voxels
+// list[0 .. n_list) (list = nullptr: voxels 0 .. n_list - 1), u and the moments in
+// place; part[tile][count]: the tile's share of each update's loss.
+template <int KIND, int PREC, bool L1>
+__global__ void __launch_bounds__(32, PREC == GAC_PREC_FP32 ? 20 : 8)
+    fit_many_kernel(const ModelConst mc, const FitArgs<typename PrecTraits<PREC>::R> fa, const int *list, int n_list,
+                    typename PrecTraits<PREC>::R *u_io, typename PrecTraits<PREC>::R *m1, typename PrecTraits<PREC>::R *m2,
+                    const __grid_constant__ FitSteps<typename PrecTraits<PREC>::R> steps, int t0, int count, double *part) {
+    using R = typename PrecTraits<PREC>::R;
+    constexpr int P = model_n_par(KIND);
+    constexpr bool kReg = fit_reg_moments<KIND>();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float *rows_s = reinterpret_cast<float *>(smem_raw);
+    R *loss_s = reinterpret_cast<R *>(smem_raw + 32 * static_cast<size_t>(fa.row_stride) * sizeof(float));
+    R *mo = loss_s + kFitFlush * 33 + threadIdx.x;
+    const int lane = threadIdx.x;
+    const int M = mc.n_meas;
+    const int n = static_cast<int>(fa.n);
+    const int i0 = blockIdx.x * 32;
+    const int rows = min(32, n_list - i0);
+    const bool active = lane < rows;
+    const int e = i0 + (active ? lane : rows - 1);
+    const int v = list ? list[e] : e;
+    model_smem_load<KIND, 1>(mc);
+    fit_stage_rows(fa, M, v, rows, lane, rows_s);
+    cp_async_commit();
+    R u[P], ma[P], mb[P];
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        u[p] = u_io[p * n + v];
+        const R a = t0 > 1 ? m1[p * n + v] : R(0), b = t0 > 1 ? m2[p * n + v] : R(0);
+        if constexpr (kReg) {
+            ma[p] = a;
+            mb[p] = b;
+        } else {
+            mo[p * 32] = a;
+            mo[(P + p) * 32] = b;
         }
-        halt = fabs(sxy / sxx) < fa.conv_value;
     }
-    if (halt) *fa.stop = 1;
+    const R w = fa.weight ? R(fa.weight[v]) : R(1);
+    const float *y = rows_s + lane * fa.row_stride;
+    cp_async_wait<0>();
+    __syncwarp();
+    for (int k = 0; k < count; ++k) {
+        R share = R(0);
+        if (active) {
+            R loss = R(0), g[P];
+#pragma unroll
+            for (int p = 0; p < P; ++p) g[p] = R(0);
+            fit_loss_grad<KIND, PREC, L1>(mc, y, u, w, loss, g);
+            share = loss * fa.scale;
+            const R c1 = steps.c1[k], c2 = steps.c2[k];
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                const R range = sizeof(R) == 8 ? R(mc.ub_d[p] - mc.lb_d[p]) : R(mc.ub_f[p] - mc.lb_f[p]);
+                g[p] *= fa.scale * range;
+                if constexpr (kReg) {
+                    u[p] = fit_adam(fa, u[p], g[p], ma[p], mb[p], c1, c2);
+                } else {
+                    R a = mo[p * 32], b = mo[(P + p) * 32];
+                    u[p] = fit_adam(fa, u[p], g[p], a, b, c1, c2);
+                    mo[p * 32] = a;
+                    mo[(P + p) * 32] = b;
+                }
+            }
+        }
+        loss_s[(k & (kFitFlush - 1)) * 33 + lane] = share;
+        if ((k & (kFitFlush - 1)) == kFitFlush - 1 || k == count - 1) {
+            __syncwarp();
+            const int j = lane & (kFitFlush - 1), kk = (k & ~(kFitFlush - 1)) + j;
+            const R *q = loss_s + j * 33 + (lane & ~(kFitFlush - 1));
+            R hi = R(0), lo = R(0);
+#pragma unroll
+            for (int i = 0; i < kFitFlush; ++i) {
+                const R x = q[i], t = hi + x, bb = t - hi;
+                lo += (hi - (t - bb)) + (x - bb);
+                hi = t;
+            }
+            double sum = static_cast<double>(hi);
+            if (isfinite(hi)) sum += static_cast<double>(lo);
+            sum += __shfl_xor_sync(0xffffffffu, sum, kFitFlush);
+            if (lane < kFitFlush && kk <= k) part[static_cast<int64_t>(blockIdx.x) * count + kk] = sum;
+            __syncwarp();
+        }
+    }
+    if (active) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            u_io[p * n + v] = u[p];
+            m1[p * n + v] = kReg ? ma[p] : mo[p * 32];
+            m2[p * n + v] = kReg ? mb[p] : mo[(P + p) * 32];
+        }
+    }
+}
+
+// Sums the tiles' shares of `count` losses (thread k takes update k of its
+// block's range of tiles; the last block to finish adds the ranges in order),
+// records them and applies the stopping rules to each update in turn.
+template <class FA>
+__global__ void __launch_bounds__(kFitChunk) fit_losses_kernel(const FA fa, const double *part, int tiles, int t0, int count) {
+    __shared__ bool last;
+    const int k = threadIdx.x, nb = gridDim.x, b = blockIdx.x;
+    if (k < count) {
+        const int from = static_cast<int>(static_cast<int64_t>(tiles) * b / nb), to = static_cast<int>(static_cast<int64_t>(tiles) * (b + 1) / nb);
+        double s = 0.0;
+        for (int i = from; i < to; ++i) s += part[static_cast<int64_t>(i) * count + k];
+        fa.block_loss[b * kFitChunk + k] = s;
+        __threadfence();
+    }
+    __syncthreads();
+    if (k == 0) last = atomicAdd(fa.arrive, 1u) == static_cast<unsigned>(nb - 1);
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (k < count) {
+        double s = 0.0;
+        for (int i = 0; i < nb; ++i) s += __ldcg(fa.block_loss + i * kFitChunk + k);
+        fa.hist[t0 - 1 + k] = s;
+    }
+    __syncthreads();
+    if (k == 0) {
+        *fa.arrive = 0u;
+        int t = t0;
+        bool halt = fit_halts(fa, t);
+        while (!halt && t < t0 + count - 1) halt = fit_halts(fa, ++t);
+        *fa.done = t;
+        if (halt) *fa.stop = 1;
+    }
+}
+
+// ------------------------------------------------------- the fitted voxels --
+// The indices of the non-zero mask bytes, in order: counts per kMaskChunk bytes,
+// their exclusive sums (one block), then every chunk writes its own.
+constexpr int kMaskBlock = 256, kMaskPer = 8, kMaskChunk = kMaskBlock * kMaskPer;
+
+__device__ __forceinline__ int mask_scan_block(int c, int *warp_sums) {  // exclusive sum over the block
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_sums[warp] = x;
+    __syncthreads();
+    int before = 0;
+    for (int i = 0; i < warp; ++i) before += warp_sums[i];
+    return before + x - c;
+}
+
+__global__ void __launch_bounds__(kMaskBlock) mask_list_kernel(const uint8_t *mask, int n, int *chunk_count, const int *chunk_first, int *list) {
+    __shared__ int warp_sums[kMaskBlock / 32];
+    const int first = blockIdx.x * kMaskChunk + threadIdx.x * kMaskPer;
+    unsigned bits = 0;
+#pragma unroll
+    for (int i = 0; i < kMaskPer; ++i)
+        if (first + i < n && mask[first + i]) bits |= 1u << i;
+    const int c = __popc(bits);
+    int at = mask_scan_block(c, warp_sums);
+    if (!list) {  // first pass: counts only
+        if (threadIdx.x == kMaskBlock - 1) chunk_count[blockIdx.x] = at + c;
+        return;
+    }
+    at += chunk_first[blockIdx.x];
+#pragma unroll
+    for (int i = 0; i < kMaskPer; ++i)
+        if ((bits >> i) & 1u) list[at++] = first + i;
+}
+
+__global__ void __launch_bounds__(kMaskBlock) mask_first_kernel(const int *chunk_count, int chunks, int *chunk_first) {
+    __shared__ int warp_sums[kMaskBlock / 32];
+    __shared__ int carry_s;
+    int carry = 0;
+    for (int base = 0; base < chunks; base += kMaskBlock) {
+        const int i = base + threadIdx.x;
+        const int c = i < chunks ? chunk_count[i] : 0;
+        const int ex = mask_scan_block(c, warp_sums);
+        if (i < chunks) chunk_first[i] = carry + ex;
+        if (threadIdx.x == kMaskBlock - 1) carry_s = carry + ex + c;
+        __syncthreads();
+        carry = carry_s;
+        __syncthreads();
+    }
 }
 
 // The number of non-zero mask bytes (one atomic add per block).
@@ -674,6 +939,135 @@ __global__ void u_to_theta_kernel(const ModelConst mc, const R *u, const uint8_t
         if (mask && !mask[v]) continue;
         theta[i] = mc.lb_d[p] + static_cast<double>(u[p * n + v]) * (mc.ub_d[p] - mc.lb_d[p]);
     }
+}
+
+template <int KIND, int PREC>
+static const void *many_ptr_of(bool l1) {
+    return l1 ? reinterpret_cast<const void *>(&fit_many_kernel<KIND, PREC, true>)
+              : reinterpret_cast<const void *>(&fit_many_kernel<KIND, PREC, false>);
+}
+
+// The many-updates kernel of a kind and its shared memory for rows of row_stride floats.
+template <int PREC>
+static const void *many_ptr(int kind, bool l1, int row_stride, size_t *smem) {
+    using R = typename PrecTraits<PREC>::R;
+    switch (kind) {
+    case GAC_MODEL_MONOEXP: *smem = fit_many_smem<GAC_MODEL_MONOEXP, R>(row_stride); return many_ptr_of<GAC_MODEL_MONOEXP, PREC>(l1);
+    case GAC_MODEL_MWI3: *smem = fit_many_smem<GAC_MODEL_MWI3, R>(row_stride); return many_ptr_of<GAC_MODEL_MWI3, PREC>(l1);
+    case GAC_MODEL_SMT: *smem = fit_many_smem<GAC_MODEL_SMT, R>(row_stride); return many_ptr_of<GAC_MODEL_SMT, PREC>(l1);
+    default: *smem = fit_many_smem<GAC_MODEL_LINEAR_TEST, R>(row_stride); return many_ptr_of<GAC_MODEL_LINEAR_TEST, PREC>(l1);
+    }
+}
+
+// A device allocation of the call, returned to the pool in stream order.
+struct PoolBuf {
+    void *p = nullptr;
+    cudaStream_t s;
+    explicit PoolBuf(cudaStream_t stream) : s(stream) {}
+    PoolBuf(const PoolBuf &) = delete;
+    PoolBuf &operator=(const PoolBuf &) = delete;
+    cudaError_t make(size_t bytes) { return cudaMallocAsync(&p, bytes, s); }
+    ~PoolBuf() {
+        if (p) cudaFreeAsync(p, s);
+    }
+};
+
+// Fills *list (device) with the indices of the n_mask non-zero bytes of the mask.
+static cudaError_t list_masked(const uint8_t *d_mask, int n, int64_t n_mask, PoolBuf *list, cudaStream_t s) {
+    const int chunks = (n + kMaskChunk - 1) / kMaskChunk;
+    PoolBuf work(s);
+    cudaError_t e = list->make(static_cast<size_t>(n_mask) * sizeof(int));
+    if (e == cudaSuccess) e = work.make(2 * static_cast<size_t>(chunks) * sizeof(int));
+    if (e != cudaSuccess) return e;
+    int *count = static_cast<int *>(work.p), *first = count + chunks;
+    mask_list_kernel<<<chunks, kMaskBlock, 0, s>>>(d_mask, n, count, nullptr, nullptr);
+    mask_first_kernel<<<1, kMaskBlock, 0, s>>>(count, chunks, first);
+    mask_list_kernel<<<chunks, kMaskBlock, 0, s>>>(d_mask, n, count, first, static_cast<int *>(list->p));
+    return cudaGetLastError();
+}
+
+// Adam's bias corrections of update t, as the kernels of the precision take them.
+template <int PREC>
+static void bias_corrections(const gac_fit_opts *o, int t, double *c1, double *c2) {
+    *c1 = 1.0 - std::pow(o->beta1, t);
+    *c2 = 1.0 - std::pow(o->beta2, t);
+    if (PREC == GAC_PREC_FP32) {  // the FP32 kernels multiply by the reciprocals
+        *c1 = 1.0 / *c1;
+        *c2 = 1.0 / *c2;
+    }
+}
+
+// All updates of a fit without coupling between voxels; u, m1 and m2 as in
+// fit_run_prec, the result in u.  With stopping rules a launch takes fewer
+// updates, and one that runs past the stop is taken back: the state before it is
+// kept, and the updates up to the stop run again.  GAC_ERR_OOM: nothing has
+// been launched on the state.
+template <int PREC>
+static gac_status fit_uncoupled(const ModelConst &mc, const gac_fit_opts *o, const FitArgs<typename PrecTraits<PREC>::R> &fa,
+                                int n_list, typename PrecTraits<PREC>::R *u, typename PrecTraits<PREC>::R *m1,
+                                typename PrecTraits<PREC>::R *m2, size_t bytes_u, int *done, cudaStream_t s) {
+    using R = typename PrecTraits<PREC>::R;
+    const bool rules = o->tol > 0 || o->convergence_value > 0;
+    const int tiles = (n_list + 31) / 32;
+    // 64 MB of loss shares at most
+    const int chunk = static_cast<int>(std::max<int64_t>(4, std::min<int64_t>(rules ? 32 : kFitChunk, (int64_t(64) << 20) / (8 * static_cast<int64_t>(tiles)))));
+    PoolBuf part(s), saved(s), list_buf(s);
+    cudaError_t e = part.make(static_cast<size_t>(tiles) * chunk * sizeof(double));
+    if (e == cudaSuccess && rules) e = saved.make(3 * bytes_u);
+    if (e == cudaSuccess && fa.mask && n_list < fa.n) e = list_masked(fa.mask, static_cast<int>(fa.n), n_list, &list_buf, s);
+    if (e != cudaSuccess) return cuda_fail(e, "fit work arrays");
+    const int *list = static_cast<const int *>(list_buf.p);
+    size_t smem = 0;
+    const void *fn = many_ptr<PREC>(mc.kind, o->loss == GAC_FIT_L1, fa.row_stride, &smem);
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
+    char *sv = static_cast<char *>(saved.p);
+    auto copy_state = [&](bool save) {
+        R *const a[3] = {u, m1, m2};
+        for (int i = 0; i < 3; ++i) {
+            const cudaError_t c = save ? cudaMemcpyAsync(sv + i * bytes_u, a[i], bytes_u, cudaMemcpyDeviceToDevice, s)
+                                       : cudaMemcpyAsync(a[i], sv + i * bytes_u, bytes_u, cudaMemcpyDeviceToDevice, s);
+            if (c != cudaSuccess) return c;
+        }
+        return cudaSuccess;
+    };
+    auto run = [&](int t0, int count) {
+        FitSteps<R> steps;
+        for (int k = 0; k < kFitChunk; ++k) {
+            double c1 = 1.0, c2 = 1.0;
+            if (k < count) bias_corrections<PREC>(o, t0 + k, &c1, &c2);
+            steps.c1[k] = R(c1);
+            steps.c2[k] = R(c2);
+        }
+        double *pp = static_cast<double *>(part.p);
+        void *args[] = {const_cast<ModelConst *>(&mc), const_cast<FitArgs<R> *>(&fa), &list, &n_list, &u, &m1, &m2, &steps, &t0, &count, &pp};
+        return cudaLaunchKernel(fn, dim3(tiles), dim3(32), args, smem, s);
+    };
+    *done = 0;
+    for (int t = 1; t <= o->iterations;) {
+        const int count = std::min(chunk, o->iterations - t + 1);
+        if (rules && (e = copy_state(true)) != cudaSuccess) return cuda_fail(e, "fit state");
+        if ((e = run(t, count)) != cudaSuccess) return cuda_fail(e, "fit updates");
+        fit_losses_kernel<<<std::min(tiles, kFitLossBlocks), kFitChunk, 0, s>>>(fa, static_cast<const double *>(part.p), tiles, t, count);
+        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "fit losses");
+        *done = t + count - 1;
+        if (rules) {
+            int flag[2] = {0, 0};  // stop, done
+            if ((e = cudaMemcpyAsync(flag, fa.stop, sizeof flag, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return cuda_fail(e, "fit flag");
+            if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "fit");
+            if (flag[0]) {
+                if (flag[1] < *done) {
+                    if ((e = copy_state(false)) != cudaSuccess) return cuda_fail(e, "fit state");
+                    if ((e = run(t, flag[1] - t + 1)) != cudaSuccess) return cuda_fail(e, "fit updates");
+                }
+                *done = flag[1];
+                break;
+            }
+        }
+        t += count;
+    }
+    return GAC_OK;
 }
 
 template <int PREC, bool L1>
@@ -762,7 +1156,9 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     // work arrays: u (two buffers), Adam moments, block losses, history, flags
     const int I = o->iterations;
     const size_t bytes_u = static_cast<size_t>(N) * P * RB;
-    const size_t total = 4 * bytes_u + grid * sizeof(double) + static_cast<size_t>(std::max(I, 1)) * sizeof(double) + 3 * sizeof(int);
+    // the total-variation term couples voxels, and an update is then one launch
+    const bool coupled = o->tv_params != 0 && static_cast<R>(o->tv_lambda / static_cast<double>(n_mask)) != R(0);
+    const size_t total = 4 * bytes_u + std::max(grid, kFitLossBlocks * kFitChunk) * sizeof(double) + static_cast<size_t>(std::max(I, 1)) * sizeof(double) + 3 * sizeof(int);
     void *base = nullptr;
     e = cudaMallocAsync(&base, total, s);
     if (e != cudaSuccess) return cuda_fail(e, "fit work arrays");
@@ -774,9 +1170,8 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     char *b = static_cast<char *>(base);
     void *u0 = b, *u1 = b + bytes_u, *m1 = b + 2 * bytes_u, *m2 = b + 3 * bytes_u;
     double *block_loss = reinterpret_cast<double *>(b + 4 * bytes_u);
-    double *hist = block_loss + grid;
+    double *hist = block_loss + std::max(grid, kFitLossBlocks * kFitChunk);
     int *flags = reinterpret_cast<int *>(hist + std::max(I, 1));  // stop, done, arrival count
-    if ((e = cudaMemsetAsync(m1, 0, 2 * bytes_u, s)) != cudaSuccess) return cuda_fail(e, "fit memset");
     if ((e = cudaMemsetAsync(flags, 0, 3 * sizeof(int), s)) != cudaSuccess) return cuda_fail(e, "fit memset");
     const int conv_grid = static_cast<int>(std::min<int64_t>((N * P + 255) / 256, static_cast<int64_t>(sms) * 8));
     theta_to_u_kernel<R><<<conv_grid, 256, 0, s>>>(mc, static_cast<const double *>(d_theta.ptr), N, static_cast<R *>(u0));
@@ -812,39 +1207,50 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     fa.fdiv = N < (int64_t(1) << 24);
     fa.inv_nx = 1.0f / static_cast<float>(o->nx);
     fa.inv_ny = 1.0f / static_cast<float>(o->ny);
-    // iterations in chunks; the stop flag is read between chunks
-    constexpr int kChunk = 128;
-    int t = 1;
-    while (t <= I) {
-        const int t_end = std::min(I, t + kChunk - 1);
-        for (; t <= t_end; ++t) {
-            double c1 = 1.0 - std::pow(o->beta1, t), c2 = 1.0 - std::pow(o->beta2, t);
-            if (PREC == GAC_PREC_FP32) {  // the FP32 kernel multiplies by the reciprocals
-                c1 = 1.0 / c1;
-                c2 = 1.0 / c2;
-            }
-            const void *ui = (t & 1) ? u0 : u1;
-            void *uo = (t & 1) ? u1 : u0;
-            if ((e = launch_step_kind<PREC>(mc.kind, l1, grid, smem, s, mc, fa, ui, uo, m1, m2, c1, c2, t)) != cudaSuccess)
-                return cuda_fail(e, "fit step");
-        }
-        int stop = 0;
-        if ((e = cudaMemcpyAsync(&stop, flags, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-            return cuda_fail(e, "fit flag");
-        if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "fit");
-        if (stop) break;
-    }
     int done = 0;
-    if ((e = cudaMemcpyAsync(&done, flags + 1, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-        return cuda_fail(e, "fit done");
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "fit");
+    bool stepwise = coupled;  // a launch per update
+    if (!coupled) {
+        st = fit_uncoupled<PREC>(mc, o, fa, static_cast<int>(n_mask), static_cast<R *>(u0), static_cast<R *>(m1),
+                                 static_cast<R *>(m2), bytes_u, &done, s);
+        if (st == GAC_ERR_OOM) {  // no memory for its loss shares: the other path needs none
+            clear_error();
+            stepwise = true;
+        } else if (st != GAC_OK) {
+            return st;
+        }
+    }
+    if (stepwise) {
+        if ((e = cudaMemsetAsync(m1, 0, 2 * bytes_u, s)) != cudaSuccess) return cuda_fail(e, "fit memset");
+        // iterations in chunks; the stop flag is read between chunks
+        constexpr int kChunk = 128;
+        int t = 1;
+        while (t <= I) {
+            const int t_end = std::min(I, t + kChunk - 1);
+            for (; t <= t_end; ++t) {
+                double c1, c2;
+                bias_corrections<PREC>(o, t, &c1, &c2);
+                const void *ui = (t & 1) ? u0 : u1;
+                void *uo = (t & 1) ? u1 : u0;
+                if ((e = launch_step_kind<PREC>(mc.kind, l1, grid, smem, s, mc, fa, ui, uo, m1, m2, c1, c2, t)) != cudaSuccess)
+                    return cuda_fail(e, "fit step");
+            }
+            int stop = 0;
+            if ((e = cudaMemcpyAsync(&stop, flags, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+                return cuda_fail(e, "fit flag");
+            if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "fit");
+            if (stop) break;
+        }
+        if ((e = cudaMemcpyAsync(&done, flags + 1, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+            return cuda_fail(e, "fit done");
+        if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "fit");
+    }
     if (iterations_done) *iterations_done = done;
     if (loss_history && done > 0) {
         if ((e = cudaMemcpyAsync(loss_history, hist, done * sizeof(double), cudaMemcpyDefault, s)) != cudaSuccess)
             return cuda_fail(e, "loss history");
     }
-    // u of the last update (iteration `done` wrote buffer (done & 1) ? u1 : u0) -> theta
-    const void *u_fin = done == 0 ? u0 : ((done & 1) ? u1 : u0);
+    // u of the last update (stepwise, iteration `done` wrote buffer (done & 1) ? u1 : u0) -> theta
+    const void *u_fin = stepwise && (done & 1) ? u1 : u0;
     u_to_theta_kernel<R><<<conv_grid, 256, 0, s>>>(mc, static_cast<const R *>(u_fin), d_mask, N,
                                                    static_cast<double *>(d_theta.ptr));
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "u to theta");
