@@ -188,12 +188,12 @@ struct PrecTraits<GAC_PREC_FP64> {
     using Acc = PlainSumD;
 };
 
-template <int KIND, int PREC, int REP = gtab_copies(KIND)>
+template <int KIND, int PREC, int REP = gtab_copies(KIND), bool TWO = true>
 __device__ __forceinline__ typename PrecTraits<PREC>::R loglik_any(
     const typename PrecTraits<PREC>::R *th, const float *y, typename PrecTraits<PREC>::R inv_s2,
     const ModelConst &mc) {
     if constexpr (PREC == GAC_PREC_FP64) return loglik_d<KIND>(th, y, inv_s2, mc);
-    else return loglik_f<KIND, typename PrecTraits<PREC>::Acc, REP>(th, y, inv_s2, mc);
+    else return loglik_f<KIND, typename PrecTraits<PREC>::Acc, REP, TWO>(th, y, inv_s2, mc);
 }
 
 // MIXED acceptance, FP64 semantics at FP32 cost, from lu32 = __logf(u01_f(w)).
