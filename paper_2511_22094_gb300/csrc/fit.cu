@@ -56,6 +56,16 @@ struct FitArgs {
     double tol, conv_value;
     int window;
     double *block_loss;    // [gridDim.x]
+    // The n_list voxels to visit: the fitted ones in order, or nullptr: voxels 0
+    // .. n_list - 1, of which the mask leaves some out.  Parameters and moments
+    // are [P][n_list], in the list's order.
+    const int *list;
+    int n_list;
+    // With a list, the penalised maps once more over the whole grid ([maps][N],
+    // in the order of their parameters), for the neighbours: read from tv_in,
+    // and each update's new values written to tv_out.
+    const R *tv_in;
+    R *tv_out;
 };
 
 // sign(x) with sign(0) = 0, branch-free (a select and a sign-bit copy)
@@ -320,9 +330,6 @@ __device__ __forceinline__ R fit_adam(const FitArgs<R> &fa, R u, R g, R &a, R &b
     return fmin(fmax(u - stepu, R(0)), R(1));
 }
 
-// One voxel's update: forward model and Jacobian against its staged data row
-// y, the loss gradient, the total-variation subgradient, Adam and the box.
-// Returns the voxel's share of the loss (0 outside the mask).
 // One voxel's update in two phases around the warp's staging points (the
 // kernel below): phase A issues the loads of the total-variation neighbours
 // and evaluates the model and its Jacobian against the staged data row y
@@ -344,7 +351,7 @@ __device__ __forceinline__ int fit_offset(const FitTv<KIND, R> &tv, int j, const
 
 // Phase A.  The neighbours' mask bytes and values load first and are used in
 // phase B, so nothing waits on them before the model.
-template <int KIND, int PREC, bool L1>
+template <int KIND, int PREC, bool L1, bool LIST>
 __device__ __forceinline__ void fit_phase_a(const ModelConst &mc, const FitArgs<typename PrecTraits<PREC>::R> &fa, int v,
                                             const float *y, const typename PrecTraits<PREC>::R (&u)[model_n_par(KIND)],
                                             bool inside, typename PrecTraits<PREC>::R w,
@@ -382,19 +389,22 @@ __device__ __forceinline__ void fit_phase_a(const ModelConst &mc, const FitArgs<
         tv.p0 = __ffs(fa.tv_params) - 1;
         if (tv.p0 < P) {
 #pragma unroll
-            for (int j = 0; j < 6; ++j) tv.nb0[j] = u_in[tv.p0 * n + v + fit_offset(tv, j, step)];
+            for (int j = 0; j < 6; ++j) {
+                if constexpr (LIST) tv.nb0[j] = fa.tv_in[v + fit_offset(tv, j, step)];
+                else tv.nb0[j] = u_in[tv.p0 * n + v + fit_offset(tv, j, step)];
+            }
         }
     }
     loss = R(0);
 #pragma unroll
     for (int p = 0; p < P; ++p) g[p] = R(0);
-    if (inside) fit_loss_grad<KIND, PREC, L1>(mc, y, u, w, loss, g);
+    if (LIST || inside) fit_loss_grad<KIND, PREC, L1>(mc, y, u, w, loss, g);
 }
 
 // Phase B; returns the voxel's share of the loss (0 outside the mask).
-template <int KIND, int PREC>
+template <int KIND, int PREC, bool LIST>
 __device__ __forceinline__ typename PrecTraits<PREC>::R fit_phase_b(
-    const ModelConst &mc, const FitArgs<typename PrecTraits<PREC>::R> &fa, int v,
+    const ModelConst &mc, const FitArgs<typename PrecTraits<PREC>::R> &fa, int e, int v,
     const typename PrecTraits<PREC>::R (&u)[model_n_par(KIND)], bool inside, const FitTv<KIND, typename PrecTraits<PREC>::R> &tv_in,
     typename PrecTraits<PREC>::R loss, typename PrecTraits<PREC>::R (&g)[model_n_par(KIND)],
     const typename PrecTraits<PREC>::R *mo, const typename PrecTraits<PREC>::R *u_in, typename PrecTraits<PREC>::R *u_out,
@@ -403,7 +413,7 @@ __device__ __forceinline__ typename PrecTraits<PREC>::R fit_phase_b(
     using R = typename PrecTraits<PREC>::R;
     constexpr int P = model_n_par(KIND);
     const int n = static_cast<int>(fa.n);
-    if (!inside) {
+    if (!LIST && !inside) {
 #pragma unroll
         for (int p = 0; p < P; ++p) u_out[p * n + v] = u[p];
         return R(0);
@@ -423,11 +433,15 @@ __device__ __forceinline__ typename PrecTraits<PREC>::R fit_phase_b(
             for (int j = 0; j < 6; ++j) nbit &= ~(static_cast<unsigned>(tv_in.nmask[j] == 0) << j);
         }
 #pragma unroll
-        for (int p = 0; p < P; ++p) {
+        for (int p = 0, map = 0; p < P; ++p) {
             if (!((fa.tv_params >> p) & 1u)) continue;
             R nb[6];
 #pragma unroll
-            for (int j = 0; j < 6; ++j) nb[j] = p == tv_in.p0 ? tv_in.nb0[j] : u_in[p * n + v + fit_offset(tv_in, j, step)];
+            for (int j = 0; j < 6; ++j) {
+                if constexpr (LIST) nb[j] = p == tv_in.p0 ? tv_in.nb0[j] : fa.tv_in[map * n + v + fit_offset(tv_in, j, step)];
+                else nb[j] = p == tv_in.p0 ? tv_in.nb0[j] : u_in[p * n + v + fit_offset(tv_in, j, step)];
+            }
+            ++map;
             R tv = R(0), tv_loss = R(0);
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
@@ -442,12 +456,15 @@ __device__ __forceinline__ typename PrecTraits<PREC>::R fit_phase_b(
             vl += fa.lambda_n * tv_loss;
         }
     }
+    const int stride = LIST ? fa.n_list : n;
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
+    for (int p = 0, map = 0; p < P; ++p) {
         R a = mo[p * 32], b = mo[(P + p) * 32];
-        u_out[p * n + v] = fit_adam(fa, u[p], g[p], a, b, c1, c2);
-        m1[p * n + v] = a;
-        m2[p * n + v] = b;
+        const R un = fit_adam(fa, u[p], g[p], a, b, c1, c2);
+        u_out[p * stride + e] = un;
+        m1[p * stride + e] = a;
+        m2[p * stride + e] = b;
+        if (LIST && ((fa.tv_params >> p) & 1u)) fa.tv_out[map++ * n + v] = un;
     }
     return vl;
 }
@@ -518,6 +535,38 @@ __host__ __device__ constexpr size_t fit_warp_smem(int row_stride, int P, size_t
     return 32 * static_cast<size_t>(row_stride) * sizeof(float) + 2 * static_cast<size_t>(P) * 32 * rbytes;
 }
 
+template <class FA>
+__device__ void fit_check(const FA &fa, int n_blocks, int t, double *red);
+
+// The end of an update: the block's share of the loss, summed in a fixed order
+// (lanes by shuffles within each warp, then the warps); the last block to finish
+// sums the shares.
+template <class R>
+__device__ __forceinline__ void fit_block_loss(const FitArgs<R> &fa, R my_loss, int t_iter) {
+    __shared__ double red[kFitBlock];
+    __shared__ bool last;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double sum = static_cast<double>(my_loss);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+    if (lane == 0) red[warp] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+#pragma unroll
+        for (int i = 0; i < kFitWarps; ++i) t += red[i];
+        fa.block_loss[blockIdx.x] = t;
+        __threadfence();  // the share is visible before the count says so
+        last = atomicAdd(fa.arrive, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (last) {  // every other block's share has landed
+        __threadfence();
+        fit_check(fa, gridDim.x, t_iter, red);
+        if (threadIdx.x == 0) *fa.arrive = 0u;  // for the next launch, which starts after this one ends
+    }
+}
+
 template <int KIND, int PREC, bool L1>
 __global__ void __launch_bounds__(kFitBlock, fit_min_blocks(PREC)) fit_step_kernel(const ModelConst mc, const FitArgs<typename PrecTraits<PREC>::R> fa,
                                                              const typename PrecTraits<PREC>::R *u_in,
@@ -528,8 +577,6 @@ __global__ void __launch_bounds__(kFitBlock, fit_min_blocks(PREC)) fit_step_kern
                                                              typename PrecTraits<PREC>::R c2, int t_iter) {
     using R = typename PrecTraits<PREC>::R;
     constexpr int P = model_n_par(KIND);
-    __shared__ double red[kFitBlock];
-    __shared__ bool last;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // launched as a programmatic dependent of the previous update: its blocks
     // become resident while that launch drains, and wait here until it has
@@ -607,39 +654,114 @@ __global__ void __launch_bounds__(kFitBlock, fit_min_blocks(PREC)) fit_step_kern
         const R w = w_n;
         FitTv<KIND, R> tv;
         R loss, g[P];
-        if (active) fit_phase_a<KIND, PREC, L1>(mc, fa, v, rows_s + lane * fa.row_stride, u, inside, w, u_in, tv, loss, g);
+        if (active) fit_phase_a<KIND, PREC, L1, false>(mc, fa, v, rows_s + lane * fa.row_stride, u, inside, w, u_in, tv, loss, g);
         __syncwarp();  // the model has read every row: the buffer takes the next tile's
         const int next = tile + stride;
         if (next < n_tiles) stage_rows(next);
         cp_async_commit();
         load_next(next * 32 + lane);
-        if (active) my_loss += fit_phase_b<KIND, PREC>(mc, fa, v, u, inside, tv, loss, g, mo_s + lane, u_in, u_out, m1, m2, c1, c2);
+        if (active) my_loss += fit_phase_b<KIND, PREC, false>(mc, fa, v, v, u, inside, tv, loss, g, mo_s + lane, u_in, u_out, m1, m2, c1, c2);
         __syncwarp();  // phase B has read every moment
         if (next < n_tiles) stage_moments(next);
         cp_async_commit();
     }
     cp_async_wait<0>();
-    // the block's share of the loss, summed in a fixed order: lanes by
-    // shuffles within each warp, then the warps
-    double sum = static_cast<double>(my_loss);
+    fit_block_loss(fa, my_loss, t_iter);
+}
+
+// The same over the list of fitted voxels of a masked grid: parameters and
+// moments lie in the list's order, so that their accesses stay whole lines, and
+// the penalised maps once more over the grid, where the neighbours read them.
+// Tiles hold fitted voxels only: 552,960 voxels, 68% inside, 3-pool, 61 -> 50 us
+// an update.
+template <int KIND, int PREC, bool L1>
+__global__ void __launch_bounds__(kFitBlock, fit_min_blocks(PREC)) fit_list_kernel(const ModelConst mc, const FitArgs<typename PrecTraits<PREC>::R> fa,
+                                                             const typename PrecTraits<PREC>::R *u_in,
+                                                             typename PrecTraits<PREC>::R *u_out,
+                                                             typename PrecTraits<PREC>::R *m1,
+                                                             typename PrecTraits<PREC>::R *m2,
+                                                             typename PrecTraits<PREC>::R c1,
+                                                             typename PrecTraits<PREC>::R c2, int t_iter) {
+    using R = typename PrecTraits<PREC>::R;
+    constexpr int P = model_n_par(KIND);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    // what no update changes (the first rows, the list) loads before the wait for
+    // the previous update.  (Letting the next update start earlier still, by
+    // griddepcontrol.launch_dependents here, stacked its blocks on the SMs that
+    // the current one leaves free: 98,304 voxels 16.7 -> 22.1 us an update.)
+    model_smem_load<KIND, 1>(mc);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int M = mc.n_meas;
+    const int cnt = fa.n_list;
+    const int n_tiles = (cnt + 31) / 32;
+    unsigned char *wmem = smem_raw + warp * fit_warp_smem(fa.row_stride, P, sizeof(R));
+    float *rows_s = reinterpret_cast<float *>(wmem);
+    R *mo_s = reinterpret_cast<R *>(wmem + 32 * static_cast<size_t>(fa.row_stride) * sizeof(float));
+    auto voxel = [&](int e) { return e < cnt ? fa.list[e] : 0; };
+    auto stage_rows = [&](int tile, int v) { fit_stage_rows(fa, M, v, min(32, cnt - tile * 32), lane, rows_s); };
+    auto stage_moments = [&](int tile) {
+        const int e = tile * 32 + lane;
+        if (e < cnt) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
-    if (lane == 0) red[warp] = sum;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
+            for (int p = 0; p < P; ++p) {
+                cp_async_elem(mo_s + p * 32 + lane, m1 + p * cnt + e);
+                cp_async_elem(mo_s + (P + p) * 32 + lane, m2 + p * cnt + e);
+            }
+        }
+    };
+    // the lane's next voxel: parameters and weight
+    R un[P];
+    R w_n = R(1);
+    auto load_next = [&](int e, int v) {
+        if (e < cnt) {
 #pragma unroll
-        for (int i = 0; i < kFitWarps; ++i) t += red[i];
-        fa.block_loss[blockIdx.x] = t;
-        __threadfence();  // the share is visible before the count says so
-        last = atomicAdd(fa.arrive, 1u) == gridDim.x - 1;
+            for (int p = 0; p < P; ++p) un[p] = u_in[p * cnt + e];
+            w_n = fa.weight ? R(fa.weight[v]) : R(1);
+        }
+    };
+    R my_loss = R(0);
+    const int stride = gridDim.x * kFitWarps;
+    int tile = blockIdx.x * kFitWarps + warp;
+    // the lane's voxel and its next one (read a tile ahead)
+    int v = voxel(tile * 32 + lane), v_next = voxel((tile + stride) * 32 + lane);
+    if (tile < n_tiles) stage_rows(tile, v);
+    __syncthreads();  // the model's table
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (*fa.stop) {  // the same for every thread
+        cp_async_commit();
+        cp_async_wait<0>();
+        return;
     }
-    __syncthreads();
-    if (last) {  // every other block's share has landed
-        __threadfence();
-        fit_check(fa, gridDim.x, t_iter, red);
-        if (threadIdx.x == 0) *fa.arrive = 0u;  // for the next launch, which starts after this one ends
+    if (tile < n_tiles) stage_moments(tile);
+    cp_async_commit();
+    load_next(tile * 32 + lane, v);
+    for (; tile < n_tiles; tile += stride) {
+        cp_async_wait<0>();
+        __syncwarp();
+        const int e = tile * 32 + lane;
+        const bool active = e < cnt;
+        R u[P];
+#pragma unroll
+        for (int p = 0; p < P; ++p) u[p] = un[p];
+        const R w = w_n;
+        FitTv<KIND, R> tv;
+        R loss, g[P];
+        if (active) fit_phase_a<KIND, PREC, L1, true>(mc, fa, v, rows_s + lane * fa.row_stride, u, true, w, u_in, tv, loss, g);
+        __syncwarp();  // the model has read every row: the buffer takes the next tile's
+        const int next = tile + stride;
+        if (next < n_tiles) stage_rows(next, v_next);
+        cp_async_commit();
+        load_next(next * 32 + lane, v_next);
+        const int v_after = voxel((next + stride) * 32 + lane);
+        if (active) my_loss += fit_phase_b<KIND, PREC, true>(mc, fa, e, v, u, true, tv, loss, g, mo_s + lane, u_in, u_out, m1, m2, c1, c2);
+        __syncwarp();  // phase B has read every moment
+        if (next < n_tiles) stage_moments(next);
+        cp_async_commit();
+        v = v_next;
+        v_next = v_after;
     }
+    cp_async_wait<0>();
+    fit_block_loss(fa, my_loss, t_iter);
 }
 
 // The stopping rules after iteration t, whose loss is hist[t - 1]: loss < tol, or
@@ -713,12 +835,11 @@ __host__ __device__ constexpr size_t fit_many_smem(int row_stride) {
            (fit_reg_moments<KIND>() ? 0 : 2 * static_cast<size_t>(model_n_par(KIND)) * 32 * sizeof(R));
 }
 
-// Updates t0 .. t0 + count - 1 (t0 = 1: from zero moments) of the voxels
-// list[0 .. n_list) (list = nullptr: voxels 0 .. n_list - 1), u and the moments in
-// place; part[tile][count]: the tile's share of each update's loss.
+// Updates t0 .. t0 + count - 1 (t0 = 1: from zero moments) of the fitted
+// voxels, u and the moments in place; part[tile][count]: the tile's share of each update's loss.
 template <int KIND, int PREC, bool L1>
 __global__ void __launch_bounds__(32, PREC == GAC_PREC_FP32 ? 20 : 8)
-    fit_many_kernel(const ModelConst mc, const FitArgs<typename PrecTraits<PREC>::R> fa, const int *list, int n_list,
+    fit_many_kernel(const ModelConst mc, const FitArgs<typename PrecTraits<PREC>::R> fa,
                     typename PrecTraits<PREC>::R *u_io, typename PrecTraits<PREC>::R *m1, typename PrecTraits<PREC>::R *m2,
                     const __grid_constant__ FitSteps<typename PrecTraits<PREC>::R> steps, int t0, int count, double *part) {
     using R = typename PrecTraits<PREC>::R;
@@ -730,20 +851,20 @@ __global__ void __launch_bounds__(32, PREC == GAC_PREC_FP32 ? 20 : 8)
     R *mo = loss_s + kFitFlush * 33 + threadIdx.x;
     const int lane = threadIdx.x;
     const int M = mc.n_meas;
-    const int n = static_cast<int>(fa.n);
+    const int n = fa.n_list;
     const int i0 = blockIdx.x * 32;
-    const int rows = min(32, n_list - i0);
+    const int rows = min(32, fa.n_list - i0);
     const bool active = lane < rows;
     const int e = i0 + (active ? lane : rows - 1);
-    const int v = list ? list[e] : e;
+    const int v = fa.list ? fa.list[e] : e;
     model_smem_load<KIND, 1>(mc);
     fit_stage_rows(fa, M, v, rows, lane, rows_s);
     cp_async_commit();
     R u[P], ma[P], mb[P];
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        u[p] = u_io[p * n + v];
-        const R a = t0 > 1 ? m1[p * n + v] : R(0), b = t0 > 1 ? m2[p * n + v] : R(0);
+        u[p] = u_io[p * n + e];
+        const R a = t0 > 1 ? m1[p * n + e] : R(0), b = t0 > 1 ? m2[p * n + e] : R(0);
         if constexpr (kReg) {
             ma[p] = a;
             mb[p] = b;
@@ -801,9 +922,9 @@ __global__ void __launch_bounds__(32, PREC == GAC_PREC_FP32 ? 20 : 8)
     if (active) {
 #pragma unroll
         for (int p = 0; p < P; ++p) {
-            u_io[p * n + v] = u[p];
-            m1[p * n + v] = kReg ? ma[p] : mo[p * 32];
-            m2[p * n + v] = kReg ? mb[p] : mo[(P + p) * 32];
+            u_io[p * n + e] = u[p];
+            m1[p * n + e] = kReg ? ma[p] : mo[p * 32];
+            m2[p * n + e] = kReg ? mb[p] : mo[(P + p) * 32];
         }
     }
 }
@@ -916,28 +1037,35 @@ __global__ void count_mask_kernel(const uint8_t *mask, int64_t n, unsigned long 
     }
 }
 
-// theta [N][P] (double) <-> u [P][N]; outside the mask theta is left alone.
+// theta [N][P] (double) <-> u [P][n_list], and the penalised maps over the grid
+// (tv_out) when there is a list.
 template <class R>
-__global__ void theta_to_u_kernel(const ModelConst mc, const double *theta, int64_t n, R *u) {
+__global__ void theta_to_u_kernel(const ModelConst mc, const FitArgs<R> fa, const double *theta, R *u) {
     const int P = mc.n_par;
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n * P;
+    const int64_t total = static_cast<int64_t>(fa.n_list) * P;
+    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int64_t v = i / P;
-        const int p = static_cast<int>(i - v * P);
+        const int64_t e = i / P;
+        const int p = static_cast<int>(i - e * P);
+        const int64_t v = fa.list ? fa.list[e] : e;
         const double range = mc.ub_d[p] - mc.lb_d[p];
-        const double x = range > 0 ? (theta[i] - mc.lb_d[p]) / range : 0.0;
-        u[p * n + v] = static_cast<R>(fmin(fmax(x, 0.0), 1.0));
+        const double x = range > 0 ? (theta[v * P + p] - mc.lb_d[p]) / range : 0.0;
+        const R un = static_cast<R>(fmin(fmax(x, 0.0), 1.0));
+        u[p * static_cast<int64_t>(fa.n_list) + e] = un;
+        if (fa.list && fa.tv_out && ((fa.tv_params >> p) & 1u)) fa.tv_out[__popc(fa.tv_params & ((1u << p) - 1u)) * fa.n + v] = un;
     }
 }
 template <class R>
-__global__ void u_to_theta_kernel(const ModelConst mc, const R *u, const uint8_t *mask, int64_t n, double *theta) {
+__global__ void u_to_theta_kernel(const ModelConst mc, const FitArgs<R> fa, const R *u, double *theta) {
     const int P = mc.n_par;
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n * P;
+    const int64_t total = static_cast<int64_t>(fa.n_list) * P;
+    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int64_t v = i / P;
-        const int p = static_cast<int>(i - v * P);
-        if (mask && !mask[v]) continue;
-        theta[i] = mc.lb_d[p] + static_cast<double>(u[p * n + v]) * (mc.ub_d[p] - mc.lb_d[p]);
+        const int64_t e = i / P;
+        const int p = static_cast<int>(i - e * P);
+        const int64_t v = fa.list ? fa.list[e] : e;
+        if (!fa.list && fa.mask && !fa.mask[v]) continue;  // a voxel outside keeps its theta
+        theta[v * P + p] = mc.lb_d[p] + static_cast<double>(u[p * static_cast<int64_t>(fa.n_list) + e]) * (mc.ub_d[p] - mc.lb_d[p]);
     }
 }
 
@@ -1004,19 +1132,17 @@ static void bias_corrections(const gac_fit_opts *o, int t, double *c1, double *c
 // been launched on the state.
 template <int PREC>
 static gac_status fit_uncoupled(const ModelConst &mc, const gac_fit_opts *o, const FitArgs<typename PrecTraits<PREC>::R> &fa,
-                                int n_list, typename PrecTraits<PREC>::R *u, typename PrecTraits<PREC>::R *m1,
+                                typename PrecTraits<PREC>::R *u, typename PrecTraits<PREC>::R *m1,
                                 typename PrecTraits<PREC>::R *m2, size_t bytes_u, int *done, cudaStream_t s) {
     using R = typename PrecTraits<PREC>::R;
     const bool rules = o->tol > 0 || o->convergence_value > 0;
-    const int tiles = (n_list + 31) / 32;
+    const int tiles = (fa.n_list + 31) / 32;
     // 64 MB of loss shares at most
     const int chunk = static_cast<int>(std::max<int64_t>(4, std::min<int64_t>(rules ? 32 : kFitChunk, (int64_t(64) << 20) / (8 * static_cast<int64_t>(tiles)))));
-    PoolBuf part(s), saved(s), list_buf(s);
+    PoolBuf part(s), saved(s);
     cudaError_t e = part.make(static_cast<size_t>(tiles) * chunk * sizeof(double));
     if (e == cudaSuccess && rules) e = saved.make(3 * bytes_u);
-    if (e == cudaSuccess && fa.mask && n_list < fa.n) e = list_masked(fa.mask, static_cast<int>(fa.n), n_list, &list_buf, s);
     if (e != cudaSuccess) return cuda_fail(e, "fit work arrays");
-    const int *list = static_cast<const int *>(list_buf.p);
     size_t smem = 0;
     const void *fn = many_ptr<PREC>(mc.kind, o->loss == GAC_FIT_L1, fa.row_stride, &smem);
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -1041,7 +1167,7 @@ static gac_status fit_uncoupled(const ModelConst &mc, const gac_fit_opts *o, con
             steps.c2[k] = R(c2);
         }
         double *pp = static_cast<double *>(part.p);
-        void *args[] = {const_cast<ModelConst *>(&mc), const_cast<FitArgs<R> *>(&fa), &list, &n_list, &u, &m1, &m2, &steps, &t0, &count, &pp};
+        void *args[] = {const_cast<ModelConst *>(&mc), const_cast<FitArgs<R> *>(&fa), &u, &m1, &m2, &steps, &t0, &count, &pp};
         return cudaLaunchKernel(fn, dim3(tiles), dim3(32), args, smem, s);
     };
     *done = 0;
@@ -1070,25 +1196,29 @@ static gac_status fit_uncoupled(const ModelConst &mc, const gac_fit_opts *o, con
     return GAC_OK;
 }
 
-template <int PREC, bool L1>
-static const void *step_ptr(int kind) {
+template <int KIND, int PREC>
+static const void *step_ptr_of(bool l1, bool list) {
+    return l1 ? (list ? reinterpret_cast<const void *>(&fit_list_kernel<KIND, PREC, true>)
+                      : reinterpret_cast<const void *>(&fit_step_kernel<KIND, PREC, true>))
+              : (list ? reinterpret_cast<const void *>(&fit_list_kernel<KIND, PREC, false>)
+                      : reinterpret_cast<const void *>(&fit_step_kernel<KIND, PREC, false>));
+}
+
+template <int PREC>
+static const void *step_ptr(int kind, bool l1, bool list) {
     switch (kind) {
-    case GAC_MODEL_MONOEXP: return reinterpret_cast<const void *>(&fit_step_kernel<GAC_MODEL_MONOEXP, PREC, L1>);
-    case GAC_MODEL_MWI3: return reinterpret_cast<const void *>(&fit_step_kernel<GAC_MODEL_MWI3, PREC, L1>);
-    case GAC_MODEL_SMT: return reinterpret_cast<const void *>(&fit_step_kernel<GAC_MODEL_SMT, PREC, L1>);
-    default: return reinterpret_cast<const void *>(&fit_step_kernel<GAC_MODEL_LINEAR_TEST, PREC, L1>);
+    case GAC_MODEL_MONOEXP: return step_ptr_of<GAC_MODEL_MONOEXP, PREC>(l1, list);
+    case GAC_MODEL_MWI3: return step_ptr_of<GAC_MODEL_MWI3, PREC>(l1, list);
+    case GAC_MODEL_SMT: return step_ptr_of<GAC_MODEL_SMT, PREC>(l1, list);
+    default: return step_ptr_of<GAC_MODEL_LINEAR_TEST, PREC>(l1, list);
     }
 }
 
-template <int KIND, int PREC>
-static cudaError_t launch_step(bool l1, int grid, size_t smem, cudaStream_t s, const ModelConst &mc,
-                               const FitArgs<typename PrecTraits<PREC>::R> &fa, const void *u_in, void *u_out,
-                               void *m1, void *m2, double c1, double c2, int t) {
-    using R = typename PrecTraits<PREC>::R;
-    auto *ui = static_cast<const R *>(u_in);
-    auto *uo = static_cast<R *>(u_out);
-    // programmatic stream serialization: the launch may begin while the
-    // previous kernel in the stream drains (the kernel waits for it first)
+// One update, with programmatic stream serialization: the launch may begin
+// while the previous kernel in the stream drains (the kernel waits for it first).
+template <class R>
+static cudaError_t launch_step(const void *fn, int grid, size_t smem, cudaStream_t s, const ModelConst &mc, const FitArgs<R> &fa,
+                               const R *u_in, R *u_out, R *m1, R *m2, R c1, R c2, int t) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kFitBlock);
@@ -1099,22 +1229,8 @@ static cudaError_t launch_step(bool l1, int grid, size_t smem, cudaStream_t s, c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    auto *m1r = static_cast<R *>(m1);
-    auto *m2r = static_cast<R *>(m2);
-    if (l1) return cudaLaunchKernelEx(&cfg, fit_step_kernel<KIND, PREC, true>, mc, fa, ui, uo, m1r, m2r, R(c1), R(c2), t);
-    return cudaLaunchKernelEx(&cfg, fit_step_kernel<KIND, PREC, false>, mc, fa, ui, uo, m1r, m2r, R(c1), R(c2), t);
-}
-
-template <int PREC>
-static cudaError_t launch_step_kind(int kind, bool l1, int grid, size_t smem, cudaStream_t s, const ModelConst &mc,
-                                    const FitArgs<typename PrecTraits<PREC>::R> &fa, const void *u_in, void *u_out,
-                                    void *m1, void *m2, double c1, double c2, int t) {
-    switch (kind) {
-    case GAC_MODEL_MONOEXP: return launch_step<GAC_MODEL_MONOEXP, PREC>(l1, grid, smem, s, mc, fa, u_in, u_out, m1, m2, c1, c2, t);
-    case GAC_MODEL_MWI3: return launch_step<GAC_MODEL_MWI3, PREC>(l1, grid, smem, s, mc, fa, u_in, u_out, m1, m2, c1, c2, t);
-    case GAC_MODEL_SMT: return launch_step<GAC_MODEL_SMT, PREC>(l1, grid, smem, s, mc, fa, u_in, u_out, m1, m2, c1, c2, t);
-    default: return launch_step<GAC_MODEL_LINEAR_TEST, PREC>(l1, grid, smem, s, mc, fa, u_in, u_out, m1, m2, c1, c2, t);
-    }
+    void *args[] = {const_cast<ModelConst *>(&mc), const_cast<FitArgs<R> *>(&fa), &u_in, &u_out, &m1, &m2, &c1, &c2, &t};
+    return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
 template <int PREC>
@@ -1142,23 +1258,38 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
         return fail(GAC_ERR_INVALID_ARG, "fit: %d measurements per voxel need %zu bytes of staging, more than the %d a block has",
                     mc.n_meas, smem, smem_max);
     const bool l1 = o->loss == GAC_FIT_L1;
-    const void *fn = l1 ? step_ptr<PREC, true>(mc.kind) : step_ptr<PREC, false>(mc.kind);
+    // the total-variation term couples voxels, and an update is then one launch
+    const bool coupled = o->tv_params != 0 && static_cast<R>(o->tv_lambda / static_cast<double>(n_mask)) != R(0);
+    // A mask becomes a list of its voxels where that saves the persistent warps a
+    // round of tiles (below, with 20 warps an SM in FP32); a warp's only tile
+    // would just wait for the list (3-pool, 13,653 voxels, 63% inside: 9.7 ->
+    // 10.2 us an update; 552,960 voxels, 68%: 61 -> 50).
+    const int64_t warps = static_cast<int64_t>(sms) * kFitMinBlocks32 * kFitWarps;
+    auto rounds = [&](int64_t n) { return ((n + 31) / 32 + warps - 1) / warps; };
+    const bool use_list = d_mask && n_mask < N && (!coupled || rounds(n_mask) < rounds(N));
+    const int64_t n_list = use_list ? n_mask : N;
+    const void *fn = step_ptr<PREC>(mc.kind, l1, use_list);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     int per_sm = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kFitBlock, smem);
     if (e != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
     // persistent warps, each given the same number of 32-voxel tiles (+-1)
-    const int64_t tiles = (N + 31) / 32;
+    PoolBuf list(s);
+    if (use_list && (e = list_masked(d_mask, static_cast<int>(N), n_mask, &list, s)) != cudaSuccess)
+        return cuda_fail(e, "fitted voxels");
+    const int64_t tiles = (n_list + 31) / 32;
     const int64_t slots = static_cast<int64_t>(sms) * std::max(per_sm, 1) * kFitWarps;
     const int64_t per_warp = (tiles + slots - 1) / slots;
     const int grid = static_cast<int>((tiles + per_warp * kFitWarps - 1) / (per_warp * kFitWarps));
     // work arrays: u (two buffers), Adam moments, block losses, history, flags
     const int I = o->iterations;
-    const size_t bytes_u = static_cast<size_t>(N) * P * RB;
-    // the total-variation term couples voxels, and an update is then one launch
-    const bool coupled = o->tv_params != 0 && static_cast<R>(o->tv_lambda / static_cast<double>(n_mask)) != R(0);
-    const size_t total = 4 * bytes_u + std::max(grid, kFitLossBlocks * kFitChunk) * sizeof(double) + static_cast<size_t>(std::max(I, 1)) * sizeof(double) + 3 * sizeof(int);
+    const size_t bytes_u = (static_cast<size_t>(n_list) * P * RB + 15) / 16 * 16;
+    // the penalised maps over the grid, two buffers, when there is a list
+    const size_t tv_n = use_list && coupled ? static_cast<size_t>(__builtin_popcount(o->tv_params & ((1u << P) - 1u))) * N : 0;
+    const size_t bytes_tv = (tv_n * RB + 15) / 16 * 16;
+    const size_t total = 4 * bytes_u + 2 * bytes_tv + std::max(grid, kFitLossBlocks * kFitChunk) * sizeof(double) +
+                         static_cast<size_t>(std::max(I, 1)) * sizeof(double) + 3 * sizeof(int);
     void *base = nullptr;
     e = cudaMallocAsync(&base, total, s);
     if (e != cudaSuccess) return cuda_fail(e, "fit work arrays");
@@ -1168,24 +1299,25 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
         ~Free() { cudaFreeAsync(p, s); }
     } guard{base, s};
     char *b = static_cast<char *>(base);
-    void *u0 = b, *u1 = b + bytes_u, *m1 = b + 2 * bytes_u, *m2 = b + 3 * bytes_u;
-    double *block_loss = reinterpret_cast<double *>(b + 4 * bytes_u);
+    R *const u0 = reinterpret_cast<R *>(b), *const u1 = reinterpret_cast<R *>(b + bytes_u);
+    R *const m1 = reinterpret_cast<R *>(b + 2 * bytes_u), *const m2 = reinterpret_cast<R *>(b + 3 * bytes_u);
+    R *const tv0 = reinterpret_cast<R *>(b + 4 * bytes_u), *const tv1 = reinterpret_cast<R *>(b + 4 * bytes_u + bytes_tv);
+    double *block_loss = reinterpret_cast<double *>(b + 4 * bytes_u + 2 * bytes_tv);
     double *hist = block_loss + std::max(grid, kFitLossBlocks * kFitChunk);
     int *flags = reinterpret_cast<int *>(hist + std::max(I, 1));  // stop, done, arrival count
     if ((e = cudaMemsetAsync(flags, 0, 3 * sizeof(int), s)) != cudaSuccess) return cuda_fail(e, "fit memset");
-    const int conv_grid = static_cast<int>(std::min<int64_t>((N * P + 255) / 256, static_cast<int64_t>(sms) * 8));
-    theta_to_u_kernel<R><<<conv_grid, 256, 0, s>>>(mc, static_cast<const double *>(d_theta.ptr), N, static_cast<R *>(u0));
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "theta to u");
     FitArgs<R> fa;
     std::memset(&fa, 0, sizeof fa);
     fa.data = d_data;
     fa.mask = d_mask;
+    fa.list = static_cast<const int *>(list.p);
+    fa.n_list = static_cast<int>(n_list);
     fa.weight = d_weight;
     fa.nx = o->nx;
     fa.ny = o->ny;
     fa.nz = o->nz;
     fa.n = N;
-    fa.tv_params = o->tv_params;
+    fa.tv_params = coupled ? o->tv_params : 0;
     fa.tv_dims = o->tv_dims;
     fa.scale = static_cast<R>(1.0 / (static_cast<double>(n_mask) * mc.n_meas));
     fa.lambda_n = static_cast<R>(o->tv_lambda / static_cast<double>(n_mask));
@@ -1207,11 +1339,14 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     fa.fdiv = N < (int64_t(1) << 24);
     fa.inv_nx = 1.0f / static_cast<float>(o->nx);
     fa.inv_ny = 1.0f / static_cast<float>(o->ny);
+    fa.tv_out = tv_n ? tv0 : nullptr;  // filled with the first update's neighbours
+    const int conv_grid = static_cast<int>(std::min<int64_t>((n_list * P + 255) / 256, static_cast<int64_t>(sms) * 8));
+    theta_to_u_kernel<R><<<conv_grid, 256, 0, s>>>(mc, fa, static_cast<const double *>(d_theta.ptr), u0);
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "theta to u");
     int done = 0;
     bool stepwise = coupled;  // a launch per update
     if (!coupled) {
-        st = fit_uncoupled<PREC>(mc, o, fa, static_cast<int>(n_mask), static_cast<R *>(u0), static_cast<R *>(m1),
-                                 static_cast<R *>(m2), bytes_u, &done, s);
+        st = fit_uncoupled<PREC>(mc, o, fa, u0, m1, m2, bytes_u, &done, s);
         if (st == GAC_ERR_OOM) {  // no memory for its loss shares: the other path needs none
             clear_error();
             stepwise = true;
@@ -1229,9 +1364,10 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
             for (; t <= t_end; ++t) {
                 double c1, c2;
                 bias_corrections<PREC>(o, t, &c1, &c2);
-                const void *ui = (t & 1) ? u0 : u1;
-                void *uo = (t & 1) ? u1 : u0;
-                if ((e = launch_step_kind<PREC>(mc.kind, l1, grid, smem, s, mc, fa, ui, uo, m1, m2, c1, c2, t)) != cudaSuccess)
+                const bool odd = t & 1;
+                fa.tv_in = tv_n ? (odd ? tv0 : tv1) : nullptr;
+                fa.tv_out = tv_n ? (odd ? tv1 : tv0) : nullptr;
+                if ((e = launch_step<R>(fn, grid, smem, s, mc, fa, odd ? u0 : u1, odd ? u1 : u0, m1, m2, R(c1), R(c2), t)) != cudaSuccess)
                     return cuda_fail(e, "fit step");
             }
             int stop = 0;
@@ -1250,9 +1386,7 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
             return cuda_fail(e, "loss history");
     }
     // u of the last update (stepwise, iteration `done` wrote buffer (done & 1) ? u1 : u0) -> theta
-    const void *u_fin = stepwise && (done & 1) ? u1 : u0;
-    u_to_theta_kernel<R><<<conv_grid, 256, 0, s>>>(mc, static_cast<const R *>(u_fin), d_mask, N,
-                                                   static_cast<double *>(d_theta.ptr));
+    u_to_theta_kernel<R><<<conv_grid, 256, 0, s>>>(mc, fa, stepwise && (done & 1) ? u1 : u0, static_cast<double *>(d_theta.ptr));
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "u to theta");
     if ((st = d_theta.copy_out()) != GAC_OK) return st;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "fit");
