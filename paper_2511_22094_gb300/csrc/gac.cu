@@ -661,11 +661,13 @@ static gac_status plan_spec(const ModelConst &mc, int depth, int C, int64_t n_vo
     const void *fn = mh_spec_ptr(mc.kind, depth, all);
     if (!fn) return fail(GAC_ERR_INVALID_ARG, "no speculative kernel for kind %d of depth %d", mc.kind, depth);
     const SpecShape sh = spec_shape(depth, C, n_vox);
-    const size_t smem = spec_smem_bytes(mc.n_par, 1 << depth, sh.threads, sh.vb, row_stride_for(mc.kind, mc.n_meas), all);
+    const bool help = spec_moment_warps(depth, all);
+    const size_t smem = spec_smem_bytes(mc.n_par, 1 << depth, sh.threads, sh.vb, row_stride_for(mc.kind, mc.n_meas), all, help);
+    const int block = sh.threads + (help ? 32 * moment_warps(mc.n_par * (sh.threads >> depth), kMomMaxWarps) : 0);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     int per_sm = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, sh.threads, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block, smem);
     if (e != cudaSuccess) return cuda_fail(e, "speculative kernel occupancy");
     if (per_sm < 1) return fail(GAC_ERR_INVALID_ARG, "speculative kernel does not fit on an SM (smem %zu)", smem);
     *vb = sh.vb;
@@ -673,7 +675,8 @@ static gac_status plan_spec(const ModelConst &mc, int depth, int C, int64_t n_vo
     cfg->grid = static_cast<int>(std::min<int64_t>(sh.n_tiles, static_cast<int64_t>(per_sm) * sm_count()));
     cfg->fn = fn;
     cfg->smem = smem;
-    cfg->block = sh.threads;
+    cfg->block = block;
+    cfg->sampling = sh.threads;
     return GAC_OK;
 }
 
@@ -903,7 +906,7 @@ gac_status gac_mcmc_run(int model_id, const void *data, int64_t n_vox, const flo
     if ((st = d_scale.make(out->step_scale, C * N * sizeof(float), false, s, "step_scale")) != GAC_OK) return st;
 
     const bool trace = o->trace_n_vox > 0;
-    LaunchCfg cfg;
+    LaunchCfg cfg{};
     int64_t n_tiles = 0;
     int vb = 0;
     const int depth = choose_depth(mc, o, n_vox, lanes > 1);
@@ -939,6 +942,7 @@ gac_status gac_mcmc_run(int model_id, const void *data, int64_t n_vox, const flo
     ra.row_stride = row_stride_for(mc.kind, M);
     ra.data_vec4 = (M % 4 == 0) && ((reinterpret_cast<uintptr_t>(ra.data) & 15) == 0);
     ra.n_tiles = n_tiles;
+    ra.sampling_threads = cfg.sampling;
     set_adaptation(ra, o);
     ra.rhat = static_cast<double *>(d_rhat.ptr);
     ra.step_scale = static_cast<float *>(d_scale.ptr);

@@ -12,7 +12,8 @@ namespace gac {
 struct LaunchCfg {
     const void *fn;
     int grid;
-    int block;  // threads per block
+    int block;     // threads per block
+    int sampling;  // of them, those before the moment warps (speculative kernel)
     size_t smem;
 };
 

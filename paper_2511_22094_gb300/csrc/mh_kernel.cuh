@@ -93,6 +93,7 @@ struct RunArgs {
     int adapt_window, adapt_lo, adapt_hi;
     double *rhat;        // [P][N] or nullptr
     float *step_scale;   // [C][N] or nullptr
+    int sampling_threads;  // speculative kernel: threads of the block before its moment warps
 };
 
 // Chain state kept in HBM between slices, structure of arrays over the

@@ -19,8 +19,10 @@
 //    Box-Muller pairs; the nodes fetch the normals by shuffle.
 //  - Rounds end at the burn-in adaptation's windows (and at the last
 //    iteration), so all chains stay at the same t.
-//  - Lane g keeps the FP64 Welford accumulators (and the MIXED block
-//    partials) of parameters g, g + G, ... and stores those samples.
+//  - Lane g stores the samples of parameters g, g + G, ... and keeps their
+//    MIXED block partials.  The FP64 Welford updates run on moment warps
+//    (moment_warps.cuh); at depth 2, whose warps fill the schedulers, lane g
+//    keeps those too.
 //
 // What bounds it: a lone warp per scheduler issues its instructions in turn
 // and waits out every latency (ncu, AxCaliberSMT at depth 5: 1,295 instructions
@@ -36,6 +38,7 @@
 // precision, one launch per job, no trace.
 #pragma once
 #include "mh_split.cuh"
+#include "moment_warps.cuh"
 
 namespace gac {
 
@@ -44,11 +47,14 @@ constexpr int kSpecBlock = 256;
 
 // Shared-memory bytes of a block of `threads` threads: the Welford
 // accumulators, the measurement tile, and for moments over every post-burn-in
-// state the block partials and the rows the states are exchanged through.
+// state the block partials and the rows the states are exchanged through
+// (`threads`: the sampling threads), or the moment warps' ring.
 __host__ __device__ constexpr int spec_row(int P) { return P | 1; }  // odd: a warp's rows start in distinct banks
-__host__ __device__ inline size_t spec_smem_bytes(int P, int G, int threads, int VB, int row_stride, bool all) {
+__host__ __device__ constexpr bool spec_moment_warps(int depth, bool all) { return depth >= 3 && !all; }
+__host__ __device__ inline size_t spec_smem_bytes(int P, int G, int threads, int VB, int row_stride, bool all, bool ring) {
     return tile_smem_bytes(P, sizeof(double), VB, row_stride, true, all, threads / G) +
-           (all ? static_cast<size_t>(threads) * spec_row(P) * sizeof(float) : 0);
+           (all ? static_cast<size_t>(threads) * spec_row(P) * sizeof(float) : 0) +
+           (ring ? moment_ring_bytes(P * (threads / G)) : 0);
 }
 
 // The draws of one round: lane g holds items g, g + G, ... (Philox call i %
@@ -90,8 +96,10 @@ __device__ __forceinline__ void run_tile_spec(const ModelConst &mc, const RunArg
     constexpr int G = 1 << D;
     constexpr uint32_t kGroup = G == 32 ? 0xffffffffu : (1u << G) - 1u;
     using Draw = SpecDraw<P, D>;
+    constexpr bool kHelp = spec_moment_warps(D, ALL);
     const int nthr = blockDim.x;
-    const int CB = nthr / G;  // chain slots of the block
+    const int nsamp = kHelp ? ra.sampling_threads : nthr;
+    const int CB = nsamp / G;  // chain slots of the block
     const int tid = threadIdx.x;
     const int C = ra.C;
     const int VB = ra.vox_per_block;
@@ -102,12 +110,14 @@ __device__ __forceinline__ void run_tile_spec(const ModelConst &mc, const RunArg
     const int64_t v0 = tile * VB;
     const int64_t left = ra.n_vox - v0;
     const int nv = left < VB ? static_cast<int>(left) : VB;
-    const bool active = slot < VB * C && lv < nv;
+    const bool active = tid < nsamp && slot < VB * C && lv < nv;
     double *wf_mean = reinterpret_cast<double *>(smem);
     double *wf_m2 = wf_mean + P * CB;
     float *ytile = reinterpret_cast<float *>(wf_m2 + P * CB);
     float *bs = ytile + VB * ra.row_stride;  // ALL: FP32 block partials s1 [P][CB], s2, reference
     float *exch = bs + 3 * P * CB;           // ALL: the nodes' proposals [thread][spec_row(P)]
+    // the moment warps' ring: the sampling warps with a chain are the first ones
+    const MomentRing mom{bs, P * CB, ra.S, (nv * C * G + 31) / 32 * 32 + nthr - nsamp};
 
     // a1: stage measurements of voxels [v0, v0 + nv) (and the model's table)
     __syncthreads();
@@ -151,7 +161,10 @@ __device__ __forceinline__ void run_tile_spec(const ModelConst &mc, const RunArg
     auto path_bit = [&](int k) { return k < lvl && ((node >> (lvl - 1 - k)) & 1); };
 
     int n_acc = 0, n_bad = 0, ad_e = 0;
-    if (__any_sync(kFullMask, active)) {
+    if (kHelp && tid >= nsamp) {
+        constexpr int kSeries = P * (kSpecBlock / G);  // at most
+        moment_warp_run<(kSeries + 32 * kMomMaxWarps - 1) / (32 * kMomMaxWarps)>(mom, tid - nsamp, nthr - nsamp, wf_mean, wf_m2);
+    } else if (__any_sync(kFullMask, active)) {
         // a2: initial state
         float th[P];
         if (ra.x0) {
@@ -165,7 +178,7 @@ __device__ __forceinline__ void run_tile_spec(const ModelConst &mc, const RunArg
             for (int p = 0; p < P; ++p) th[p] = fmaf(mc.ub_f[p] - mc.lb_f[p], u01_f(w0[p]), mc.lb_f[p]);
         }
         float L = loglik_f<KIND, KahanSum>(th, y, inv_s2, mc);
-        if (active) {
+        if (!kHelp && active) {
 #pragma unroll
             for (int p = 0; p < P; ++p)
                 if (p % G == g) {
@@ -174,7 +187,7 @@ __device__ __forceinline__ void run_tile_spec(const ModelConst &mc, const RunArg
                 }
         }
         int ad_acc0 = 0, n_mom = 0, blk_n = 0;
-        // thinned moments: lane g's parameters p = g + kG in registers, each
+        // thinned moments without moment warps: lane g's parameters p = g + kG in registers, each
         // update's second half deferred to the next event (as in the
         // lane-split kernel: two short FP64 chains instead of one long one)
         constexpr int PL = (P + G - 1) / G;
@@ -282,7 +295,15 @@ __device__ __forceinline__ void run_tile_spec(const ModelConst &mc, const RunArg
                         for (int k = 0; k < PL; ++k)
                             if (g + k * G < P) dst[(g + k * G) * ra.n_vox] = x[k];
                     }
-                    if constexpr (!ALL) {
+                    if constexpr (kHelp) {
+                        __syncwarp();
+                        mom.open(n_thin);
+                        float *ev = mom.at(n_thin);
+#pragma unroll
+                        for (int k = 0; k < PL; ++k)
+                            if (g + k * G < P) ev[(g + k * G) * CB + slot] = x[k];
+                        mom.close(n_thin);
+                    } else if constexpr (!ALL) {
                         ++n_mom;
                         const double inv_n = inv_count<double, true>(n_mom);
                         if (g < P) {
@@ -365,7 +386,7 @@ __device__ __forceinline__ void run_tile_spec(const ModelConst &mc, const RunArg
             }
             next_round(t0);
         }
-        if constexpr (!ALL) {
+        if constexpr (!ALL && !kHelp) {
             if (active && g < P) {
 #pragma unroll
                 for (int k = 0; k < PL; ++k)
@@ -399,7 +420,7 @@ __device__ __forceinline__ void run_tile_spec(const ModelConst &mc, const RunArg
 }
 
 template <int KIND, int D, bool ALL>
-__global__ void __launch_bounds__(kSpecBlock, 2) mh_spec_kernel(const ModelConst mc, const RunArgs ra) {
+__global__ void __launch_bounds__(kSpecBlock + (spec_moment_warps(D, ALL) ? 32 * kMomMaxWarps : 0), D == 2 ? 2 : 1) mh_spec_kernel(const ModelConst mc, const RunArgs ra) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     for (int64_t tile = blockIdx.x; tile < ra.n_tiles; tile += gridDim.x)
         run_tile_spec<KIND, D, ALL>(mc, ra, tile, smem_raw);
