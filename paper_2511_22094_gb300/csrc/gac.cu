@@ -509,6 +509,94 @@ static gac_status plan_launch(const ModelConst &mc, int prec, bool trace, int C,
     return GAC_OK;
 }
 
+// A run in slices (mh_slice_kernel).
+struct SlicePlan {
+    const void *fn = nullptr;  // nullptr: one launch
+    size_t smem = 0;
+    int slots = 0;  // resident blocks
+    int q = 0;      // iterations of a slice
+    int count = 0;  // slices of a tile
+    int vb = 0;
+    int64_t n_tiles = 0;
+};
+
+// Slices for a problem whose last wave of tiles would leave the GPU partly idle:
+// the tiles take turns, so that all launches but the last are full.  n_tiles
+// tiles in `count` slices take ceil(count n_tiles / slots) launches.  Chosen where
+// that is estimated 3% shorter than one launch: whole waves and, for a last one
+// that fills the fullest SM to a share f, 0.2 + f / 2 (an AxCaliberSMT wave and
+// 0.29 measured 1.45 waves), with 2% for the launches' ends.  Only for the two
+// models whose kernels hold 2 blocks an SM, where a wave is longest; thinning of
+// at least 16, as the moments live in HBM between slices, and for the 3-pool
+// model not over every state (its partial sums cost more to keep than the last
+// wave).  us per iteration, one launch -> slices: AxCaliberSMT, 80,000 chains
+// 4.21 -> 3.40, 100,004 4.73 -> 4.16, 140,000 6.19 -> 5.66; 3-pool, 80,000 3.56 ->
+// 3.21, 93,000 4.18 -> 3.58, 140,000 5.65 -> 5.34; past three waves nothing.
+static gac_status plan_slices(const ModelConst &mc, const gac_mcmc_opts *o, int64_t n_vox, const LaunchCfg &one,
+                              int64_t one_tiles, SlicePlan *sp) {
+    const int C = o->n_chains;
+    const bool all = o->moments_mode == GAC_MOMENTS_ALL_POSTBURNIN;
+    const void *fn = mc.kind == GAC_MODEL_AXCAL_SMT     ? mh_slice_ptr_axcal()
+                     : mc.kind == GAC_MODEL_MWI3 && !all ? mh_slice_ptr_mwi3()
+                                                         : nullptr;
+    if (!fn || o->precision != GAC_PREC_MIXED || o->trace_n_vox != 0 || o->lanes_per_chain != 0 || o->iterations < 256 ||
+        (!all && o->thin < 16))
+        return GAC_OK;
+    SlicePlan p;
+    p.vb = std::max(1, kBlock / C);
+    p.n_tiles = (n_vox + p.vb - 1) / p.vb;
+    if (one_tiles <= one.grid) return GAC_OK;  // a single wave
+    p.smem = tile_smem_bytes(mc.n_par, sizeof(double), p.vb, row_stride_for(mc.kind, mc.n_meas), false, all);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(p.smem));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    int per_sm = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, p.smem);
+    if (e != cudaSuccess) return cuda_fail(e, "slice kernel occupancy");
+    p.slots = per_sm * sm_count();
+    if (p.slots < 1 || p.n_tiles <= p.slots) return GAC_OK;
+    const int64_t rest = one_tiles % one.grid;
+    const double f = static_cast<double>((rest + sm_count() - 1) / sm_count() * sm_count()) / one.grid;
+    // in waves of `slots` full blocks
+    const double plain = (static_cast<double>(one_tiles / one.grid) + (rest == 0 ? 0.0 : f >= 1.0 ? 1.0 : 0.2 + 0.5 * f)) *
+                         one.grid * one.block / (static_cast<double>(p.slots) * kBlock);
+    double best = 0.97 * plain;
+    for (int m = 2; m <= 24 && o->iterations / m >= 64; ++m) {
+        const double t = 1.02 * static_cast<double>((m * p.n_tiles + p.slots - 1) / p.slots) / m;
+        if (t < best) {
+            best = t;
+            p.q = (o->iterations + m - 1) / m;
+        }
+    }
+    if (p.q == 0) return GAC_OK;
+    p.count = (o->iterations + p.q - 1) / p.q;
+    p.fn = fn;
+    *sp = p;
+    return GAC_OK;
+}
+
+// Device memory of the chains' state between slices (struct SliceState), carved
+// from one allocation: its bytes, and the pointers when `base` is given.
+static size_t slice_state(const ModelConst &mc, int64_t chains, bool all, char *base, SliceState *ss) {
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = off;
+        off += (bytes + 255) & ~static_cast<size_t>(255);
+        return base ? base + at : nullptr;
+    };
+    const size_t P = mc.n_par, n = static_cast<size_t>(chains);
+    SliceState s{};
+    s.theta = take(P * n * 4);
+    s.L = take(n * 4);
+    s.n_acc = reinterpret_cast<int32_t *>(take(n * 4));
+    s.n_bad = reinterpret_cast<int32_t *>(take(n * 4));
+    s.wf_mean = take(P * n * 8);
+    s.wf_m2 = take(P * n * 8);
+    s.adapt = reinterpret_cast<int32_t *>(take(2 * n * 4));
+    s.blk = all ? reinterpret_cast<float *>(take(3 * P * n * 4)) : nullptr;
+    if (ss) *ss = s;
+    return off;
+}
+
 gac_status validate_opts(const gac_mcmc_opts *o, int64_t n_vox) {
     if (!o) return fail(GAC_ERR_INVALID_ARG, "opts is NULL");
     if (o->iterations < 0 || o->iterations == INT32_MAX)
@@ -914,6 +1002,27 @@ gac_status gac_mcmc_run(int model_id, const void *data, int64_t n_vox, const flo
        : lanes > 1 ? plan_split(mc, lanes, C, n_vox, o->moments_mode, &cfg, &n_tiles, &vb)
                    : plan_launch(mc, o->precision, trace, C, n_vox, o->moments_mode, &cfg, &n_tiles, &vb);
     if (st != GAC_OK) return st;
+    // slices read the data once each: not over the link from host memory
+    SlicePlan sp;
+    if (depth == 0 && lanes == 1 && is_device_ptr(d_data.ptr) &&
+        (st = plan_slices(mc, o, n_vox, cfg, n_tiles, &sp)) != GAC_OK)
+        return st;
+    const bool all = o->moments_mode == GAC_MOMENTS_ALL_POSTBURNIN;
+    SliceState ss{};
+    DevBuf d_state;  // freed in stream order
+    if (sp.fn) {
+        d_state.stream = s;
+        if (cudaMallocAsync(&d_state.ptr, slice_state(mc, n_vox * C, all, nullptr, nullptr), s) == cudaSuccess) {
+            d_state.owned = true;
+            slice_state(mc, n_vox * C, all, static_cast<char *>(d_state.ptr), &ss);
+            n_tiles = sp.n_tiles;
+            vb = sp.vb;
+        } else {  // no memory for the state: one launch
+            cudaGetLastError();
+            d_state.ptr = nullptr;
+            sp.fn = nullptr;
+        }
+    }
 
     RunArgs ra;
     std::memset(&ra, 0, sizeof ra);
@@ -947,8 +1056,17 @@ gac_status gac_mcmc_run(int model_id, const void *data, int64_t n_vox, const flo
     ra.rhat = static_cast<double *>(d_rhat.ptr);
     ra.step_scale = static_cast<float *>(d_scale.ptr);
 
-    void *args[] = {&mc, &ra};
-    cudaError_t e = cudaLaunchKernel(cfg.fn, dim3(cfg.grid), dim3(cfg.block), args, cfg.smem, s);
+    cudaError_t e = cudaSuccess;
+    if (sp.fn) {
+        const int64_t end = sp.count * sp.n_tiles;
+        for (int64_t pos = 0; pos < end && e == cudaSuccess; pos += sp.slots) {
+            void *args[] = {&mc, &ra, &ss, &pos, &sp.q};
+            e = cudaLaunchKernel(sp.fn, dim3(static_cast<unsigned>(std::min<int64_t>(sp.slots, end - pos))), dim3(kBlock), args, sp.smem, s);
+        }
+    } else {
+        void *args[] = {&mc, &ra};
+        e = cudaLaunchKernel(cfg.fn, dim3(cfg.grid), dim3(cfg.block), args, cfg.smem, s);
+    }
     if (e != cudaSuccess) return cuda_fail(e, "MH kernel launch");
     for (DevBuf *b : {&d_mean, &d_std, &d_samples, &d_acc, &d_bad, &d_trace, &d_rhat, &d_scale})
         if ((st = b->copy_out()) != GAC_OK) return st;

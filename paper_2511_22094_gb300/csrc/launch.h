@@ -23,6 +23,9 @@ const void *mh_ptr_mwi3(int prec, bool trace, int block);
 const void *mh_ptr_smt(int prec, bool trace, int block);
 const void *mh_ptr_axcal(int prec, bool trace, int block);
 const void *mh_ptr_linear(int prec, bool trace, int block);
+// In slices (mh_slice_kernel: further arguments ss, pos0, q), MIXED.
+const void *mh_slice_ptr_mwi3();
+const void *mh_slice_ptr_axcal();
 // Lane-split kernels (mh_split.cuh): G = 2 or 4 lanes per chain, MIXED; all:
 // moments over every post-burn-in state.
 const void *mh_split_ptr_monoexp(int G, bool all);

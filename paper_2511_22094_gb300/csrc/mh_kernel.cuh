@@ -599,6 +599,20 @@ __global__ void __launch_bounds__(BLK, mh_min_blocks<KIND, PREC>() * (kBlock / B
         run_tile<KIND, PREC, TRACE, false, BLK>(mc, ra, none, tile, 0, ra.I, smem_raw);
 }
 
+// One job in slices of q iterations, for problems of a few waves of tiles: tile k
+// of slice s stands at position s n_tiles + k, and a launch takes the positions
+// from pos0 on, one a block and at most n_tiles of them, so that a tile's slices
+// come in order in different launches and every launch but the last fills the
+// GPU (plan_slices in gac.cu).
+template <int KIND>
+__global__ void __launch_bounds__(kBlock, mh_min_blocks<KIND, GAC_PREC_MIXED>())
+    mh_slice_kernel(const ModelConst mc, const RunArgs ra, const SliceState ss, const int64_t pos0, const int q) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int64_t pos = pos0 + blockIdx.x;
+    const int s = static_cast<int>(pos / ra.n_tiles);
+    run_tile<KIND, GAC_PREC_MIXED, false, true>(mc, ra, ss, pos - s * ra.n_tiles, s * q, min(ra.I, (s + 1) * q), smem_raw);
+}
+
 // The kernel of a kind for (precision, trace, threads per block), or nullptr.
 template <int KIND>
 const void *mh_kernel_ptr_of(int prec, bool trace, int block) {
