@@ -718,15 +718,19 @@ static SpecShape spec_shape(int depth, int C, int64_t n_vox) {
 //             spec   0.40   0.49   0.62   0.77   1.10   1.41    1.68
 //             depth  5      4      3      3      2      2       2
 //   mono-exp  split  0.19   0.20   0.20   0.20   0.19   0.26    0.26
-//             spec   0.14   0.17   -      -      -      -       -
+//             spec   0.14   0.17   0.19   -      -      -       -
+//             depth  5      4      4
 // A round of the trees of depth 3 and more takes as long with a second warp on
 // its scheduler only where it waits on table lookups (SMT, AxCaliberSMT); the
 // 3-pool round issues paired multiply-adds for most of its cycles.  Depth 2
 // doubles the work per iteration and halves the serial path: it pays up to
 // four warps a scheduler for AxCaliberSMT, three for SMT and two for the 3-pool
-// model, the least latency-bound of the three.  The mono-exponential round is short enough that the lane-split
-// kernel's shorter path wins where it applies (`split`) once two warps share
-// a scheduler.
+// model, the least latency-bound of the three.  The mono-exponential round is
+// short enough that the lane-split kernel's shorter path wins where it applies
+// (`split`) past two warps a scheduler at depth 4; with thinning of 4 or less,
+// where that kernel's own moment updates weigh, past two at depth 3 (2,000
+// iterations of 4,096 chains, thinning 2: 0.76 ms split, 0.62; thinning 5: 0.51
+// both).
 static int choose_depth(const ModelConst &mc, const gac_mcmc_opts *o, int64_t n_vox, bool split) {
     if (o->precision != GAC_PREC_MIXED || o->trace_n_vox != 0 || o->lanes_per_chain != 0 ||
         !mh_spec_ptr(mc.kind, 2, false))
@@ -734,10 +738,16 @@ static int choose_depth(const ModelConst &mc, const gac_mcmc_opts *o, int64_t n_
     const int C = o->n_chains;
     const int64_t schedulers = static_cast<int64_t>(sm_count()) * 4;
     const bool mwi3 = mc.kind == GAC_MODEL_MWI3, mono = mc.kind == GAC_MODEL_MONOEXP;
+    const bool all = o->moments_mode == GAC_MOMENTS_ALL_POSTBURNIN;
     for (int depth = 5; depth >= 2; --depth) {
         if (C << depth > kSpecBlock || n_vox * C > (schedulers * 32 * 4 >> depth)) continue;
-        const int per = depth >= 4 ? 1 : depth == 3 ? (mwi3 || mono ? 1 : 2) : mwi3 ? 2 : mc.kind == GAC_MODEL_SMT ? 3 : 4;
-        if (depth < 4 && mono && split) return 0;
+        // warps a scheduler
+        const int per = depth == 5   ? 1
+                        : depth == 4 ? (mono && !all ? 2 : 1)
+                        : depth == 3 ? (mwi3 ? 1 : 2)
+                        : mwi3       ? 2
+                        : mc.kind == GAC_MODEL_SMT ? 3 : 4;
+        if (mono && split && (depth == 2 || (depth == 3 && (all || o->thin > 4)))) return 0;
         if (spec_shape(depth, C, n_vox).warps() <= per * schedulers) return depth;
     }
     return 0;

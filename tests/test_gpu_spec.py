@@ -77,3 +77,16 @@ def test_no_iterations_and_no_samples(gac, orc):
             if one[k] is not None:
                 np.testing.assert_array_equal(spec[k], one[k], err_msg=k)
         assert np.isnan(spec["mean"]).all()
+
+
+@pytest.mark.parametrize("n,thin", [(2400, 3), (4800, 1), (4800, 4), (4096, 5)])
+def test_monoexp_depth_follows_the_thinning(gac, orc, n, thin):
+    """Two warps a scheduler at depth 4, and at depth 3 where thinning is short; the lane-split
+    kernel otherwise: the same bits as one thread per chain."""
+    w = W.MONOEXP_4K
+    mid = gac.gac_model_register(w.kind, w.acq, w.lb, w.ub, w.step)
+    th, sig, y = make_voxels(orc, w.with_(n_vox=n), 0, n)
+    run = lambda lanes: gac.run_host(mid, y, sig, iterations=120, burnin=17, thin=thin, n_chains=1, seed=6, lanes_per_chain=lanes)
+    one, auto = run(1), run(0)
+    for k in KEYS:
+        np.testing.assert_array_equal(auto[k], one[k], err_msg=k)
