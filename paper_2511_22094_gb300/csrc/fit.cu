@@ -66,6 +66,10 @@ struct FitArgs {
     // and each update's new values written to tv_out.
     const R *tv_in;
     R *tv_out;
+    // The kernels over a list and those of many updates leave each voxel's share
+    // of an update's loss here ([updates][N], 0 outside the list) for
+    // fit_losses_kernel.
+    R *vloss;
 };
 
 // sign(x) with sign(0) = 0, branch-free (a select and a sign-bit copy)
@@ -672,7 +676,7 @@ __global__ void __launch_bounds__(kFitBlock, fit_min_blocks(PREC)) fit_step_kern
 // The same over the list of fitted voxels of a masked grid: parameters and
 // moments lie in the list's order, so that their accesses stay whole lines, and
 // the penalised maps once more over the grid, where the neighbours read them.
-// Tiles hold fitted voxels only: 552,960 voxels, 68% inside, 3-pool, 61 -> 50 us
+// Tiles hold fitted voxels only: 552,960 voxels, 68% inside, 3-pool, 61 -> 49.5 us
 // an update.
 template <int KIND, int PREC, bool L1>
 __global__ void __launch_bounds__(kFitBlock, fit_min_blocks(PREC)) fit_list_kernel(const ModelConst mc, const FitArgs<typename PrecTraits<PREC>::R> fa,
@@ -719,7 +723,6 @@ __global__ void __launch_bounds__(kFitBlock, fit_min_blocks(PREC)) fit_list_kern
             w_n = fa.weight ? R(fa.weight[v]) : R(1);
         }
     };
-    R my_loss = R(0);
     const int stride = gridDim.x * kFitWarps;
     int tile = blockIdx.x * kFitWarps + warp;
     // the lane's voxel and its next one (read a tile ahead)
@@ -753,7 +756,7 @@ __global__ void __launch_bounds__(kFitBlock, fit_min_blocks(PREC)) fit_list_kern
         cp_async_commit();
         load_next(next * 32 + lane, v_next);
         const int v_after = voxel((next + stride) * 32 + lane);
-        if (active) my_loss += fit_phase_b<KIND, PREC, true>(mc, fa, e, v, u, true, tv, loss, g, mo_s + lane, u_in, u_out, m1, m2, c1, c2);
+        if (active) fa.vloss[v] = fit_phase_b<KIND, PREC, true>(mc, fa, e, v, u, true, tv, loss, g, mo_s + lane, u_in, u_out, m1, m2, c1, c2);
         __syncwarp();  // phase B has read every moment
         if (next < n_tiles) stage_moments(next);
         cp_async_commit();
@@ -761,7 +764,6 @@ __global__ void __launch_bounds__(kFitBlock, fit_min_blocks(PREC)) fit_list_kern
         v_next = v_after;
     }
     cp_async_wait<0>();
-    fit_block_loss(fa, my_loss, t_iter);
 }
 
 // The stopping rules after iteration t, whose loss is hist[t - 1]: loss < tol, or
@@ -814,12 +816,10 @@ __device__ void fit_check(const FA &fa, int n_blocks, int t, double *red) {
 // a voxel-update moves when every update is a launch.  Measured, whole calls on
 // a GB300, a launch per update -> this: mono-exponential, 37 x 41 x 9 voxels, 300
 // updates 1.70 -> 0.22 ms; 3-pool, 96 x 96 x 60, 100 updates 5.6 -> 3.3 ms, with
-// a mask of 68% of it 5.7 -> 2.4 ms.  The losses
-// of kFitFlush updates cross the warp through shared memory: two lanes add the 32
-// voxels' shares of one update, in FP32 with the rounding errors carried along
-// (TwoSum; FP64 adds hold the FP64 pipe for 76 cycles each).
-constexpr int kFitChunk = 128, kFitFlush = 16;
-constexpr int kFitLossBlocks = 128;  // blocks of fit_losses_kernel
+// a mask of 68% of it 5.7 -> 2.4 ms.
+constexpr int kFitChunk = 128;
+constexpr int kFitLossThreads = 256;  // >= kFitChunk
+constexpr int kFitLossBlocks = 32;  // blocks of fit_losses_kernel an update, at most
 
 template <class R>
 struct FitSteps {
@@ -831,24 +831,23 @@ __host__ __device__ constexpr bool fit_reg_moments() { return model_n_par(KIND) 
 
 template <int KIND, class R>
 __host__ __device__ constexpr size_t fit_many_smem(int row_stride) {
-    return 32 * static_cast<size_t>(row_stride) * sizeof(float) + kFitFlush * 33 * sizeof(R) +
+    return 32 * static_cast<size_t>(row_stride) * sizeof(float) +
            (fit_reg_moments<KIND>() ? 0 : 2 * static_cast<size_t>(model_n_par(KIND)) * 32 * sizeof(R));
 }
 
 // Updates t0 .. t0 + count - 1 (t0 = 1: from zero moments) of the fitted
-// voxels, u and the moments in place; part[tile][count]: the tile's share of each update's loss.
+// voxels, u and the moments in place.
 template <int KIND, int PREC, bool L1>
 __global__ void __launch_bounds__(32, PREC == GAC_PREC_FP32 ? 20 : 8)
     fit_many_kernel(const ModelConst mc, const FitArgs<typename PrecTraits<PREC>::R> fa,
                     typename PrecTraits<PREC>::R *u_io, typename PrecTraits<PREC>::R *m1, typename PrecTraits<PREC>::R *m2,
-                    const __grid_constant__ FitSteps<typename PrecTraits<PREC>::R> steps, int t0, int count, double *part) {
+                    const __grid_constant__ FitSteps<typename PrecTraits<PREC>::R> steps, int t0, int count) {
     using R = typename PrecTraits<PREC>::R;
     constexpr int P = model_n_par(KIND);
     constexpr bool kReg = fit_reg_moments<KIND>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *rows_s = reinterpret_cast<float *>(smem_raw);
-    R *loss_s = reinterpret_cast<R *>(smem_raw + 32 * static_cast<size_t>(fa.row_stride) * sizeof(float));
-    R *mo = loss_s + kFitFlush * 33 + threadIdx.x;
+    R *mo = reinterpret_cast<R *>(smem_raw + 32 * static_cast<size_t>(fa.row_stride) * sizeof(float)) + threadIdx.x;
     const int lane = threadIdx.x;
     const int M = mc.n_meas;
     const int n = fa.n_list;
@@ -878,13 +877,12 @@ __global__ void __launch_bounds__(32, PREC == GAC_PREC_FP32 ? 20 : 8)
     cp_async_wait<0>();
     __syncwarp();
     for (int k = 0; k < count; ++k) {
-        R share = R(0);
         if (active) {
             R loss = R(0), g[P];
 #pragma unroll
             for (int p = 0; p < P; ++p) g[p] = R(0);
             fit_loss_grad<KIND, PREC, L1>(mc, y, u, w, loss, g);
-            share = loss * fa.scale;
+            fa.vloss[k * fa.n + v] = loss * fa.scale;
             const R c1 = steps.c1[k], c2 = steps.c2[k];
 #pragma unroll
             for (int p = 0; p < P; ++p) {
@@ -900,24 +898,6 @@ __global__ void __launch_bounds__(32, PREC == GAC_PREC_FP32 ? 20 : 8)
                 }
             }
         }
-        loss_s[(k & (kFitFlush - 1)) * 33 + lane] = share;
-        if ((k & (kFitFlush - 1)) == kFitFlush - 1 || k == count - 1) {
-            __syncwarp();
-            const int j = lane & (kFitFlush - 1), kk = (k & ~(kFitFlush - 1)) + j;
-            const R *q = loss_s + j * 33 + (lane & ~(kFitFlush - 1));
-            R hi = R(0), lo = R(0);
-#pragma unroll
-            for (int i = 0; i < kFitFlush; ++i) {
-                const R x = q[i], t = hi + x, bb = t - hi;
-                lo += (hi - (t - bb)) + (x - bb);
-                hi = t;
-            }
-            double sum = static_cast<double>(hi);
-            if (isfinite(hi)) sum += static_cast<double>(lo);
-            sum += __shfl_xor_sync(0xffffffffu, sum, kFitFlush);
-            if (lane < kFitFlush && kk <= k) part[static_cast<int64_t>(blockIdx.x) * count + kk] = sum;
-            __syncwarp();
-        }
     }
     if (active) {
 #pragma unroll
@@ -929,32 +909,48 @@ __global__ void __launch_bounds__(32, PREC == GAC_PREC_FP32 ? 20 : 8)
     }
 }
 
-// Sums the tiles' shares of `count` losses (thread k takes update k of its
-// block's range of tiles; the last block to finish adds the ranges in order),
-// records them and applies the stopping rules to each update in turn.
-template <class FA>
-__global__ void __launch_bounds__(kFitChunk) fit_losses_kernel(const FA fa, const double *part, int tiles, int t0, int count) {
+// The losses of `count` updates from the voxels' shares (fa.vloss), summed as
+// fit_step_kernel's threads do it: voxels g, g + group, ... in the kernel's
+// precision, everything after that in FP64.  (An exact sum would differ from
+// theirs: 345,840 voxels, L2, by 9e-9 of the loss.)  blockIdx.y: the update.  The last
+// block to finish adds the blocks' shares in order, records the losses and
+// applies the stopping rules to each update in turn.  Bound by the reads, which
+// come from L2: about 0.5 us an update of 552,960 voxels.
+template <class R>
+__global__ void __launch_bounds__(kFitLossThreads) fit_losses_kernel(const FitArgs<R> fa, const R *vloss, int group, int t0, int count) {
+    __shared__ double red[kFitLossThreads / 32];
     __shared__ bool last;
-    const int k = threadIdx.x, nb = gridDim.x, b = blockIdx.x;
-    if (k < count) {
-        const int from = static_cast<int>(static_cast<int64_t>(tiles) * b / nb), to = static_cast<int>(static_cast<int64_t>(tiles) * (b + 1) / nb);
-        double s = 0.0;
-        for (int i = from; i < to; ++i) s += part[static_cast<int64_t>(i) * count + k];
-        fa.block_loss[b * kFitChunk + k] = s;
-        __threadfence();
+    if (*fa.stop) return;  // the same for every thread; only this kernel's last block sets it
+    const int nb = gridDim.x, tid = threadIdx.x;
+    const R *x = vloss + blockIdx.y * fa.n;
+    double sum = 0.0;
+    for (int g = blockIdx.x * kFitLossThreads + tid; g < group; g += nb * kFitLossThreads) {
+        R s = R(0);
+        for (int64_t v = g; v < fa.n; v += group) s += x[v];
+        sum += static_cast<double>(s);
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+    if ((tid & 31) == 0) red[tid >> 5] = sum;
     __syncthreads();
-    if (k == 0) last = atomicAdd(fa.arrive, 1u) == static_cast<unsigned>(nb - 1);
+    if (tid == 0) {
+        double t = 0.0;
+#pragma unroll
+        for (int i = 0; i < kFitLossThreads / 32; ++i) t += red[i];
+        fa.block_loss[blockIdx.y * nb + blockIdx.x] = t;
+        __threadfence();  // the share is visible before the count says so
+        last = atomicAdd(fa.arrive, 1u) == static_cast<unsigned>(nb * count - 1);
+    }
     __syncthreads();
     if (!last) return;
     __threadfence();
-    if (k < count) {
-        double s = 0.0;
-        for (int i = 0; i < nb; ++i) s += __ldcg(fa.block_loss + i * kFitChunk + k);
-        fa.hist[t0 - 1 + k] = s;
+    if (tid < count) {
+        double t = 0.0;
+        for (int i = 0; i < nb; ++i) t += __ldcg(fa.block_loss + tid * nb + i);
+        fa.hist[t0 - 1 + tid] = t;
     }
     __syncthreads();
-    if (k == 0) {
+    if (tid == 0) {
         *fa.arrive = 0u;
         int t = t0;
         bool halt = fit_halts(fa, t);
@@ -962,6 +958,14 @@ __global__ void __launch_bounds__(kFitChunk) fit_losses_kernel(const FA fa, cons
         *fa.done = t;
         if (halt) *fa.stop = 1;
     }
+}
+
+template <class R>
+static cudaError_t launch_losses(const FitArgs<R> &fa, const R *vloss, int group, int t0, int count, cudaStream_t s) {
+    // 16 sums a thread: every block ends with an atomic on one counter
+    const int nb = std::min(kFitLossBlocks, (group + 16 * kFitLossThreads - 1) / (16 * kFitLossThreads));
+    fit_losses_kernel<R><<<dim3(nb, count), kFitLossThreads, 0, s>>>(fa, vloss, group, t0, count);
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------- the fitted voxels --
@@ -1133,16 +1137,13 @@ static void bias_corrections(const gac_fit_opts *o, int t, double *c1, double *c
 template <int PREC>
 static gac_status fit_uncoupled(const ModelConst &mc, const gac_fit_opts *o, const FitArgs<typename PrecTraits<PREC>::R> &fa,
                                 typename PrecTraits<PREC>::R *u, typename PrecTraits<PREC>::R *m1,
-                                typename PrecTraits<PREC>::R *m2, size_t bytes_u, int *done, cudaStream_t s) {
+                                typename PrecTraits<PREC>::R *m2, size_t bytes_u, int chunk, int group, int *done, cudaStream_t s) {
     using R = typename PrecTraits<PREC>::R;
     const bool rules = o->tol > 0 || o->convergence_value > 0;
     const int tiles = (fa.n_list + 31) / 32;
-    // 64 MB of loss shares at most
-    const int chunk = static_cast<int>(std::max<int64_t>(4, std::min<int64_t>(rules ? 32 : kFitChunk, (int64_t(64) << 20) / (8 * static_cast<int64_t>(tiles)))));
-    PoolBuf part(s), saved(s);
-    cudaError_t e = part.make(static_cast<size_t>(tiles) * chunk * sizeof(double));
-    if (e == cudaSuccess && rules) e = saved.make(3 * bytes_u);
-    if (e != cudaSuccess) return cuda_fail(e, "fit work arrays");
+    PoolBuf saved(s);
+    cudaError_t e = cudaSuccess;
+    if (rules && (e = saved.make(3 * bytes_u)) != cudaSuccess) return cuda_fail(e, "fit work arrays");
     size_t smem = 0;
     const void *fn = many_ptr<PREC>(mc.kind, o->loss == GAC_FIT_L1, fa.row_stride, &smem);
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -1166,8 +1167,7 @@ static gac_status fit_uncoupled(const ModelConst &mc, const gac_fit_opts *o, con
             steps.c1[k] = R(c1);
             steps.c2[k] = R(c2);
         }
-        double *pp = static_cast<double *>(part.p);
-        void *args[] = {const_cast<ModelConst *>(&mc), const_cast<FitArgs<R> *>(&fa), &u, &m1, &m2, &steps, &t0, &count, &pp};
+        void *args[] = {const_cast<ModelConst *>(&mc), const_cast<FitArgs<R> *>(&fa), &u, &m1, &m2, &steps, &t0, &count};
         return cudaLaunchKernel(fn, dim3(tiles), dim3(32), args, smem, s);
     };
     *done = 0;
@@ -1175,8 +1175,7 @@ static gac_status fit_uncoupled(const ModelConst &mc, const gac_fit_opts *o, con
         const int count = std::min(chunk, o->iterations - t + 1);
         if (rules && (e = copy_state(true)) != cudaSuccess) return cuda_fail(e, "fit state");
         if ((e = run(t, count)) != cudaSuccess) return cuda_fail(e, "fit updates");
-        fit_losses_kernel<<<std::min(tiles, kFitLossBlocks), kFitChunk, 0, s>>>(fa, static_cast<const double *>(part.p), tiles, t, count);
-        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "fit losses");
+        if ((e = launch_losses<R>(fa, fa.vloss, group, t, count, s)) != cudaSuccess) return cuda_fail(e, "fit losses");
         *done = t + count - 1;
         if (rules) {
             int flag[2] = {0, 0};  // stop, done
@@ -1260,28 +1259,56 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     const bool l1 = o->loss == GAC_FIT_L1;
     // the total-variation term couples voxels, and an update is then one launch
     const bool coupled = o->tv_params != 0 && static_cast<R>(o->tv_lambda / static_cast<double>(n_mask)) != R(0);
-    // A mask becomes a list of its voxels where that saves the persistent warps a
-    // round of tiles (below, with 20 warps an SM in FP32); a warp's only tile
-    // would just wait for the list (3-pool, 13,653 voxels, 63% inside: 9.7 ->
-    // 10.2 us an update; 552,960 voxels, 68%: 61 -> 50).
-    const int64_t warps = static_cast<int64_t>(sms) * kFitMinBlocks32 * kFitWarps;
-    auto rounds = [&](int64_t n) { return ((n + 31) / 32 + warps - 1) / warps; };
-    const bool use_list = d_mask && n_mask < N && (!coupled || rounds(n_mask) < rounds(N));
+    // A mask becomes a list of its voxels where at most four fifths of them are
+    // inside, if the persistent warps have more than one tile each (a warp's only
+    // tile would just wait for the list: 3-pool, 13,653 voxels, 63% inside: 9.7 ->
+    // 10.2 us an update).  The list's scattered rows cost a tile about a sixth more
+    // than the grid's whole ones.  Grid -> list, ms per 50 updates with 20 warps an SM:
+    //   inside           55%          70%          80%          90%          95%
+    //   3-pool  122,880  1.04 -> 0.86 1.06 -> 0.97 1.14 -> 1.05 1.14 -> 1.05 1.14 -> 1.17
+    //           552,960  3.15 -> 2.16 3.20 -> 2.66 3.22 -> 3.11 3.23 -> 3.59 3.25 -> 3.56
+    //         1,000,000  5.02 -> 3.69 5.32 -> 4.61 5.38 -> 5.06 5.40 -> 5.67 5.40 -> 5.74
+    //   SMT     552,960  2.01 -> 1.42 2.04 -> 1.62 2.04 -> 1.88 2.05 -> 2.15 2.05 -> 2.16
+    //   mono    552,960  1.28 -> 0.93 1.31 -> 1.07 1.30 -> 1.21 1.31 -> 1.33 1.32 -> 1.36
+    const int64_t one_round = static_cast<int64_t>(sms) * kFitMinBlocks32 * kFitWarps * 32;
+    // Stopping rules ask for each loss before the next update, which the grid's
+    // kernel gives at no extra launch.
+    const bool rules = o->tol > 0 || o->convergence_value > 0;
+    bool many = !coupled;  // many updates a launch
+    bool use_list = d_mask && n_mask < N && (!coupled || (!rules && N > one_round && 5 * n_mask <= 4 * N));
+    // the list, and the voxels' shares of the losses of `chunk` updates (64 MB at
+    // most, or one update's); without memory for them, the grid's kernel, which needs neither
+    PoolBuf list(s), vloss(s);
+    const int chunk = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(rules ? 32 : kFitChunk, (int64_t(64) << 20) / (static_cast<int64_t>(RB) * N))));
+    cudaError_t e = cudaSuccess;
+    if (many || use_list) {
+        e = vloss.make(static_cast<size_t>(chunk) * N * RB);
+        if (e == cudaSuccess && use_list) e = list_masked(d_mask, static_cast<int>(N), n_mask, &list, s);
+        if (e == cudaSuccess && use_list) e = cudaMemsetAsync(vloss.p, 0, static_cast<size_t>(chunk) * N * RB, s);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            many = use_list = false;
+        } else if (e != cudaSuccess) {
+            return cuda_fail(e, "fitted voxels");
+        }
+    }
     const int64_t n_list = use_list ? n_mask : N;
-    const void *fn = step_ptr<PREC>(mc.kind, l1, use_list);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    int per_sm = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kFitBlock, smem);
-    if (e != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
     // persistent warps, each given the same number of 32-voxel tiles (+-1)
-    PoolBuf list(s);
-    if (use_list && (e = list_masked(d_mask, static_cast<int>(N), n_mask, &list, s)) != cudaSuccess)
-        return cuda_fail(e, "fitted voxels");
-    const int64_t tiles = (n_list + 31) / 32;
-    const int64_t slots = static_cast<int64_t>(sms) * std::max(per_sm, 1) * kFitWarps;
-    const int64_t per_warp = (tiles + slots - 1) / slots;
-    const int grid = static_cast<int>((tiles + per_warp * kFitWarps - 1) / (per_warp * kFitWarps));
+    auto shape = [&](const void *f, int64_t n, int *blocks) {
+        cudaError_t c = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        if (c == cudaSuccess) c = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        int per_sm = 0;
+        if (c == cudaSuccess) c = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kFitBlock, smem);
+        const int64_t tiles = (n + 31) / 32, slots = static_cast<int64_t>(sms) * std::max(per_sm, 1) * kFitWarps;
+        const int64_t per_warp = (tiles + slots - 1) / slots;
+        *blocks = static_cast<int>((tiles + per_warp * kFitWarps - 1) / (per_warp * kFitWarps));
+        return c;
+    };
+    int grid = 0, full_grid = 0;
+    const void *fn = step_ptr<PREC>(mc.kind, l1, use_list);
+    if ((e = shape(step_ptr<PREC>(mc.kind, l1, false), N, &full_grid)) != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
+    if ((e = shape(fn, n_list, &grid)) != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
+    const int group = full_grid * kFitBlock;  // voxels between two of a thread's in the grid's kernel
     // work arrays: u (two buffers), Adam moments, block losses, history, flags
     const int I = o->iterations;
     const size_t bytes_u = (static_cast<size_t>(n_list) * P * RB + 15) / 16 * 16;
@@ -1310,7 +1337,7 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     std::memset(&fa, 0, sizeof fa);
     fa.data = d_data;
     fa.mask = d_mask;
-    fa.list = static_cast<const int *>(list.p);
+    fa.list = use_list ? static_cast<const int *>(list.p) : nullptr;
     fa.n_list = static_cast<int>(n_list);
     fa.weight = d_weight;
     fa.nx = o->nx;
@@ -1340,14 +1367,16 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     fa.inv_nx = 1.0f / static_cast<float>(o->nx);
     fa.inv_ny = 1.0f / static_cast<float>(o->ny);
     fa.tv_out = tv_n ? tv0 : nullptr;  // filled with the first update's neighbours
+    R *const shares = static_cast<R *>(vloss.p);
+    fa.vloss = shares;
     const int conv_grid = static_cast<int>(std::min<int64_t>((n_list * P + 255) / 256, static_cast<int64_t>(sms) * 8));
     theta_to_u_kernel<R><<<conv_grid, 256, 0, s>>>(mc, fa, static_cast<const double *>(d_theta.ptr), u0);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "theta to u");
     int done = 0;
-    bool stepwise = coupled;  // a launch per update
-    if (!coupled) {
-        st = fit_uncoupled<PREC>(mc, o, fa, u0, m1, m2, bytes_u, &done, s);
-        if (st == GAC_ERR_OOM) {  // no memory for its loss shares: the other path needs none
+    bool stepwise = !many;  // a launch per update
+    if (many) {
+        st = fit_uncoupled<PREC>(mc, o, fa, u0, m1, m2, bytes_u, chunk, group, &done, s);
+        if (st == GAC_ERR_OOM) {  // no memory for its saved state: the other path needs none
             clear_error();
             stepwise = true;
         } else if (st != GAC_OK) {
@@ -1358,17 +1387,24 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
         if ((e = cudaMemsetAsync(m1, 0, 2 * bytes_u, s)) != cudaSuccess) return cuda_fail(e, "fit memset");
         // iterations in chunks; the stop flag is read between chunks
         constexpr int kChunk = 128;
-        int t = 1;
+        const int sum_every = rules ? 1 : chunk;  // the list's kernel leaves its losses to be summed
+        int t = 1, unsummed = 0;
         while (t <= I) {
             const int t_end = std::min(I, t + kChunk - 1);
             for (; t <= t_end; ++t) {
                 double c1, c2;
                 bias_corrections<PREC>(o, t, &c1, &c2);
                 const bool odd = t & 1;
+                fa.vloss = shares + unsummed * N;
                 fa.tv_in = tv_n ? (odd ? tv0 : tv1) : nullptr;
                 fa.tv_out = tv_n ? (odd ? tv1 : tv0) : nullptr;
                 if ((e = launch_step<R>(fn, grid, smem, s, mc, fa, odd ? u0 : u1, odd ? u1 : u0, m1, m2, R(c1), R(c2), t)) != cudaSuccess)
                     return cuda_fail(e, "fit step");
+                if (use_list && (++unsummed == sum_every || t == t_end)) {
+                    if ((e = launch_losses<R>(fa, shares, group, t - unsummed + 1, unsummed, s)) != cudaSuccess)
+                        return cuda_fail(e, "fit losses");
+                    unsummed = 0;
+                }
             }
             int stop = 0;
             if ((e = cudaMemcpyAsync(&stop, flags, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
