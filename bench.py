@@ -104,13 +104,13 @@ MEASURED = {
     # traffic: DRAM bytes of a quarter-size launch (262,144 / 393,216 / 65,536
     # voxels, all iterations, so every term scales with the voxels) x 3.81;
     # the lines still in L2 when the small launch ends are not counted
-    # (~1-3% of its writes).  warp_instr: from the small-case --set full captures.
-    "mwi3_1m": dict(sources="a8792946f2bdfa8f", traffic_bytes=(78.07e6 + 1696.83e6) * 1e6 / 262144, warp_instr=918.8),
-    "smt_1p5m": dict(sources="559b4e0b19e2b689", traffic_bytes=(32.19e6 + 1120.72e6) * 1.5e6 / 393216, warp_instr=495.2),
-    "axcal_250k": dict(sources="493f595b548eebc5", traffic_bytes=(37.59e6 + 910.33e6) * 250000 / 65536, warp_instr=1215.1),
+    # (~1-3% of its writes).  warp_instr: smsp__inst_executed of small cases.
+    "mwi3_1m": dict(sources="9abb6a90ec58d117", traffic_bytes=(78.36e6 + 1697.09e6) * 1e6 / 262144, warp_instr=912.8),
+    "smt_1p5m": dict(sources="a55baf101b33f8b8", traffic_bytes=(27.15e6 + 1119.01e6) * 1.5e6 / 393216, warp_instr=415.2),
+    "axcal_250k": dict(sources="08a0242b2918f34f", traffic_bytes=(37.45e6 + 908.68e6) * 250000 / 65536, warp_instr=1154.0),
     # the lane-split kernel (2 lanes a chain): the 4,096-voxel workload's data
     # and samples stay in L2, so no DRAM figure
-    "monoexp_4k": dict(sources="cd550974b7613703", traffic_bytes=None, warp_instr=368.8),
+    "monoexp_4k": dict(sources="afb9ab015406985b", traffic_bytes=None, warp_instr=368.8),
 }
 
 
