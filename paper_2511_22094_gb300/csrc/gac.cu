@@ -564,11 +564,11 @@ static gac_status plan_slices(const ModelConst &mc, const gac_mcmc_opts *o, int6
         const double t = 1.02 * static_cast<double>((m * p.n_tiles + p.slots - 1) / p.slots) / m;
         if (t < best) {
             best = t;
-            p.q = (o->iterations + m - 1) / m;
+            p.q = static_cast<int>((static_cast<int64_t>(o->iterations) + m - 1) / m);
         }
     }
     if (p.q == 0) return GAC_OK;
-    p.count = (o->iterations + p.q - 1) / p.q;
+    p.count = static_cast<int>((static_cast<int64_t>(o->iterations) + p.q - 1) / p.q);  // I + q passes 2^31
     p.fn = fn;
     *sp = p;
     return GAC_OK;

@@ -610,7 +610,8 @@ __global__ void __launch_bounds__(kBlock, mh_min_blocks<KIND, GAC_PREC_MIXED>())
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int64_t pos = pos0 + blockIdx.x;
     const int s = static_cast<int>(pos / ra.n_tiles);
-    run_tile<KIND, GAC_PREC_MIXED, false, true>(mc, ra, ss, pos - s * ra.n_tiles, s * q, min(ra.I, (s + 1) * q), smem_raw);
+    const int64_t t_end = static_cast<int64_t>(s + 1) * q;  // may pass 2^31 in the last slice
+    run_tile<KIND, GAC_PREC_MIXED, false, true>(mc, ra, ss, pos - s * ra.n_tiles, s * q, static_cast<int>(t_end < ra.I ? t_end : ra.I), smem_raw);
 }
 
 // The kernel of a kind for (precision, trace, threads per block), or nullptr.
