@@ -136,7 +136,7 @@ extern "C" gac_status gac_ensemble_run(int model_id, const void *data, int64_t n
                                        o->precision == GAC_PREC_MIXED && o->moments_mode == GAC_MOMENTS_ALL_POSTBURNIN);
     const void *fn = nullptr;
     ens_dispatch(mc.kind, o->precision, trace, 0, 0, s, mc, ra, ea, &fn);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return cuda_fail(e, "ensemble kernel smem");
     // the walkers' positions and Welford accumulators live in shared memory:
     // prefer the largest carveout, so that the register limit (2 blocks) binds

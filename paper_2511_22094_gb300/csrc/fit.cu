@@ -1146,7 +1146,7 @@ static gac_status fit_uncoupled(const ModelConst &mc, const gac_fit_opts *o, con
     if (rules && (e = saved.make(3 * bytes_u)) != cudaSuccess) return cuda_fail(e, "fit work arrays");
     size_t smem = 0;
     const void *fn = many_ptr<PREC>(mc.kind, o->loss == GAC_FIT_L1, fa.row_stride, &smem);
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    e = allow_smem(fn, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
     char *sv = static_cast<char *>(saved.p);
@@ -1295,7 +1295,7 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     const int64_t n_list = use_list ? n_mask : N;
     // persistent warps, each given the same number of 32-voxel tiles (+-1)
     auto shape = [&](const void *f, int64_t n, int *blocks) {
-        cudaError_t c = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        cudaError_t c = allow_smem(f, smem);
         if (c == cudaSuccess) c = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         int per_sm = 0;
         if (c == cudaSuccess) c = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kFitBlock, smem);

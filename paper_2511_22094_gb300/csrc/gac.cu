@@ -148,6 +148,24 @@ void keep_staging_pool() {
     done[dev] = true;
 }
 
+// Lets a kernel be launched with `bytes` of dynamic shared memory.  The limit is
+// the process's, not the call's: a call that set its own size would fail another
+// thread's launch of the same kernel with a larger one.  So every call sets the
+// same value, all that the device gives a block beside the kernel's static
+// shared memory, whatever it needs itself.
+cudaError_t allow_smem(const void *fn, size_t bytes) {
+    cudaFuncAttributes a;
+    int dev = 0, block_max = 0;
+    cudaError_t e = cudaFuncGetAttributes(&a, fn);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&block_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    const int most = block_max - static_cast<int>(a.sharedSizeBytes);
+    if (most < 0 || bytes > static_cast<size_t>(most)) return cudaErrorInvalidValue;
+    return a.maxDynamicSharedSizeBytes == most ? cudaSuccess
+                                               : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // ------------------------------------------------------ SMT g(x) table ----
 // g(x) = int_0^1 exp(-x u^2) du by 40-point Gauss-Legendre quadrature: the
 // integrand is entire in u, and for -13 <= x <= 17 the rule agrees with
@@ -435,8 +453,7 @@ static gac_status mh_resident(const ModelConst &mc, int prec, bool trace, int C,
     if (!cfg->fn) return fail(GAC_ERR_INVALID_ARG, "no kernel for kind %d precision %d", mc.kind, prec);
     cfg->block = block;
     cfg->smem = smem_bytes_for(mc.kind, prec, C, mc.n_meas, moments_mode, block);
-    cudaError_t e = cudaFuncSetAttribute(cfg->fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(cfg->smem));
+    cudaError_t e = allow_smem(cfg->fn, cfg->smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
     // prefer the largest shared-memory carveout: the tile and Welford
     // accumulators, not L1, decide how many blocks fit
@@ -547,7 +564,7 @@ static gac_status plan_slices(const ModelConst &mc, const gac_mcmc_opts *o, int6
     p.n_tiles = (n_vox + p.vb - 1) / p.vb;
     if (one_tiles <= one.grid) return GAC_OK;  // a single wave
     p.smem = tile_smem_bytes(mc.n_par, sizeof(double), p.vb, row_stride_for(mc.kind, mc.n_meas), false, all);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(p.smem));
+    cudaError_t e = allow_smem(fn, p.smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     int per_sm = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, p.smem);
@@ -661,7 +678,7 @@ static gac_status plan_split(const ModelConst &mc, int G, int C, int64_t n_vox, 
     threads = std::max(threads, 32 * ((C * G + 31) / 32));  // at least one voxel
     *vb = std::max(1, threads / (C * G));
     const size_t smem = split_smem_bytes(mc.n_par, G, threads, *vb, row_stride_for(mc.kind, mc.n_meas), all);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem)) != cudaSuccess)
@@ -762,7 +779,7 @@ static gac_status plan_spec(const ModelConst &mc, int depth, int C, int64_t n_vo
     const bool help = spec_moment_warps(depth, all);
     const size_t smem = spec_smem_bytes(mc.n_par, 1 << depth, sh.threads, sh.vb, row_stride_for(mc.kind, mc.n_meas), all, help);
     const int block = sh.threads + (help ? 32 * moment_warps(mc.n_par * (sh.threads >> depth), kMomMaxWarps) : 0);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaError_t e = allow_smem(fn, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     int per_sm = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block, smem);

@@ -18,6 +18,7 @@ int n_samples(int I, int B, int T);
 gac_status validate_opts(const gac_mcmc_opts *o, int64_t n_vox);
 int row_stride_for(int kind, int M);
 void keep_staging_pool();
+cudaError_t allow_smem(const void *fn, size_t bytes);
 
 // Device view of a caller buffer (see DevBuf::make in gac.cu).
 struct DevBuf {

@@ -153,8 +153,7 @@ static cudaError_t launch_forward(int prec, const ModelConst &mc, const double *
     const int row_stride = row_stride_for(KIND, std::max(mc.n_meas, mc.n_par));
     const size_t smem = static_cast<size_t>(kFwdBlock) * row_stride * sizeof(float);
     if (smem > 44 * 1024) {  // beside the model's tables, past the default 48 KB
-        const cudaError_t e = cudaFuncSetAttribute(forward_f_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   static_cast<int>(smem));
+        const cudaError_t e = allow_smem(reinterpret_cast<const void *>(&forward_f_kernel<KIND>), smem);
         if (e != cudaSuccess) return e;
     }
     const int64_t blocks = (n + kFwdBlock - 1) / kFwdBlock;

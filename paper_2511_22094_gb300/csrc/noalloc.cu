@@ -153,7 +153,7 @@ extern "C" gac_status gac_mcmc_run_noalloc(int model_id, const void *data, int64
 
     const void *fn = noalloc_fn(mc.kind);
     const size_t smem = tile_smem_bytes(mc.n_par, 8, ra.vox_per_block, ra.row_stride, false, blocked);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
     e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(carveout)");

@@ -12,7 +12,7 @@
 
 // op: "malloc" (x: bytes), "free" (x: bytes), "attr" (x: attribute, value), "launch" (x: grid
 // x, grid y, block, dynamic shared bytes; args: the kernel's) return an error code or 0;
-// "occupancy" (x: block, dynamic shared bytes) returns resident blocks an SM.
+// ("attr" once it is set); "occupancy" (x: block, dynamic shared bytes) returns resident blocks an SM.
 using Hook = int (*)(const char *op, const char *kernel, const long long *x, void **args);
 
 namespace {
@@ -51,6 +51,7 @@ cudaError_t launch(const void *fn, dim3 grid, dim3 block, void **args, size_t sm
 
 extern "C" {
 void fake_set_hook(Hook h) { g_hook = h; }
+void fake_forget_limits() { g_limit.clear(); }
 void fake_mark_device(void *p, int on) {
     if (on) g_alloc[p] = 0;
     else g_alloc.erase(p);
@@ -82,13 +83,11 @@ cudaError_t cudaLaunchKernel(const void *fn, dim3 grid, dim3 block, void **args,
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *fn, void **args) { return launch(fn, c->gridDim, c->blockDim, args, c->dynamicSmemBytes); }
 
 cudaError_t cudaFuncSetAttribute(const void *fn, cudaFuncAttribute a, int v) {
-    const cudaError_t e = call("attr", fn, a, v);
-    if (e != cudaSuccess) return e;
     if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) {
         if (v < 0 || v + kStatic > 227 * 1024) return cudaErrorInvalidValue;
         g_limit[fn] = v;
     }
-    return cudaSuccess;
+    return call("attr", fn, a, v);
 }
 cudaError_t cudaFuncGetAttributes(cudaFuncAttributes *a, const void *fn) {
     std::memset(a, 0, sizeof *a);

@@ -34,7 +34,8 @@ def short(mangled):
 
 class FakeGpu:
     """Records launches (name, grid x, grid y, block, shared bytes) and settings; `memory` bounds the
-    device memory in use; `on_launch(name, args)` may return an error code."""
+    device memory in use; `on_launch(name, args)` may return an error code; `on_limit(name)` runs when
+    a call has set a kernel's shared-memory limit."""
 
     def __init__(self, lib):
         self.lib = lib
@@ -46,7 +47,8 @@ class FakeGpu:
         self.launches, self.limits, self.sizes = [], [], []
         self.in_use = self.peak = 0
         self.memory = None
-        self.on_launch = None
+        self.on_launch = self.on_limit = None
+        self.lib.fake_forget_limits()
 
     def _call(self, op, kernel, x, args):
         name = short(kernel.decode())
@@ -60,6 +62,8 @@ class FakeGpu:
             self.in_use -= x[0]
         elif op == b"attr" and x[0] == 8:  # MaxDynamicSharedMemorySize
             self.limits.append((name, x[1]))
+            if self.on_limit:
+                self.on_limit(name)
         elif op == b"occupancy":
             block, smem = x[0], x[1]
             by_regs = next(n for pat, n in RESIDENT if re.search(pat, name)) * (1 if "fit_" in name or "mh_s" in name else 256 // block)

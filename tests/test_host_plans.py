@@ -47,3 +47,69 @@ def test_slices_cover_every_iteration_of_every_tile(fake, w, n, iterations):
         assert (pos, qi, block) == (end, q, 256) and 1 <= grid <= n_tiles
         end += grid
     assert end == count * n_tiles
+
+
+def _echoes(n):
+    return W.MWI3_1M.with_(acq=tuple(2.0 + 0.7 * k for k in range(n)))
+
+
+def _forward(fake, n_acq, n):
+    g, _ = fake
+    w = _echoes(n_acq)
+    g.forward_host(g.gac_model_register(w.kind, w.acq, w.lb, w.ub, w.step), np.tile(w.ub, (n, 1)))
+
+
+def _fit(fake, w, shape, **kw):
+    g, _ = fake
+    mid = g.gac_model_register(w.kind, w.acq, w.lb, w.ub, w.step)
+    n = int(np.prod(shape))
+    return g.fit_host(mid, np.zeros((n, g.gac_model_info(mid)[1]), np.float32), np.tile(w.ub, (n, 1)), shape=shape, **kw)
+
+
+def _ensemble(fake, w, n):
+    g, _ = fake
+    mid = g.gac_model_register(w.kind, w.acq, w.lb, w.ub, w.step)
+    g.run_ensemble_host(mid, np.zeros((n, g.gac_model_info(mid)[1]), np.float32), None, sigma_scalar=1.0, iterations=10,
+                        burnin=0, thin=5, n_walkers=20, seed=1)
+
+
+def _run(w, n, C, **kw):
+    return lambda fake: _sampler(fake, w, n, C, iterations=300, burnin=0, thin=100, **kw)
+
+
+#: calls that launch the same kernel with more, then with less shared memory
+SAME_KERNEL = {
+    "forward": (lambda f: _forward(f, 64, 100), lambda f: _forward(f, 48, 100)),
+    "sampler": (_run(_echoes(64), 100_000, 4), _run(_echoes(6), 100_000, 4)),
+    "sampler-slices": (_run(_echoes(64), 23_250, 4), _run(_echoes(24), 23_250, 4)),
+    "sampler-lanes": (_run(_echoes(24), 3000, 1, lanes_per_chain=4), _run(_echoes(18), 300, 1, lanes_per_chain=4)),
+    "sampler-tree": (_run(_echoes(64), 301, 4), _run(_echoes(6), 290, 4)),
+    "ensemble": (lambda f: _ensemble(f, _echoes(64), 100), lambda f: _ensemble(f, _echoes(6), 100)),
+    "fit": (lambda f: _fit(f, _echoes(24), (9, 8, 7), iterations=20), lambda f: _fit(f, _echoes(12), (9, 8, 7), iterations=20)),
+    "fit-tv": (lambda f: _fit(f, _echoes(24), (9, 8, 7), iterations=20, tv_lambda=0.1, tv_params=1),
+               lambda f: _fit(f, _echoes(12), (9, 8, 7), iterations=20, tv_lambda=0.1, tv_params=1)),
+}
+
+
+@pytest.mark.parametrize("calls", SAME_KERNEL.values(), ids=SAME_KERNEL)
+def test_another_threads_smaller_launch_does_not_fail_a_larger_one(fake, calls):
+    """The kernels' shared-memory limits are the process's: a call with less between another
+    call's settings and its launches leaves those as they are."""
+    _, gpu = fake
+    large, small = calls
+    gpu.reset()
+    small(fake)
+    names = set(gpu.names())
+    gpu.reset()
+    inside = []
+
+    def on_limit(name):
+        if name not in inside:
+            inside.append(name)
+            small(fake)
+
+    gpu.on_limit = on_limit
+    large(fake)  # a launch past the kernel's limit fails
+    assert inside and names <= set(gpu.names())
+    for name in names:
+        assert len({v for k, v in gpu.limits if k == name}) <= 1
