@@ -1132,29 +1132,25 @@ static void bias_corrections(const gac_fit_opts *o, int t, double *c1, double *c
 // All updates of a fit without coupling between voxels; u, m1 and m2 as in
 // fit_run_prec, the result in u.  With stopping rules a launch takes fewer
 // updates, and one that runs past the stop is taken back: the state before it is
-// kept, and the updates up to the stop run again.  GAC_ERR_OOM: nothing has
-// been launched on the state.
+// kept (in `saved`, 3 bytes_u bytes), and the updates up to the stop run again.
 template <int PREC>
 static gac_status fit_uncoupled(const ModelConst &mc, const gac_fit_opts *o, const FitArgs<typename PrecTraits<PREC>::R> &fa,
                                 typename PrecTraits<PREC>::R *u, typename PrecTraits<PREC>::R *m1,
-                                typename PrecTraits<PREC>::R *m2, size_t bytes_u, int chunk, int group, int *done, cudaStream_t s) {
+                                typename PrecTraits<PREC>::R *m2, size_t bytes_u, char *saved, int chunk, int group, int *done, cudaStream_t s) {
     using R = typename PrecTraits<PREC>::R;
     const bool rules = o->tol > 0 || o->convergence_value > 0;
     const int tiles = (fa.n_list + 31) / 32;
-    PoolBuf saved(s);
     cudaError_t e = cudaSuccess;
-    if (rules && (e = saved.make(3 * bytes_u)) != cudaSuccess) return cuda_fail(e, "fit work arrays");
     size_t smem = 0;
     const void *fn = many_ptr<PREC>(mc.kind, o->loss == GAC_FIT_L1, fa.row_stride, &smem);
     e = allow_smem(fn, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
-    char *sv = static_cast<char *>(saved.p);
     auto copy_state = [&](bool save) {
         R *const a[3] = {u, m1, m2};
         for (int i = 0; i < 3; ++i) {
-            const cudaError_t c = save ? cudaMemcpyAsync(sv + i * bytes_u, a[i], bytes_u, cudaMemcpyDeviceToDevice, s)
-                                       : cudaMemcpyAsync(a[i], sv + i * bytes_u, bytes_u, cudaMemcpyDeviceToDevice, s);
+            const cudaError_t c = save ? cudaMemcpyAsync(saved + i * bytes_u, a[i], bytes_u, cudaMemcpyDeviceToDevice, s)
+                                       : cudaMemcpyAsync(a[i], saved + i * bytes_u, bytes_u, cudaMemcpyDeviceToDevice, s);
             if (c != cudaSuccess) return c;
         }
         return cudaSuccess;
@@ -1373,17 +1369,18 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     theta_to_u_kernel<R><<<conv_grid, 256, 0, s>>>(mc, fa, static_cast<const double *>(d_theta.ptr), u0);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "theta to u");
     int done = 0;
-    bool stepwise = !many;  // a launch per update
-    if (many) {
-        st = fit_uncoupled<PREC>(mc, o, fa, u0, m1, m2, bytes_u, chunk, group, &done, s);
-        if (st == GAC_ERR_OOM) {  // no memory for its saved state: the other path needs none
-            clear_error();
-            stepwise = true;
-        } else if (st != GAC_OK) {
-            return st;
-        }
+    // without memory for the state that stopping rules keep: a launch per update,
+    // decided before the first launch, as the updates change the state in place
+    PoolBuf saved(s);
+    if (many && rules && (e = saved.make(3 * bytes_u)) != cudaSuccess) {
+        if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "fit work arrays");
+        cudaGetLastError();
+        many = false;
     }
-    if (stepwise) {
+    if (many) {
+        st = fit_uncoupled<PREC>(mc, o, fa, u0, m1, m2, bytes_u, static_cast<char *>(saved.p), chunk, group, &done, s);
+        if (st != GAC_OK) return st;
+    } else {
         if ((e = cudaMemsetAsync(m1, 0, 2 * bytes_u, s)) != cudaSuccess) return cuda_fail(e, "fit memset");
         // iterations in chunks; the stop flag is read between chunks
         constexpr int kChunk = 128;
@@ -1421,8 +1418,8 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
         if ((e = cudaMemcpyAsync(loss_history, hist, done * sizeof(double), cudaMemcpyDefault, s)) != cudaSuccess)
             return cuda_fail(e, "loss history");
     }
-    // u of the last update (stepwise, iteration `done` wrote buffer (done & 1) ? u1 : u0) -> theta
-    u_to_theta_kernel<R><<<conv_grid, 256, 0, s>>>(mc, fa, stepwise && (done & 1) ? u1 : u0, static_cast<double *>(d_theta.ptr));
+    // u of the last update (a launch per update: iteration `done` wrote buffer (done & 1) ? u1 : u0) -> theta
+    u_to_theta_kernel<R><<<conv_grid, 256, 0, s>>>(mc, fa, !many && (done & 1) ? u1 : u0, static_cast<double *>(d_theta.ptr));
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "u to theta");
     if ((st = d_theta.copy_out()) != GAC_OK) return st;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "fit");

@@ -28,6 +28,7 @@ cudaError_t call(const char *op, const void *fn, long long a, long long b, long 
     const long long x[4] = {a, b, c, d};
     return g_hook ? static_cast<cudaError_t>(g_hook(op, fn ? names()[fn].c_str() : "", x, args)) : cudaSuccess;
 }
+thread_local cudaError_t t_last = cudaSuccess;  // of the last failed launch
 size_t limit(const void *fn) { return g_limit.count(fn) ? g_limit[fn] : 48 * 1024 - kStatic; }
 cudaError_t alloc(void **p, size_t n) {
     const cudaError_t e = call("malloc", nullptr, static_cast<long long>(n), 0);
@@ -44,8 +45,10 @@ cudaError_t release(void *p) {
     return cudaSuccess;
 }
 cudaError_t launch(const void *fn, dim3 grid, dim3 block, void **args, size_t smem) {
-    if (smem > limit(fn) || grid.x < 1 || grid.x > 2147483647u || block.x < 1 || block.x > 1024) return cudaErrorInvalidValue;
-    return call("launch", fn, grid.x, grid.y, block.x, static_cast<long long>(smem), args);
+    const bool bad = smem > limit(fn) || grid.x < 1 || grid.x > 2147483647u || block.x < 1 || block.x > 1024;
+    const cudaError_t e = bad ? cudaErrorInvalidValue : call("launch", fn, grid.x, grid.y, block.x, static_cast<long long>(smem), args);
+    if (e != cudaSuccess) t_last = e;
+    return e;
 }
 }  // namespace
 
@@ -131,7 +134,11 @@ cudaError_t cudaGetDevice(int *d) {
     return cudaSuccess;
 }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError() {
+    const cudaError_t e = t_last;
+    t_last = cudaSuccess;
+    return e;
+}
 const char *cudaGetErrorString(cudaError_t e) { return e == cudaErrorMemoryAllocation ? "out of memory" : "error"; }
 cudaError_t cudaDeviceGetDefaultMemPool(cudaMemPool_t *, int) { return cudaErrorNotSupported; }
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void *) { return cudaSuccess; }

@@ -113,3 +113,37 @@ def test_another_threads_smaller_launch_does_not_fail_a_larger_one(fake, calls):
     assert inside and names <= set(gpu.names())
     for name in names:
         assert len({v for k, v in gpu.limits if k == name}) <= 1
+
+
+def _count(gpu, kernel):
+    return sum(n.startswith(kernel) for n in gpu.names())
+
+
+@pytest.mark.parametrize("kernel,launch", [("fit_many", 1), ("fit_losses", 1), ("fit_many", 2), ("fit_losses", 2)])
+@pytest.mark.parametrize("tol", [0.0, 1e-300])
+def test_a_fit_whose_launch_fails_reports_it(fake, kernel, launch, tol):
+    """Also where the failure is a want of memory: the updates before it have changed the state in
+    place, so no other path may start from it."""
+    g, gpu = fake
+    gpu.reset()
+    gpu.on_launch = lambda name, args: fake_gpu.OOM if name.startswith(kernel) and _count(gpu, kernel) == launch else 0
+    with pytest.raises(g.GacError) as err:
+        _fit(fake, _echoes(12), (9, 8, 7), iterations=300, tol=tol)
+    assert err.value.status == 4 and _count(gpu, "fit_step") == 0 and gpu.in_use == 0
+
+
+def test_a_fit_without_memory_for_its_saved_state(fake):
+    """Stopping rules keep the state of before a launch of many updates; without memory for it
+    every update is a launch, from the first on."""
+    _, gpu = fake
+    shape, n = (9, 8, 7), 504
+    gpu.reset()
+    _fit(fake, _echoes(12), shape, iterations=70, tol=1e-300)
+    assert _count(gpu, "fit_many") == 3
+    saved = 3 * n * 9 * 4
+    assert gpu.sizes[-1] == saved
+    peak = gpu.peak
+    gpu.reset()
+    gpu.memory = peak - 1
+    _fit(fake, _echoes(12), shape, iterations=70, tol=1e-300)
+    assert _count(gpu, "fit_many") == 0 and _count(gpu, "fit_step") == 70 and gpu.in_use == 0
