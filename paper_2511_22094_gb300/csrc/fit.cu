@@ -1099,9 +1099,11 @@ struct PoolBuf {
     PoolBuf(const PoolBuf &) = delete;
     PoolBuf &operator=(const PoolBuf &) = delete;
     cudaError_t make(size_t bytes) { return cudaMallocAsync(&p, bytes, s); }
-    ~PoolBuf() {
+    void release() {
         if (p) cudaFreeAsync(p, s);
+        p = nullptr;
     }
+    ~PoolBuf() { release(); }
 };
 
 // Fills *list (device) with the indices of the n_mask non-zero bytes of the mask.
@@ -1272,23 +1274,6 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     const bool rules = o->tol > 0 || o->convergence_value > 0;
     bool many = !coupled;  // many updates a launch
     bool use_list = d_mask && n_mask < N && (!coupled || (!rules && N > one_round && 5 * n_mask <= 4 * N));
-    // the list, and the voxels' shares of the losses of `chunk` updates (64 MB at
-    // most, or one update's); without memory for them, the grid's kernel, which needs neither
-    PoolBuf list(s), vloss(s);
-    const int chunk = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(rules ? 32 : kFitChunk, (int64_t(64) << 20) / (static_cast<int64_t>(RB) * N))));
-    cudaError_t e = cudaSuccess;
-    if (many || use_list) {
-        e = vloss.make(static_cast<size_t>(chunk) * N * RB);
-        if (e == cudaSuccess && use_list) e = list_masked(d_mask, static_cast<int>(N), n_mask, &list, s);
-        if (e == cudaSuccess && use_list) e = cudaMemsetAsync(vloss.p, 0, static_cast<size_t>(chunk) * N * RB, s);
-        if (e == cudaErrorMemoryAllocation) {
-            cudaGetLastError();
-            many = use_list = false;
-        } else if (e != cudaSuccess) {
-            return cuda_fail(e, "fitted voxels");
-        }
-    }
-    const int64_t n_list = use_list ? n_mask : N;
     // persistent warps, each given the same number of 32-voxel tiles (+-1)
     auto shape = [&](const void *f, int64_t n, int *blocks) {
         cudaError_t c = allow_smem(f, smem);
@@ -1300,28 +1285,46 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
         *blocks = static_cast<int>((tiles + per_warp * kFitWarps - 1) / (per_warp * kFitWarps));
         return c;
     };
-    int grid = 0, full_grid = 0;
-    const void *fn = step_ptr<PREC>(mc.kind, l1, use_list);
-    if ((e = shape(step_ptr<PREC>(mc.kind, l1, false), N, &full_grid)) != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
-    if ((e = shape(fn, n_list, &grid)) != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
-    const int group = full_grid * kFitBlock;  // voxels between two of a thread's in the grid's kernel
-    // work arrays: u (two buffers), Adam moments, block losses, history, flags
+    // The list, the voxels' shares of the losses of `chunk` updates (64 MB at most,
+    // or one update's) and the state that stopping rules keep are allocated before
+    // the first launch; where they, or the work arrays beside them, do not fit,
+    // they are given back and the grid's kernel runs, which needs none of them.
+    const int chunk = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(rules ? 32 : kFitChunk, (int64_t(64) << 20) / (static_cast<int64_t>(RB) * N))));
     const int I = o->iterations;
-    const size_t bytes_u = (static_cast<size_t>(n_list) * P * RB + 15) / 16 * 16;
-    // the penalised maps over the grid, two buffers, when there is a list
-    const size_t tv_n = use_list && coupled ? static_cast<size_t>(__builtin_popcount(o->tv_params & ((1u << P) - 1u))) * N : 0;
-    const size_t bytes_tv = (tv_n * RB + 15) / 16 * 16;
-    const size_t total = 4 * bytes_u + 2 * bytes_tv + std::max(grid, kFitLossBlocks * kFitChunk) * sizeof(double) +
-                         static_cast<size_t>(std::max(I, 1)) * sizeof(double) + 3 * sizeof(int);
-    void *base = nullptr;
-    e = cudaMallocAsync(&base, total, s);
-    if (e != cudaSuccess) return cuda_fail(e, "fit work arrays");
-    struct Free {
-        void *p;
-        cudaStream_t s;
-        ~Free() { cudaFreeAsync(p, s); }
-    } guard{base, s};
-    char *b = static_cast<char *>(base);
+    PoolBuf list(s), vloss(s), saved(s), work(s);
+    cudaError_t e = cudaSuccess;
+    int grid = 0, full_grid = 0;
+    if ((e = shape(step_ptr<PREC>(mc.kind, l1, false), N, &full_grid)) != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
+    const int group = full_grid * kFitBlock;  // voxels between two of a thread's in the grid's kernel
+    const void *fn = nullptr;
+    int64_t n_list = 0;
+    size_t bytes_u = 0, bytes_tv = 0, tv_n = 0;
+    for (;;) {
+        n_list = use_list ? n_mask : N;
+        fn = step_ptr<PREC>(mc.kind, l1, use_list);
+        if ((e = shape(fn, n_list, &grid)) != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
+        // work arrays: u (two buffers), Adam moments, the penalised maps over the grid
+        // (two buffers) when there is a list, block losses, history, flags
+        bytes_u = (static_cast<size_t>(n_list) * P * RB + 15) / 16 * 16;
+        tv_n = use_list && coupled ? static_cast<size_t>(__builtin_popcount(o->tv_params & ((1u << P) - 1u))) * N : 0;
+        bytes_tv = (tv_n * RB + 15) / 16 * 16;
+        const size_t total = 4 * bytes_u + 2 * bytes_tv + std::max(grid, kFitLossBlocks * kFitChunk) * sizeof(double) +
+                             static_cast<size_t>(std::max(I, 1)) * sizeof(double) + 3 * sizeof(int);
+        if (many || use_list) e = vloss.make(static_cast<size_t>(chunk) * N * RB);
+        if (e == cudaSuccess && use_list) e = list_masked(d_mask, static_cast<int>(N), n_mask, &list, s);
+        if (e == cudaSuccess && use_list) e = cudaMemsetAsync(vloss.p, 0, static_cast<size_t>(chunk) * N * RB, s);
+        if (e == cudaSuccess && many && rules) e = saved.make(3 * bytes_u);
+        if (e == cudaSuccess) e = work.make(total);
+        if (e == cudaSuccess) break;
+        if (e != cudaErrorMemoryAllocation || !(many || use_list)) return cuda_fail(e, "fit work arrays");
+        cudaGetLastError();
+        vloss.release();
+        list.release();
+        saved.release();
+        many = use_list = false;
+        e = cudaSuccess;
+    }
+    char *b = static_cast<char *>(work.p);
     R *const u0 = reinterpret_cast<R *>(b), *const u1 = reinterpret_cast<R *>(b + bytes_u);
     R *const m1 = reinterpret_cast<R *>(b + 2 * bytes_u), *const m2 = reinterpret_cast<R *>(b + 3 * bytes_u);
     R *const tv0 = reinterpret_cast<R *>(b + 4 * bytes_u), *const tv1 = reinterpret_cast<R *>(b + 4 * bytes_u + bytes_tv);
@@ -1369,14 +1372,6 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     theta_to_u_kernel<R><<<conv_grid, 256, 0, s>>>(mc, fa, static_cast<const double *>(d_theta.ptr), u0);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "theta to u");
     int done = 0;
-    // without memory for the state that stopping rules keep: a launch per update,
-    // decided before the first launch, as the updates change the state in place
-    PoolBuf saved(s);
-    if (many && rules && (e = saved.make(3 * bytes_u)) != cudaSuccess) {
-        if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "fit work arrays");
-        cudaGetLastError();
-        many = false;
-    }
     if (many) {
         st = fit_uncoupled<PREC>(mc, o, fa, u0, m1, m2, bytes_u, static_cast<char *>(saved.p), chunk, group, &done, s);
         if (st != GAC_OK) return st;

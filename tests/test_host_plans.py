@@ -140,10 +140,39 @@ def test_a_fit_without_memory_for_its_saved_state(fake):
     gpu.reset()
     _fit(fake, _echoes(12), shape, iterations=70, tol=1e-300)
     assert _count(gpu, "fit_many") == 3
-    saved = 3 * n * 9 * 4
-    assert gpu.sizes[-1] == saved
+    assert 3 * n * 9 * 4 in gpu.sizes
     peak = gpu.peak
     gpu.reset()
     gpu.memory = peak - 1
     _fit(fake, _echoes(12), shape, iterations=70, tol=1e-300)
     assert _count(gpu, "fit_many") == 0 and _count(gpu, "fit_step") == 70 and gpu.in_use == 0
+
+
+@pytest.mark.parametrize("name", ["uncoupled", "uncoupled-masked", "uncoupled-rules", "tv-masked"])
+def test_a_fit_runs_in_the_memory_that_a_launch_per_update_needs(fake, name):
+    """The list of voxels, the loss shares and the saved state are extras: a call that has no room for
+    them beside the work arrays does without, wherever the room ends."""
+    _, gpu = fake
+    tv = dict(tv_lambda=0.1, tv_params=1)
+    shape = (64, 50, 40) if name == "tv-masked" else (40, 30, 11)
+    n = int(np.prod(shape))
+    kw = dict(iterations=50, tol=1e-300 if name == "uncoupled-rules" else 0.0)
+    if "masked" in name:
+        kw["mask"] = (np.arange(n) % 3 != 0).astype(np.uint8)
+    plain = {**kw, **tv, "tol": 1e-300}
+    if name == "tv-masked":
+        kw.update(tv)
+    run = lambda **k: (gpu.reset(), setattr(gpu, "memory", k.pop("memory", None)), _fit(fake, W.MONOEXP_4K, shape, **k))
+    run(**plain)
+    least = gpu.peak
+    assert _count(gpu, "fit_step") == 50
+    run(**kw)
+    most = gpu.peak
+    assert most > least and _count(gpu, "fit_step") == 0
+    for memory in np.linspace(least, most, 33).astype(int):
+        run(**kw, memory=memory)
+        assert _count(gpu, "theta_to_u") == 1 and gpu.in_use == 0
+        assert (_count(gpu, "fit_step") == 50) == (memory < most)
+    with pytest.raises(fake[0].GacError) as err:
+        run(**kw, memory=least - 100_000)
+    assert err.value.status == 4 and gpu.in_use == 0
