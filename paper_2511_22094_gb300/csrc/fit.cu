@@ -51,11 +51,12 @@ struct FitArgs {
     float inv_nx, inv_ny;  // 1 / nx, 1 / ny rounded to float
     int *stop;             // set by the last block of the iteration that stops
     int *done;             // updates taken
-    unsigned *arrive;      // blocks of the current launch that have finished (reset by the last)
+    unsigned *arrive;      // blocks of the current launch that have finished (reset by the last);
+                           // fit_losses_kernel: [0] updates summed, [1 + k] blocks of update k
     double *hist;          // [iterations] loss history
     double tol, conv_value;
     int window;
-    double *block_loss;    // [gridDim.x]
+    double *block_loss;    // [gridDim.x], or fit_losses_kernel's [updates][virtual warps]
     // The n_list voxels to visit: the fitted ones in order, or nullptr: voxels 0
     // .. n_list - 1, of which the mask leaves some out.  Parameters and moments
     // are [P][n_list], in the list's order.
@@ -818,8 +819,7 @@ __device__ void fit_check(const FA &fa, int n_blocks, int t, double *red) {
 // updates 1.70 -> 0.22 ms; 3-pool, 96 x 96 x 60, 100 updates 5.6 -> 3.3 ms, with
 // a mask of 68% of it 5.7 -> 2.4 ms.
 constexpr int kFitChunk = 128;
-constexpr int kFitLossThreads = 256;  // >= kFitChunk
-constexpr int kFitLossBlocks = 32;  // blocks of fit_losses_kernel an update, at most
+constexpr int kFitLossThreads = 256;
 
 template <class R>
 struct FitSteps {
@@ -909,62 +909,78 @@ __global__ void __launch_bounds__(32, PREC == GAC_PREC_FP32 ? 20 : 8)
     }
 }
 
-// The losses of `count` updates from the voxels' shares (fa.vloss), summed as
-// fit_step_kernel's threads do it: voxels g, g + group, ... in the kernel's
-// precision, everything after that in FP64.  (An exact sum would differ from
-// theirs: 345,840 voxels, L2, by 9e-9 of the loss.)  blockIdx.y: the update.  The last
-// block to finish adds the blocks' shares in order, records the losses and
-// applies the stopping rules to each update in turn.  Bound by the reads, which
-// come from L2: about 0.5 us an update of 552,960 voxels.
+// The losses of `count` updates from the voxels' shares (fa.vloss), summed in the
+// order of fit_step_kernel on `blocks` blocks, so that a loss and what the
+// stopping rules make of it are the same bits on every path: a lane adds its
+// voxels v, v + 32 warps, ... in the kernel's precision, a warp its lanes in FP64,
+// then four warps make a block's share and the blocks' shares are added as
+// fit_check does.  blockIdx.y: the update; its last block adds the shares and
+// records the loss, and the last update's applies the stopping rules to each in
+// turn.  Bound by the reads, which come from L2 (about 0.5 us an update of 552,960
+// voxels) or, with few updates a launch, from HBM: the blocks then fill the GPU.
+// (24 blocks for a single update of 16 million voxels read at 100 GB/s.)
 template <class R>
-__global__ void __launch_bounds__(kFitLossThreads) fit_losses_kernel(const FitArgs<R> fa, const R *vloss, int group, int t0, int count) {
-    __shared__ double red[kFitLossThreads / 32];
+__global__ void __launch_bounds__(kFitLossThreads) fit_losses_kernel(const FitArgs<R> fa, const R *vloss, int blocks, int t0, int count) {
+    __shared__ double red[kFitBlock];
     __shared__ bool last;
     if (*fa.stop) return;  // the same for every thread; only this kernel's last block sets it
-    const int nb = gridDim.x, tid = threadIdx.x;
-    const R *x = vloss + blockIdx.y * fa.n;
-    double sum = 0.0;
-    for (int g = blockIdx.x * kFitLossThreads + tid; g < group; g += nb * kFitLossThreads) {
+    const int tid = threadIdx.x, lane = tid & 31, k = blockIdx.y;
+    const int warps = blocks * kFitWarps;
+    const R *x = vloss + k * fa.n;
+    double *sums = fa.block_loss + static_cast<int64_t>(k) * warps;
+    for (int w = blockIdx.x * (kFitLossThreads / 32) + (tid >> 5); w < warps; w += gridDim.x * (kFitLossThreads / 32)) {
         R s = R(0);
-        for (int64_t v = g; v < fa.n; v += group) s += x[v];
-        sum += static_cast<double>(s);
-    }
+#pragma unroll 8
+        for (int64_t v = w * 32 + lane; v < fa.n; v += warps * 32) s += x[v];
+        double sum = static_cast<double>(s);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
-    if ((tid & 31) == 0) red[tid >> 5] = sum;
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+        if (lane == 0) sums[w] = sum;
+    }
+    __threadfence();  // the sums are visible before the count says so
     __syncthreads();
-    if (tid == 0) {
-        double t = 0.0;
-#pragma unroll
-        for (int i = 0; i < kFitLossThreads / 32; ++i) t += red[i];
-        fa.block_loss[blockIdx.y * nb + blockIdx.x] = t;
-        __threadfence();  // the share is visible before the count says so
-        last = atomicAdd(fa.arrive, 1u) == static_cast<unsigned>(nb * count - 1);
-    }
+    if (tid == 0) last = atomicAdd(fa.arrive + 1 + k, 1u) == gridDim.x - 1;
     __syncthreads();
     if (!last) return;
     __threadfence();
-    if (tid < count) {
-        double t = 0.0;
-        for (int i = 0; i < nb; ++i) t += __ldcg(fa.block_loss + tid * nb + i);
-        fa.hist[t0 - 1 + tid] = t;
+    if (tid < kFitBlock) {
+        double s = 0.0;
+        for (int b = tid; b < blocks; b += kFitBlock) {
+            double t = 0.0;
+#pragma unroll
+            for (int i = 0; i < kFitWarps; ++i) t += __ldcg(sums + b * kFitWarps + i);
+            s += t;
+        }
+        red[tid] = s;
     }
     __syncthreads();
+    for (int n = kFitBlock / 2; n > 0; n >>= 1) {
+        if (tid < n) red[tid] += red[tid + n];
+        __syncthreads();
+    }
     if (tid == 0) {
-        *fa.arrive = 0u;
-        int t = t0;
-        bool halt = fit_halts(fa, t);
-        while (!halt && t < t0 + count - 1) halt = fit_halts(fa, ++t);
-        *fa.done = t;
-        if (halt) *fa.stop = 1;
+        fa.hist[t0 - 1 + k] = red[0];
+        fa.arrive[1 + k] = 0u;
+        __threadfence();
+        if (atomicAdd(fa.arrive, 1u) == static_cast<unsigned>(count - 1)) {
+            __threadfence();
+            *fa.arrive = 0u;
+            int t = t0;
+            bool halt = fit_halts(fa, t);
+            while (!halt && t < t0 + count - 1) halt = fit_halts(fa, ++t);
+            *fa.done = t;
+            if (halt) *fa.stop = 1;
+        }
     }
 }
 
 template <class R>
-static cudaError_t launch_losses(const FitArgs<R> &fa, const R *vloss, int group, int t0, int count, cudaStream_t s) {
-    // 16 sums a thread: every block ends with an atomic on one counter
-    const int nb = std::min(kFitLossBlocks, (group + 16 * kFitLossThreads - 1) / (16 * kFitLossThreads));
-    fit_losses_kernel<R><<<dim3(nb, count), kFitLossThreads, 0, s>>>(fa, vloss, group, t0, count);
+static cudaError_t launch_losses(const FitArgs<R> &fa, const R *vloss, int blocks, int sms, int t0, int count, cudaStream_t s) {
+    // 16 sums a lane (every block ends with an atomic), or fewer where a launch of few
+    // updates would leave SMs idle
+    const int all = (blocks * kFitWarps * 32 + kFitLossThreads - 1) / kFitLossThreads;
+    const int nb = std::min(all, std::max((all + 15) / 16, (8 * sms + count - 1) / count));
+    fit_losses_kernel<R><<<dim3(nb, count), kFitLossThreads, 0, s>>>(fa, vloss, blocks, t0, count);
     return cudaGetLastError();
 }
 
@@ -1138,7 +1154,7 @@ static void bias_corrections(const gac_fit_opts *o, int t, double *c1, double *c
 template <int PREC>
 static gac_status fit_uncoupled(const ModelConst &mc, const gac_fit_opts *o, const FitArgs<typename PrecTraits<PREC>::R> &fa,
                                 typename PrecTraits<PREC>::R *u, typename PrecTraits<PREC>::R *m1,
-                                typename PrecTraits<PREC>::R *m2, size_t bytes_u, char *saved, int chunk, int group, int *done, cudaStream_t s) {
+                                typename PrecTraits<PREC>::R *m2, size_t bytes_u, char *saved, int chunk, int blocks, int sms, int *done, cudaStream_t s) {
     using R = typename PrecTraits<PREC>::R;
     const bool rules = o->tol > 0 || o->convergence_value > 0;
     const int tiles = (fa.n_list + 31) / 32;
@@ -1173,7 +1189,7 @@ static gac_status fit_uncoupled(const ModelConst &mc, const gac_fit_opts *o, con
         const int count = std::min(chunk, o->iterations - t + 1);
         if (rules && (e = copy_state(true)) != cudaSuccess) return cuda_fail(e, "fit state");
         if ((e = run(t, count)) != cudaSuccess) return cuda_fail(e, "fit updates");
-        if ((e = launch_losses<R>(fa, fa.vloss, group, t, count, s)) != cudaSuccess) return cuda_fail(e, "fit losses");
+        if ((e = launch_losses<R>(fa, fa.vloss, blocks, sms, t, count, s)) != cudaSuccess) return cuda_fail(e, "fit losses");
         *done = t + count - 1;
         if (rules) {
             int flag[2] = {0, 0};  // stop, done
@@ -1295,21 +1311,21 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     cudaError_t e = cudaSuccess;
     int grid = 0, full_grid = 0;
     if ((e = shape(step_ptr<PREC>(mc.kind, l1, false), N, &full_grid)) != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
-    const int group = full_grid * kFitBlock;  // voxels between two of a thread's in the grid's kernel
     const void *fn = nullptr;
     int64_t n_list = 0;
-    size_t bytes_u = 0, bytes_tv = 0, tv_n = 0;
+    size_t bytes_u = 0, bytes_tv = 0, tv_n = 0, n_shares = 0;
     for (;;) {
         n_list = use_list ? n_mask : N;
         fn = step_ptr<PREC>(mc.kind, l1, use_list);
         if ((e = shape(fn, n_list, &grid)) != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
         // work arrays: u (two buffers), Adam moments, the penalised maps over the grid
-        // (two buffers) when there is a list, block losses, history, flags
+        // (two buffers) when there is a list, shares of the losses, history, flags
         bytes_u = (static_cast<size_t>(n_list) * P * RB + 15) / 16 * 16;
         tv_n = use_list && coupled ? static_cast<size_t>(__builtin_popcount(o->tv_params & ((1u << P) - 1u))) * N : 0;
         bytes_tv = (tv_n * RB + 15) / 16 * 16;
-        const size_t total = 4 * bytes_u + 2 * bytes_tv + std::max(grid, kFitLossBlocks * kFitChunk) * sizeof(double) +
-                             static_cast<size_t>(std::max(I, 1)) * sizeof(double) + 3 * sizeof(int);
+        n_shares = many || use_list ? static_cast<size_t>(chunk) * full_grid * kFitWarps : grid;
+        const size_t total = 4 * bytes_u + 2 * bytes_tv + n_shares * sizeof(double) +
+                             static_cast<size_t>(std::max(I, 1)) * sizeof(double) + (3 + kFitChunk) * sizeof(int);
         if (many || use_list) e = vloss.make(static_cast<size_t>(chunk) * N * RB);
         if (e == cudaSuccess && use_list) e = list_masked(d_mask, static_cast<int>(N), n_mask, &list, s);
         if (e == cudaSuccess && use_list) e = cudaMemsetAsync(vloss.p, 0, static_cast<size_t>(chunk) * N * RB, s);
@@ -1329,9 +1345,9 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     R *const m1 = reinterpret_cast<R *>(b + 2 * bytes_u), *const m2 = reinterpret_cast<R *>(b + 3 * bytes_u);
     R *const tv0 = reinterpret_cast<R *>(b + 4 * bytes_u), *const tv1 = reinterpret_cast<R *>(b + 4 * bytes_u + bytes_tv);
     double *block_loss = reinterpret_cast<double *>(b + 4 * bytes_u + 2 * bytes_tv);
-    double *hist = block_loss + std::max(grid, kFitLossBlocks * kFitChunk);
-    int *flags = reinterpret_cast<int *>(hist + std::max(I, 1));  // stop, done, arrival count
-    if ((e = cudaMemsetAsync(flags, 0, 3 * sizeof(int), s)) != cudaSuccess) return cuda_fail(e, "fit memset");
+    double *hist = block_loss + n_shares;
+    int *flags = reinterpret_cast<int *>(hist + std::max(I, 1));  // stop, done, arrival counts
+    if ((e = cudaMemsetAsync(flags, 0, (3 + kFitChunk) * sizeof(int), s)) != cudaSuccess) return cuda_fail(e, "fit memset");
     FitArgs<R> fa;
     std::memset(&fa, 0, sizeof fa);
     fa.data = d_data;
@@ -1373,7 +1389,7 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "theta to u");
     int done = 0;
     if (many) {
-        st = fit_uncoupled<PREC>(mc, o, fa, u0, m1, m2, bytes_u, static_cast<char *>(saved.p), chunk, group, &done, s);
+        st = fit_uncoupled<PREC>(mc, o, fa, u0, m1, m2, bytes_u, static_cast<char *>(saved.p), chunk, full_grid, sms, &done, s);
         if (st != GAC_OK) return st;
     } else {
         if ((e = cudaMemsetAsync(m1, 0, 2 * bytes_u, s)) != cudaSuccess) return cuda_fail(e, "fit memset");
@@ -1393,7 +1409,7 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
                 if ((e = launch_step<R>(fn, grid, smem, s, mc, fa, odd ? u0 : u1, odd ? u1 : u0, m1, m2, R(c1), R(c2), t)) != cudaSuccess)
                     return cuda_fail(e, "fit step");
                 if (use_list && (++unsummed == sum_every || t == t_end)) {
-                    if ((e = launch_losses<R>(fa, shares, group, t - unsummed + 1, unsummed, s)) != cudaSuccess)
+                    if ((e = launch_losses<R>(fa, shares, full_grid, sms, t - unsummed + 1, unsummed, s)) != cudaSuccess)
                         return cuda_fail(e, "fit losses");
                     unsummed = 0;
                 }

@@ -176,3 +176,17 @@ def test_a_fit_runs_in_the_memory_that_a_launch_per_update_needs(fake, name):
     with pytest.raises(fake[0].GacError) as err:
         run(**kw, memory=least - 100_000)
     assert err.value.status == 4 and gpu.in_use == 0
+
+
+@pytest.mark.parametrize("n,updates", [(504, 128), (345_000, 48), (4_000_003, 4), (20_000_000, 1)])
+def test_losses_of_few_updates_are_summed_by_the_whole_gpu(fake, n, updates):
+    """The 64 MB of loss shares hold few updates of a large grid; the launch that sums them fills
+    the SMs all the same."""
+    _, gpu = fake
+    gpu.reset()
+    w = W.MONOEXP_4K.with_(acq=(2.0, 5.0))
+    _fit(fake, w, (n, 1, 1), iterations=2 * updates)
+    losses = [x for x in gpu.launches if x[0].startswith("fit_losses")]
+    assert [x[2] for x in losses] == [updates] * 2
+    for _, grid, count, block, _ in losses:
+        assert grid * count >= min(8 * 152, count * -(-min(n, 97_280) // block))
