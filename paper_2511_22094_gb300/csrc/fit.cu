@@ -1288,8 +1288,18 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     // Stopping rules ask for each loss before the next update, which the grid's
     // kernel gives at no extra launch.
     const bool rules = o->tol > 0 || o->convergence_value > 0;
-    bool many = !coupled;  // many updates a launch
-    bool use_list = d_mask && n_mask < N && (!coupled || (!rules && N > one_round && 5 * n_mask <= 4 * N));
+    // Many updates a launch.  With stopping rules a launch of 32 runs up to 31
+    // updates past the stop and then those before it again, while the grid's
+    // launches after a stop return at once.  In FP32, with at most a voxel a lane of
+    // the persistent warps, that is never slower, wherever the fit stops (ms, grid ->
+    // 32 a launch, stop at update 1, 33, 129 of 200: 3-pool, 97,200 voxels 0.37 ->
+    // 0.35, 0.67 -> 0.58, 1.92 -> 1.25; SMT 0.36 -> 0.25, 0.70 -> 0.39, 2.10 -> 0.83;
+    // mono-exponential, 13,653 voxels 0.35 -> 0.12, 0.36 -> 0.17, 0.93 -> 0.32).  Not so
+    // beyond that (3-pool, 552,960 voxels, stop at 1: 0.48 -> 1.25) and in FP64 (3-pool,
+    // 13,653 voxels: 0.46 -> 6.4, at 33 7.4 -> 12.6).
+    const int64_t n_fit = d_mask ? n_mask : N;
+    bool many = !coupled && (!rules || (PREC == GAC_PREC_FP32 && n_fit <= one_round));
+    bool use_list = d_mask && n_mask < N && (many || (coupled && !rules && N > one_round && 5 * n_mask <= 4 * N));
     // persistent warps, each given the same number of 32-voxel tiles (+-1)
     auto shape = [&](const void *f, int64_t n, int *blocks) {
         cudaError_t c = allow_smem(f, smem);
