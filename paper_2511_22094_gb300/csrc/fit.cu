@@ -1299,6 +1299,12 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     // 13,653 voxels: 0.46 -> 6.4, at 33 7.4 -> 12.6).
     const int64_t n_fit = d_mask ? n_mask : N;
     bool many = !coupled && (!rules || (PREC == GAC_PREC_FP32 && n_fit <= one_round));
+    // One update a launch, where the loss shares of two pass 64 MB, gains nothing
+    // over the grid's kernel, which loads a tile while it computes another, unless
+    // that visits voxels outside the mask (mono-exponential, 16.2 million voxels, 20
+    // updates: 7.7 ms, 9.6 as single updates; 8.4 million, two a launch: 4.14, 4.05).
+    const int64_t held = (int64_t(64) << 20) / (static_cast<int64_t>(RB) * N);  // updates whose shares fit
+    if (held < 2 && 5 * n_fit > 4 * N) many = false;
     bool use_list = d_mask && n_mask < N && (many || (coupled && !rules && N > one_round && 5 * n_mask <= 4 * N));
     // persistent warps, each given the same number of 32-voxel tiles (+-1)
     auto shape = [&](const void *f, int64_t n, int *blocks) {
@@ -1315,7 +1321,7 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     // or one update's) and the state that stopping rules keep are allocated before
     // the first launch; where they, or the work arrays beside them, do not fit,
     // they are given back and the grid's kernel runs, which needs none of them.
-    const int chunk = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(rules ? 32 : kFitChunk, (int64_t(64) << 20) / (static_cast<int64_t>(RB) * N))));
+    const int chunk = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(rules ? 32 : kFitChunk, held)));
     const int I = o->iterations;
     PoolBuf list(s), vloss(s), saved(s), work(s);
     cudaError_t e = cudaSuccess;

@@ -178,7 +178,7 @@ def test_a_fit_runs_in_the_memory_that_a_launch_per_update_needs(fake, name):
     assert err.value.status == 4 and gpu.in_use == 0
 
 
-@pytest.mark.parametrize("n,updates", [(504, 128), (345_000, 48), (4_000_003, 4), (20_000_000, 1)])
+@pytest.mark.parametrize("n,updates", [(504, 128), (345_000, 48), (4_000_003, 4), (8_388_608, 2)])
 def test_losses_of_few_updates_are_summed_by_the_whole_gpu(fake, n, updates):
     """The 64 MB of loss shares hold few updates of a large grid; the launch that sums them fills
     the SMs all the same."""
@@ -204,3 +204,14 @@ def test_stopping_rules_run_few_updates_past_the_stop(fake, precision, n, kernel
             _fit(fake, W.MONOEXP_4K, (n + extra, 1, 1), mask=mask, iterations=33, precision=precision, **rules)
             fits = [x.split("_kernel")[0] for x in gpu.names() if x.startswith(("fit_many", "fit_step", "fit_list"))]
             assert fits == [kernel] * (2 if kernel == "fit_many" else 33)
+
+
+@pytest.mark.parametrize("n,inside,kernel", [(8_388_608, 1.0, "fit_many"), (8_388_609, 1.0, "fit_step"), (8_388_609, 0.5, "fit_many")])
+def test_large_grids_take_the_grids_kernel(fake, n, inside, kernel):
+    """Single updates a launch (the shares of two pass 64 MB) only where they skip voxels."""
+    _, gpu = fake
+    gpu.reset()
+    mask = None if inside == 1.0 else (np.arange(n) % 2).astype(np.uint8)
+    _fit(fake, W.MONOEXP_4K.with_(acq=(2.0, 5.0)), (n, 1, 1), iterations=20, mask=mask)
+    fits = [x.split("_kernel")[0] for x in gpu.names() if x.startswith(("fit_many", "fit_step", "fit_list"))]
+    assert fits == [kernel] * (10 if n == 8_388_608 else 20)
