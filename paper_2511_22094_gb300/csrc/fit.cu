@@ -767,11 +767,10 @@ __global__ void __launch_bounds__(kFitBlock, fit_min_blocks(PREC)) fit_list_kern
     cp_async_wait<0>();
 }
 
-// The stopping rules after iteration t, whose loss is hist[t - 1]: loss < tol, or
-// |least-squares slope of the last `window` losses| < conv_value.
+// The stopping rules after iteration t, whose loss is also hist[t - 1]: loss < tol,
+// or |least-squares slope of the last `window` losses| < conv_value.
 template <class FA>
-__device__ bool fit_halts(const FA &fa, int t) {
-    const double loss = fa.hist[t - 1];
+__device__ bool fit_halts(const FA &fa, int t, double loss) {
     if (fa.tol > 0.0 && loss < fa.tol) return true;
     const int window = fa.window;
     if (fa.conv_value > 0.0 && window > 1 && t >= window) {
@@ -805,7 +804,7 @@ __device__ void fit_check(const FA &fa, int n_blocks, int t, double *red) {
     if (threadIdx.x != 0) return;
     fa.hist[t - 1] = red[0];
     *fa.done = t;
-    if (fit_halts(fa, t)) *fa.stop = 1;
+    if (fit_halts(fa, t, red[0])) *fa.stop = 1;
 }
 
 // ------------------------------------------------ fits without coupling ----
@@ -966,8 +965,11 @@ __global__ void __launch_bounds__(kFitLossThreads) fit_losses_kernel(const FitAr
             __threadfence();
             *fa.arrive = 0u;
             int t = t0;
-            bool halt = fit_halts(fa, t);
-            while (!halt && t < t0 + count - 1) halt = fit_halts(fa, ++t);
+            bool halt = fit_halts(fa, t, fa.hist[t - 1]);
+            while (!halt && t < t0 + count - 1) {
+                ++t;
+                halt = fit_halts(fa, t, fa.hist[t - 1]);
+            }
             *fa.done = t;
             if (halt) *fa.stop = 1;
         }
@@ -1317,12 +1319,12 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
         *blocks = static_cast<int>((tiles + per_warp * kFitWarps - 1) / (per_warp * kFitWarps));
         return c;
     };
+    const int I = o->iterations;
     // The list, the voxels' shares of the losses of `chunk` updates (64 MB at most,
     // or one update's) and the state that stopping rules keep are allocated before
     // the first launch; where they, or the work arrays beside them, do not fit,
     // they are given back and the grid's kernel runs, which needs none of them.
     const int chunk = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(rules ? 32 : kFitChunk, held)));
-    const int I = o->iterations;
     PoolBuf list(s), vloss(s), saved(s), work(s);
     cudaError_t e = cudaSuccess;
     int grid = 0, full_grid = 0;
@@ -1333,7 +1335,8 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     for (;;) {
         n_list = use_list ? n_mask : N;
         fn = step_ptr<PREC>(mc.kind, l1, use_list);
-        if ((e = shape(fn, n_list, &grid)) != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
+        grid = full_grid;
+        if (use_list && !many && (e = shape(fn, n_list, &grid)) != cudaSuccess) return cuda_fail(e, "fit kernel attributes");
         // work arrays: u (two buffers), Adam moments, the penalised maps over the grid
         // (two buffers) when there is a list, shares of the losses, history, flags
         bytes_u = (static_cast<size_t>(n_list) * P * RB + 15) / 16 * 16;
