@@ -215,3 +215,17 @@ def test_large_grids_take_the_grids_kernel(fake, n, inside, kernel):
     _fit(fake, W.MONOEXP_4K.with_(acq=(2.0, 5.0)), (n, 1, 1), iterations=20, mask=mask)
     fits = [x.split("_kernel")[0] for x in gpu.names() if x.startswith(("fit_many", "fit_step", "fit_list"))]
     assert fits == [kernel] * (10 if n == 8_388_608 else 20)
+
+
+@pytest.mark.parametrize("tv", [0.0, 0.1])
+def test_fits_of_few_updates(fake, tv):
+    """One or two updates take the grid's kernel, and the loss shares are sized for the updates
+    there are."""
+    _, gpu = fake
+    n = 128_000
+    for iterations in (1, 2, 3):
+        gpu.reset()
+        _fit(fake, W.MONOEXP_4K, (n, 1, 1), iterations=iterations, mask=(np.arange(n) % 2).astype(np.uint8), tv_lambda=tv,
+             tv_params=1 if tv else 0)
+        assert _count(gpu, "fit_step") == (iterations if iterations < 3 else 0)
+        assert (4 * n * 3 in gpu.sizes) == (iterations == 3)
