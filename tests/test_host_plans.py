@@ -192,10 +192,10 @@ def test_losses_of_few_updates_are_summed_by_the_whole_gpu(fake, n, updates):
         assert grid * count >= min(8 * 152, count * -(-min(n, 97_280) // block))
 
 
-@pytest.mark.parametrize("precision,n,kernel", [(1, 97_280, "fit_many"), (1, 97_281, "fit_step"), (2, 100, "fit_step")])
+@pytest.mark.parametrize("precision,n,kernel", [(1, 72_960, "fit_many"), (1, 72_961, "fit_step"), (2, 100, "fit_step")])
 def test_stopping_rules_run_few_updates_past_the_stop(fake, precision, n, kernel):
     """A launch of many updates runs past a stop: only where that costs less than the idle launches
-    it saves, in FP32 with at most one tile a warp."""
+    it saves, in FP32 with a tile for at most three warps of four."""
     _, gpu = fake
     for rules in (dict(tol=1e-300), dict(convergence_value=1e-300)):
         for extra in (0, 1000):  # voxels outside the mask
