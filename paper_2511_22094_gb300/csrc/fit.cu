@@ -818,7 +818,7 @@ __device__ void fit_check(const FA &fa, int n_blocks, int t, double *red) {
 // updates 1.70 -> 0.22 ms; 3-pool, 96 x 96 x 60, 100 updates 5.6 -> 3.3 ms, with
 // a mask of 68% of it 5.7 -> 2.4 ms.
 constexpr int kFitChunk = 128;
-constexpr int kFitLossThreads = 256;
+constexpr int kFitLossThreads = 128;
 
 template <class R>
 struct FitSteps {
@@ -911,78 +911,140 @@ __global__ void __launch_bounds__(32, PREC == GAC_PREC_FP32 ? 20 : 8)
 // The losses of `count` updates from the voxels' shares (fa.vloss), summed in the
 // order of fit_step_kernel on `blocks` blocks, so that a loss and what the
 // stopping rules make of it are the same bits on every path: a lane adds its
-// voxels v, v + 32 warps, ... in the kernel's precision, a warp its lanes in FP64,
-// then four warps make a block's share and the blocks' shares are added as
-// fit_check does.  blockIdx.y: the update; its last block adds the shares and
-// records the loss, and the last update's applies the stopping rules to each in
-// turn.  Bound by the reads, which come from L2 (about 0.5 us an update of 552,960
-// voxels) or, with few updates a launch, from HBM: the blocks then fill the GPU.
-// (24 blocks for a single update of 16 million voxels read at 100 GB/s.)
+// voxels v, v + 32 warps, ... in the kernel's precision, a warp its lanes in FP64
+// by the shuffles' tree, then four warps make a block's share and the blocks'
+// shares are added as fit_check does.  blockIdx.y: the update; its last block adds
+// the shares and records the loss, and the last update's applies the stopping
+// rules to each in turn.
+//
+// Bound by FP64 issue where the updates are many: the shuffles' tree takes a warp
+// five additions and a conversion for 32 shares (13,653 voxels x 128 updates: 20
+// us), so a warp takes eight of the grid kernel's warps at once and halves the
+// number it works on with every step of the tree, two additions and conversions
+// for 32 shares.  Few updates have too few such groups: bound by the reads, they
+// take the warps one by one, and the blocks fill the GPU (24 blocks for one update
+// of 16 million voxels read at 100 GB/s).
 template <class R>
-__global__ void __launch_bounds__(kFitLossThreads) fit_losses_kernel(const FitArgs<R> fa, const R *vloss, int blocks, int t0, int count) {
-    __shared__ double red[kFitBlock];
-    __shared__ bool last;
-    if (*fa.stop) return;  // the same for every thread; only this kernel's last block sets it
-    const int tid = threadIdx.x, lane = tid & 31, k = blockIdx.y;
-    const int warps = blocks * kFitWarps;
-    const R *x = vloss + k * fa.n;
-    double *sums = fa.block_loss + static_cast<int64_t>(k) * warps;
-    for (int w = blockIdx.x * (kFitLossThreads / 32) + (tid >> 5); w < warps; w += gridDim.x * (kFitLossThreads / 32)) {
+__device__ __forceinline__ void fit_warp_sums_few(const R *x, int64_t n, int warps, double *sums) {
+    const int lane = threadIdx.x & 31;
+    for (int w = blockIdx.x * kFitWarps + (threadIdx.x >> 5); w < warps; w += gridDim.x * kFitWarps) {
         R s = R(0);
 #pragma unroll 8
-        for (int64_t v = w * 32 + lane; v < fa.n; v += warps * 32) s += x[v];
+        for (int64_t v = w * 32 + lane; v < n; v += warps * 32) s += x[v];
         double sum = static_cast<double>(s);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
         if (lane == 0) sums[w] = sum;
     }
-    __threadfence();  // the sums are visible before the count says so
-    __syncthreads();
-    if (tid == 0) last = atomicAdd(fa.arrive + 1 + k, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    if (tid < kFitBlock) {
-        double s = 0.0;
-        for (int b = tid; b < blocks; b += kFitBlock) {
-            double t = 0.0;
-#pragma unroll
-            for (int i = 0; i < kFitWarps; ++i) t += __ldcg(sums + b * kFitWarps + i);
-            s += t;
-        }
-        red[tid] = s;
-    }
-    __syncthreads();
-    for (int n = kFitBlock / 2; n > 0; n >>= 1) {
-        if (tid < n) red[tid] += red[tid + n];
-        __syncthreads();
-    }
-    if (tid == 0) {
-        fa.hist[t0 - 1 + k] = red[0];
-        fa.arrive[1 + k] = 0u;
-        __threadfence();
-        if (atomicAdd(fa.arrive, 1u) == static_cast<unsigned>(count - 1)) {
-            __threadfence();
-            *fa.arrive = 0u;
-            int t = t0;
-            bool halt = fit_halts(fa, t, fa.hist[t - 1]);
-            while (!halt && t < t0 + count - 1) {
-                ++t;
-                halt = fit_halts(fa, t, fa.hist[t - 1]);
-            }
-            *fa.done = t;
-            if (halt) *fa.stop = 1;
-        }
-    }
 }
 
 template <class R>
+__device__ __forceinline__ void fit_warp_sums_many(const R *x, int64_t n, int warps, double *sums) {
+    const int lane = threadIdx.x & 31;
+    for (int w = 8 * (blockIdx.x * kFitWarps + (threadIdx.x >> 5)); w < warps; w += 8 * gridDim.x * kFitWarps) {
+        R s[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s[i] = R(0);
+        for (int64_t v = w * 32; v < n; v += warps * 32) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int64_t at = v + 32 * i + lane;
+                s[i] += w + i < warps && at < n ? x[at] : R(0);
+            }
+        }
+        // one step of the tree: a lane keeps one of two sets of sums, its partner the other
+        auto step = [&](auto keep_lo, auto keep_hi, int o) {
+            const bool hi = lane & o;
+            const auto give = hi ? keep_lo : keep_hi, keep = hi ? keep_hi : keep_lo;
+            return static_cast<double>(keep) + static_cast<double>(__shfl_xor_sync(0xffffffffu, give, o));
+        };
+        double t[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) t[i] = step(s[i], s[i + 4], 16);
+        double u = step(step(t[0], t[2], 8), step(t[1], t[3], 8), 4);
+        u += __shfl_xor_sync(0xffffffffu, u, 2);
+        u += __shfl_xor_sync(0xffffffffu, u, 1);
+        if ((lane & 3) == 0 && w + (lane >> 2) < warps) sums[w + (lane >> 2)] = u;
+    }
+}
+
+template <class R, bool FEW>
+__global__ void __launch_bounds__(kFitLossThreads) fit_losses_kernel(const FitArgs<R> fa, const R *vloss, int blocks, int t0, int count) {
+    __shared__ double red[kFitBlock];
+    __shared__ bool last;
+    if (*fa.stop) return;  // the same for every thread; only this kernel's last block sets it
+    const int tid = threadIdx.x, k = blockIdx.y;
+    const int warps = blocks * kFitWarps;
+    const R *x = vloss + k * fa.n;
+    double *sums = fa.block_loss + static_cast<int64_t>(k) * warps;
+    if constexpr (FEW) fit_warp_sums_few(x, fa.n, warps, sums);
+    else fit_warp_sums_many(x, fa.n, warps, sums);
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();  // the block's sums are visible before the count says so
+        last = atomicAdd(fa.arrive + 1 + k, 1u) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    double s = 0.0;
+    for (int b = tid; b < blocks; b += kFitBlock) {
+        double t = 0.0;
+#pragma unroll
+        for (int i = 0; i < kFitWarps; ++i) t += __ldcg(sums + b * kFitWarps + i);
+        s += t;
+    }
+    red[tid] = s;
+    __syncthreads();
+    if (tid >= 32) return;
+    s = (red[tid] + red[tid + 64]) + (red[tid + 32] + red[tid + 96]);  // fit_check's tree
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    const bool rules = fa.tol > 0.0 || fa.conv_value > 0.0;
+    unsigned summed = 0;  // updates before this one
+    if (tid == 0) {
+        fa.hist[t0 - 1 + k] = s;
+        fa.arrive[1 + k] = 0u;
+        if (rules) {
+            __threadfence();
+            summed = atomicAdd(fa.arrive, 1u);
+            __threadfence();
+        } else if (k == count - 1) {
+            *fa.done = t0 + k;
+        }
+    }
+    if (!rules || __shfl_sync(0xffffffffu, summed, 0) != static_cast<unsigned>(count - 1)) return;
+    int t = t0 - 1, halt = 0;
+    for (int i0 = 0; i0 < count && !halt; i0 += 32) {  // 32 losses read at once
+        const double loss = i0 + tid < count ? __ldcg(fa.hist + t0 - 1 + i0 + tid) : 0.0;
+        for (int i = 0; i < min(32, count - i0) && !halt; ++i) {
+            ++t;
+            const double li = __shfl_sync(0xffffffffu, loss, i);
+            if (tid == 0) halt = fit_halts(fa, t, li);
+            halt = __shfl_sync(0xffffffffu, halt, 0);
+        }
+    }
+    if (tid == 0) {
+        *fa.arrive = 0u;
+        *fa.done = t;
+        if (halt) *fa.stop = 1;
+    }
+}
+
+static_assert(kFitLossThreads == kFitBlock && kFitBlock == 128, "fit_losses_kernel adds the shares as fit_check's block does");
+template <class R>
 static cudaError_t launch_losses(const FitArgs<R> &fa, const R *vloss, int blocks, int sms, int t0, int count, cudaStream_t s) {
-    // 16 sums a lane (every block ends with an atomic), or fewer where a launch of few
-    // updates would leave SMs idle
-    const int all = (blocks * kFitWarps * 32 + kFitLossThreads - 1) / kFitLossThreads;
-    const int nb = std::min(all, std::max((all + 15) / 16, (8 * sms + count - 1) / count));
-    fit_losses_kernel<R><<<dim3(nb, count), kFitLossThreads, 0, s>>>(fa, vloss, blocks, t0, count);
+    // groups of eight warps, at most two a warp (every block ends with an atomic), where
+    // they are enough to hide the reads
+    const int groups = (blocks * kFitWarps + 7) / 8;
+    if (groups * count >= 8 * sms) {
+        const int per_block = (groups * count >= 16 * sms ? 2 : 1) * kFitWarps;
+        const int nb = (groups + per_block - 1) / per_block;
+        fit_losses_kernel<R, false><<<dim3(nb, count), kFitLossThreads, 0, s>>>(fa, vloss, blocks, t0, count);
+    } else {
+        const int nb = std::min(blocks, (8 * sms + count - 1) / count);
+        fit_losses_kernel<R, true><<<dim3(nb, count), kFitLossThreads, 0, s>>>(fa, vloss, blocks, t0, count);
+    }
     return cudaGetLastError();
 }
 

@@ -189,7 +189,7 @@ def test_losses_of_few_updates_are_summed_by_the_whole_gpu(fake, n, updates):
     losses = [x for x in gpu.launches if x[0].startswith("fit_losses")]
     assert [x[2] for x in losses] == [updates] * 2
     for _, grid, count, block, _ in losses:
-        assert grid * count >= min(8 * 152, count * -(-min(n, 97_280) // block))
+        assert grid * count * block // 32 >= min(8 * 152, n)
 
 
 @pytest.mark.parametrize("precision,n,kernel", [(1, 72_960, "fit_many"), (1, 72_961, "fit_step"), (2, 100, "fit_step")])
