@@ -838,7 +838,8 @@ __device__ __forceinline__ void ax_phi_table_f(float R, const AxConst &ax, float
 // and the measurement's index come from the kernel parameters (the same address
 // for every thread: no shared-memory wavefronts, of which the table lookups
 // leave few; 24.6 -> 23.5 ms for 25,001 voxels x 4 x 5,000).  A full block's
-// lookups overlap, and so do those of a pair of the rest.
+// lookups overlap; those of a partial one come one by one (in pairs, 16
+// measurements ran 1% slower and 7 in blocks of four and three 3%).
 template <bool TAIL, int REP, class V>
 __device__ __forceinline__ void eval_axcal_f(const float *th, const ModelConst &mc, V &&visit) {
     const AxConst &ax = mc.ax;
@@ -866,11 +867,7 @@ __device__ __forceinline__ void eval_axcal_f(const float *th, const ModelConst &
                 for (int k = 0; k < kAnchor; ++k) one(i0 + k);
                 i = i1;
             }
-            for (; i + 1 < i1; i += 2) {
-                one(i);
-                one(i + 1);
-            }
-            if (i < i1) one(i);
+            for (; i < i1; ++i) one(i);
             end_block(visit, 0);
         }
     }
