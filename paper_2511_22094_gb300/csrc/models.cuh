@@ -722,12 +722,21 @@ __device__ __forceinline__ void eval_smt_blocks_f(const float *th, const ModelCo
         else one(k);
     };
     // a full block has no test between its b-values, so their table lookups
-    // overlap; a protocol of one block reads them at fixed offsets; only a
-    // last, partial block tests
+    // overlap; a protocol of one block, full or not, reads them at fixed offsets
+    // (without it, four b-values, 19,000 chains: 0.71 -> 0.78 us an iteration); only
+    // a partial block tests
     if (n == kAnchor) {
         first(0);
 #pragma unroll
         for (int k = 1; k < kAnchor; ++k) one(k);
+        end_block(visit, 0);
+        return;
+    }
+    if (n < kAnchor) {
+        first(0);
+#pragma unroll
+        for (int k = 1; k < kAnchor; ++k)
+            if (k < n) one(k);
         end_block(visit, 0);
         return;
     }
