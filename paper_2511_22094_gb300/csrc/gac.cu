@@ -643,8 +643,13 @@ gac_status validate_opts(const gac_mcmc_opts *o, int64_t n_vox) {
 // library uses it for the mono-exponential model when the chains would give
 // fewer than one warp per SM sub-partition (there it shortens the latency of an
 // iteration; on larger problems one thread per chain keeps more chains in
-// flight); the 3-pool model runs faster on the speculative kernel or, from
-// about 12,000 chains, one thread per chain (1.30 against 2.35 us an iteration).
+// flight).  The 3-pool model takes it with 7 to 12 echoes, two lanes a chain, where
+// trees of depth 2 would put a second warp on a scheduler and thinning is so far
+// apart that the lanes' own FP64 moment updates weigh little (12 echoes, us an iteration, split against depth 2 at
+// 9,600 chains and against one thread at 14,400: thinning 100 0.68 and 0.77, 0.96
+// and 1.02; thinning 5 1.06 and 0.91, 1.36 and 1.37; moments over every state 1.42
+// and 1.08, 1.50 and 1.20); with more echoes, four lanes a chain, it lost to both
+// (24 echoes, 14,400 chains: 2.35 against 1.30 one thread per chain).
 static gac_status choose_lanes(const ModelConst &mc, const gac_mcmc_opts *o, int64_t n_vox, int *lanes) {
     const int nb = (mc.n_acq + kAnchor - 1) / kAnchor;
     const bool eligible = o->precision == GAC_PREC_MIXED && o->trace_n_vox == 0 && mc.even &&
@@ -660,8 +665,16 @@ static gac_status choose_lanes(const ModelConst &mc, const gac_mcmc_opts *o, int
         *lanes = o->lanes_per_chain;
         return GAC_OK;
     }
-    const int64_t one_warp_each = static_cast<int64_t>(sm_count()) * 4 * 32;
-    if (eligible && mc.kind == GAC_MODEL_MONOEXP && n_vox * o->n_chains < one_warp_each) *lanes = nb <= 2 ? 2 : 4;
+    const int64_t one_warp_each = static_cast<int64_t>(sm_count()) * 4 * 32, chains = n_vox * o->n_chains;
+    if (!eligible || chains >= one_warp_each) return GAC_OK;
+    if (mc.kind == GAC_MODEL_MONOEXP) {
+        *lanes = nb <= 2 ? 2 : 4;
+    } else if (nb == 2 && 4 * chains > one_warp_each && o->moments_mode == GAC_MOMENTS_THINNED) {
+        // the thinning from which it wins, by the kernel it replaces: depth 2; one
+        // thread, with at most one and a half split warps a scheduler; with two
+        const int least = 2 * chains <= one_warp_each ? 12 : 4 * chains <= 3 * one_warp_each ? 3 : 8;
+        if (o->thin >= least) *lanes = 2;
+    }
     return GAC_OK;
 }
 
@@ -747,7 +760,12 @@ static SpecShape spec_shape(int depth, int C, int64_t n_vox) {
 // (`split`) past two warps a scheduler at depth 4; with thinning of 4 or less,
 // where that kernel's own moment updates weigh, past two at depth 3 (2,000
 // iterations of 4,096 chains, thinning 2: 0.76 ms split, 0.62; thinning 5: 0.51
-// both).
+// both).  Where it does not apply (one block of echoes, uneven echoes, more than
+// four blocks), depth 2 pays up to three warps a scheduler, and up to four where one
+// thread's likelihood takes long for its echoes (us an iteration, one thread ->
+// depth 2, at 19,000 chains: 2 echoes 0.37 -> 0.40, 6 echoes 0.46 -> 0.42, 12 uneven
+// ones 0.72 -> 0.64, 26 echoes 0.53 -> 0.55, 32 0.59 -> 0.59, 64 0.85 -> 0.76) or
+// moments are taken often (thinning 1, 2 echoes: 1.04 -> 0.85).
 static int choose_depth(const ModelConst &mc, const gac_mcmc_opts *o, int64_t n_vox, bool split) {
     if (o->precision != GAC_PREC_MIXED || o->trace_n_vox != 0 || o->lanes_per_chain != 0 ||
         !mh_spec_ptr(mc.kind, 2, false))
@@ -756,6 +774,7 @@ static int choose_depth(const ModelConst &mc, const gac_mcmc_opts *o, int64_t n_
     const int64_t schedulers = static_cast<int64_t>(sm_count()) * 4;
     const bool mwi3 = mc.kind == GAC_MODEL_MWI3, mono = mc.kind == GAC_MODEL_MONOEXP;
     const bool all = o->moments_mode == GAC_MOMENTS_ALL_POSTBURNIN;
+    const bool mono4 = !mc.even || mc.n_acq == kAnchor || mc.n_acq >= 48 || (!all && o->thin <= 4);
     for (int depth = 5; depth >= 2; --depth) {
         if (C << depth > kSpecBlock || n_vox * C > (schedulers * 32 * 4 >> depth)) continue;
         // warps a scheduler
@@ -763,8 +782,8 @@ static int choose_depth(const ModelConst &mc, const gac_mcmc_opts *o, int64_t n_
                         : depth == 4 ? (mono && !all ? 2 : 1)
                         : depth == 3 ? (mwi3 ? 1 : 2)
                         : mwi3       ? 2
-                        : mc.kind == GAC_MODEL_SMT ? 3 : 4;
-        if (mono && split && (depth == 2 || (depth == 3 && (all || o->thin > 4)))) return 0;
+                        : mc.kind == GAC_MODEL_SMT || (mono && !mono4) ? 3 : 4;
+        if (split && (depth == 2 || (mono && depth == 3 && (all || o->thin > 4)))) return 0;
         if (spec_shape(depth, C, n_vox).warps() <= per * schedulers) return depth;
     }
     return 0;

@@ -19,7 +19,7 @@ OOM = 2  # cudaErrorMemoryAllocation
 HOOK = ct.CFUNCTYPE(ct.c_int, ct.c_char_p, ct.c_char_p, ct.POINTER(ct.c_longlong), ct.POINTER(ct.c_void_p))
 
 #: resident blocks an SM that the kernels' registers allow (launch bounds; shared memory on top)
-RESIDENT = [(r"mh(_slice)?_kernel<(2|4),", 2), (r"mh(_slice)?_kernel<3,", 4), (r"mh_kernel", 3), (r"mh_spec_kernel<\d,2,", 2),
+RESIDENT = [(r"mh(_slice)?_kernel<(2|4),", 2), (r"mh(_slice)?_kernel<3,", 4), (r"mh_kernel", 4), (r"mh_spec_kernel<\d,2,", 2),
             (r"mh_split|mh_spec", 1), (r"fit_many_kernel<\d+,1", 20), (r"fit_(step|list)_kernel<\d+,1", 5), (r"", 2)]
 
 

@@ -229,3 +229,66 @@ def test_fits_of_few_updates(fake, tv):
              tv_params=1 if tv else 0)
         assert _count(gpu, "fit_step") == (iterations if iterations < 3 else 0)
         assert (4 * n * 3 in gpu.sizes) == (iterations == 3)
+
+
+def _spec_cases():
+    from test_gpu_spec import CASES
+    return [pytest.param(name, *c, id=name) for name, c in CASES.items()]
+
+
+@pytest.mark.parametrize("name,base,acq,n,C,kw", _spec_cases())
+def test_speculative_cases_run_the_tree_they_name(fake, name, base, acq, n, C, kw):
+    _, gpu = fake
+    gpu.reset()
+    _sampler(fake, base.with_(acq=tuple(acq)), n, C, **kw)
+    depth = int(name.split("-d")[1][0])
+    if name == "axcal-d4-adapt":  # 999 chains, three a voxel: 666 warps at depth 4 (a case of 4: test_gpu_routes.py)
+        depth = 3
+    assert gpu.names() == [f"mh_spec_kernel<{base.kind},{depth},{kw.get('moments_mode', 0)}>"]
+
+
+def test_slice_and_tile_cases_run_slices_and_half_blocks(fake):
+    """The sizes that the bit-equality tests of those kernels choose do reach them."""
+    import test_gpu_slices
+    import test_gpu_tiles
+    _, gpu = fake
+    for w, n, C, kw in test_gpu_slices.CASES:
+        gpu.reset()
+        _sampler(fake, w, n, C, **kw)
+        assert set(gpu.names()) == {f"mh_slice_kernel<{w.kind}>"} and len(gpu.names()) > 2
+    half = []
+    for w, n, C in test_gpu_tiles.CASES:
+        gpu.reset()
+        _sampler(fake, w, n, C, iterations=24, burnin=12, thin=3, lanes_per_chain=1)
+        half.append(gpu.names() == [f"mh_kernel<{w.kind},0,0,128>"])
+    assert sum(half) >= len(half) - 1
+
+
+#: workload, echoes or b-values, chains, thinning, moments over every state -> kernel
+ROUTES = [
+    # 3-pool, two blocks of echoes: two lanes a chain where moments are rare
+    ("mwi3", 12, 4864, 100, 0, "mh_spec_kernel<2,2,0>"), ("mwi3", 12, 5000, 100, 0, "mh_split_kernel<2,2,0>"),
+    ("mwi3", 12, 9728, 12, 0, "mh_split_kernel<2,2,0>"), ("mwi3", 12, 9728, 11, 0, "mh_spec_kernel<2,2,0>"),
+    ("mwi3", 7, 14_000, 3, 0, "mh_split_kernel<2,2,0>"), ("mwi3", 12, 14_000, 2, 0, "mh_kernel<2,0,0,128>"),
+    ("mwi3", 12, 19_000, 8, 0, "mh_split_kernel<2,2,0>"), ("mwi3", 12, 19_000, 7, 0, "mh_kernel<2,0,0,128>"),
+    ("mwi3", 12, 9728, 100, 1, "mh_spec_kernel<2,2,1>"), ("mwi3", 13, 9728, 100, 0, "mh_spec_kernel<2,2,0>"),
+    ("mwi3", 24, 14_000, 100, 0, "mh_kernel<2,0,0,128>"),
+    # mono-exponential where the lane-split kernel does not apply: four warps a scheduler or three
+    ("monoexp", 6, 19_000, 100, 0, "mh_spec_kernel<1,2,0>"), ("monoexp", 5, 19_000, 100, 0, "mh_kernel<1,0,0,128>"),
+    ("monoexp", 5, 14_000, 100, 0, "mh_spec_kernel<1,2,0>"), ("monoexp", 5, 19_000, 4, 0, "mh_spec_kernel<1,2,0>"),
+    ("monoexp", 30, 19_000, 100, 1, "mh_kernel<1,0,0,128>"), ("monoexp", 48, 19_000, 100, 0, "mh_spec_kernel<1,2,0>"),
+    # the lane-split kernel, and trees with short thinning
+    ("monoexp", 12, 2400, 3, 0, "mh_spec_kernel<1,4,0>"), ("monoexp", 12, 4800, 4, 0, "mh_spec_kernel<1,3,0>"),
+    ("monoexp", 12, 4096, 5, 0, "mh_split_kernel<1,2,0>"), ("monoexp", 24, 9600, 5, 0, "mh_split_kernel<1,4,0>"),
+]
+
+
+@pytest.mark.parametrize("model,k,n,thin,every,kernel", ROUTES)
+def test_routes(fake, model, k, n, thin, every, kernel):
+    _, gpu = fake
+    w = {"monoexp": W.MONOEXP_4K, "mwi3": W.MWI3_1M, "smt": W.SMT_1P5M}[model]
+    if k != len(w.acq):
+        w = w.with_(acq=tuple(2.0 + 0.7 * np.arange(k)))
+    gpu.reset()
+    _sampler(fake, w, n, 1, iterations=200, burnin=0, thin=thin, moments_mode=every)
+    assert gpu.names() == [kernel]
