@@ -496,7 +496,10 @@ static gac_status plan_launch(const ModelConst &mc, int prec, bool trace, int C,
         // of four warps load them evenly, while two blocks of eight with
         // some idle warps, or a last wave of few large blocks, leave
         // schedulers with twice the warps of others.  Full waves of half
-        // blocks measured up to 3% slower (1.03).  3-pool, us per iteration,
+        // blocks measured up to 3% slower (1.03); where an SM holds more than two of
+        // kBlock, whose ends then spread of themselves, they have to promise 5.5%
+        // (mono-exponential, kBlock -> kHalfBlock: 240,000 chains, 2.2% promised,
+        // 2.39 -> 2.46; 200,000, 5.8%, 2.14 -> 2.02).  3-pool, us per iteration,
         // kBlock -> kHalfBlock: 14,400 chains 1.79 -> 1.31, 49,380 3.12 ->
         // 2.51, 120,000 6.09 -> 5.24, 200,000 9.01 -> 8.05.  Below one block
         // an SM, tiles shrink in whole warps of chains: each scheduler gets at
@@ -507,14 +510,15 @@ static gac_status plan_launch(const ModelConst &mc, int prec, bool trace, int C,
         half_per_sm = std::min(half_per_sm, 2 * per_sm);  // as many warps: 20 instead of 16 ran 2% slower (3-pool)
         const int vb1 = std::max(1, kBlock / C), vb2 = std::max(1, kHalfBlock / C);
         const double t1 = waves((n_vox + vb1 - 1) / vb1, per_sm);
-        const double t2 = 1.03 * waves((n_vox + vb2 - 1) / vb2, half_per_sm);
+        const double t2 = (per_sm > 2 ? 1.055 : 1.03) * waves((n_vox + vb2 - 1) / vb2, half_per_sm);
         const int64_t want = (chains + sm_count() - 1) / sm_count();  // chains an SM
         if (t2 < t1 || want <= kHalfBlock) {
             *cfg = half;
             per_sm = half_per_sm;
             threads = static_cast<int>(std::min<int64_t>(kHalfBlock, (want + 31) / 32 * 32));
         }
-    } else if (chains < resident * kBlock) {
+    }
+    if (cfg->block == kBlock && chains < resident * kBlock) {
         // too few chains for a full tile per resident block: tiles shrink in
         // whole warps of chains, so that the chains spread over all SMs
         const int64_t want = (chains + resident - 1) / resident;  // chains per block

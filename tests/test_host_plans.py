@@ -280,6 +280,10 @@ ROUTES = [
     # the lane-split kernel, and trees with short thinning
     ("monoexp", 12, 2400, 3, 0, "mh_spec_kernel<1,4,0>"), ("monoexp", 12, 4800, 4, 0, "mh_spec_kernel<1,3,0>"),
     ("monoexp", 12, 4096, 5, 0, "mh_split_kernel<1,2,0>"), ("monoexp", 24, 9600, 5, 0, "mh_split_kernel<1,4,0>"),
+    # blocks of 128 past one block an SM where the waves promise enough
+    ("monoexp", 12, 200_000, 100, 0, "mh_kernel<1,0,0,128>"), ("monoexp", 12, 240_000, 100, 0, "mh_kernel<1,0,0,256>"),
+    ("monoexp", 12, 400_000, 100, 0, "mh_kernel<1,0,0,256>"), ("smt", 6, 200_000, 100, 0, "mh_kernel<3,0,0,128>"),
+    ("mwi3", 24, 200_000, 100, 0, "mh_kernel<2,0,0,128>"),
 ]
 
 
@@ -292,3 +296,13 @@ def test_routes(fake, model, k, n, thin, every, kernel):
     gpu.reset()
     _sampler(fake, w, n, 1, iterations=200, burnin=0, thin=thin, moments_mode=every)
     assert gpu.names() == [kernel]
+
+
+def test_tiles_reach_every_sm(fake):
+    """Full blocks that are too few for a wave shrink to whole warps of chains."""
+    _, gpu = fake
+    for n in (20_000, 24_000, 33_000, 38_000, 60_000):
+        for prec in (0, 1):
+            gpu.reset()
+            _sampler(fake, W.MONOEXP_4K, n, 1, iterations=20, burnin=0, thin=5, precision=prec, lanes_per_chain=1)
+            assert gpu.launches[0][1] >= 152
