@@ -153,11 +153,20 @@ static cudaError_t launch_forward(int prec, const ModelConst &mc, const double *
     const int row_stride = row_stride_for(KIND, std::max(mc.n_meas, mc.n_par));
     const size_t smem = static_cast<size_t>(kFwdBlock) * row_stride * sizeof(float);
     if (smem > 44 * 1024) {  // beside the model's tables, past the default 48 KB
-        const cudaError_t e = allow_smem(reinterpret_cast<const void *>(&forward_f_kernel<KIND>), smem);
-        if (e != cudaSuccess) return e;
+        const cudaError_t lim = allow_smem(reinterpret_cast<const void *>(&forward_f_kernel<KIND>), smem);
+        if (lim != cudaSuccess) return lim;
     }
+    // one wave: 8 blocks an SM, or as many as its shared memory holds (long rows, the
+    // models' tables and the system's kilobyte)
+    constexpr int kBeside = KIND == GAC_MODEL_SMT || KIND == GAC_MODEL_AXCAL_SMT ? 6 * 1024 : 1024;
+    int dev = 0, sms = 0, smem_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    if (e != cudaSuccess) return e;
+    const int64_t per_sm = std::min<int64_t>(8, std::max<int64_t>(1, smem_sm / static_cast<int64_t>(smem + kBeside)));
     const int64_t blocks = (n + kFwdBlock - 1) / kFwdBlock;
-    const int grid = static_cast<int>(std::min<int64_t>(blocks, 152 * 8));  // 8 blocks on each SM: one wave
+    const int grid = static_cast<int>(std::min<int64_t>(blocks, sms * per_sm));
     forward_f_kernel<KIND><<<grid, kFwdBlock, smem, st>>>(mc, th, n, s, row_stride);
     return cudaGetLastError();
 }

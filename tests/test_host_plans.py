@@ -306,3 +306,14 @@ def test_tiles_reach_every_sm(fake):
             gpu.reset()
             _sampler(fake, W.MONOEXP_4K, n, 1, iterations=20, burnin=0, thin=5, precision=prec, lanes_per_chain=1)
             assert gpu.launches[0][1] >= 152
+
+
+@pytest.mark.parametrize("n_acq,per_sm", [(6, 8), (24, 8), (48, 4), (64, 3)])
+def test_forward_rows_are_one_wave(fake, n_acq, per_sm):
+    _, gpu = fake
+    gpu.reset()
+    _forward(fake, n_acq, 300_000)
+    assert gpu.launches[-1][:2] == ("forward_f_kernel<2>", 152 * per_sm)
+    gpu.reset()
+    _forward(fake, n_acq, 129)
+    assert gpu.launches[-1][1] == 2
