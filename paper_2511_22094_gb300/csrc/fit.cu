@@ -1349,6 +1349,8 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     //         1,000,000  5.02 -> 3.69 5.32 -> 4.61 5.38 -> 5.06 5.40 -> 5.67 5.40 -> 5.74
     //   SMT     552,960  2.01 -> 1.42 2.04 -> 1.62 2.04 -> 1.88 2.05 -> 2.15 2.05 -> 2.16
     //   mono    552,960  1.28 -> 0.93 1.31 -> 1.07 1.30 -> 1.21 1.31 -> 1.33 1.32 -> 1.36
+    // It costs a call a few launches, which three updates earn back (mono-exponential,
+    // 552,960 voxels, 60% inside: one update 0.173 -> 0.188 ms, three 0.207 -> 0.201).
     const int64_t one_round = static_cast<int64_t>(sms) * kFitMinBlocks32 * kFitWarps * 32;
     // Stopping rules ask for each loss before the next update, which the grid's
     // kernel gives at no extra launch.
@@ -1370,12 +1372,11 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     // updates: 7.7 ms, 9.6 as single updates; 8.4 million, two a launch: 4.14, 4.05).
     const int64_t held = (int64_t(64) << 20) / (static_cast<int64_t>(RB) * N);  // updates whose shares fit
     if (held < 2 && 5 * n_fit > 4 * N) many = false;
-    // The list and the shares cost a call a few launches, which three updates earn
-    // back (mono-exponential, 552,960 voxels, 60% inside, total variation: one update
-    // 0.173 ms on the grid, 0.188 on the list; three 0.207 and 0.201).
-    const bool few = I < 3;
-    if (few) many = false;
-    bool use_list = d_mask && n_mask < N && (many || (coupled && !rules && !few && N > one_round && 5 * n_mask <= 4 * N));
+    // A single update of many voxels does not earn back the second launch (SMT,
+    // 552,960 voxels: 0.199 ms on the grid, 0.209; 10 x 10 mono-exponential ones 0.095,
+    // 0.063: the grid's launches end with two waits of the host).
+    if (I == 1 && n_fit > one_round) many = false;
+    bool use_list = d_mask && n_mask < N && (many || (coupled && !rules && I >= 3 && N > one_round && 5 * n_mask <= 4 * N));
     // persistent warps, each given the same number of 32-voxel tiles (+-1)
     auto shape = [&](const void *f, int64_t n, int *blocks) {
         cudaError_t c = allow_smem(f, smem);

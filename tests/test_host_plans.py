@@ -217,18 +217,18 @@ def test_large_grids_take_the_grids_kernel(fake, n, inside, kernel):
     assert fits == [kernel] * (10 if n == 8_388_608 else 20)
 
 
-@pytest.mark.parametrize("tv", [0.0, 0.1])
-def test_fits_of_few_updates(fake, tv):
-    """One or two updates take the grid's kernel, and the loss shares are sized for the updates
-    there are."""
+@pytest.mark.parametrize("tv,n,many_from", [(0.0, 1000, 1), (0.0, 128_000, 2), (0.1, 128_000, 3)])
+def test_fits_of_few_updates(fake, tv, n, many_from):
+    """One update of many voxels and one or two with a list take the grid's kernel, and the loss
+    shares are sized for the updates there are."""
     _, gpu = fake
-    n = 128_000
+    mask = (np.arange(n) % 5 > 0).astype(np.uint8)
     for iterations in (1, 2, 3):
         gpu.reset()
-        _fit(fake, W.MONOEXP_4K, (n, 1, 1), iterations=iterations, mask=(np.arange(n) % 2).astype(np.uint8), tv_lambda=tv,
-             tv_params=1 if tv else 0)
-        assert _count(gpu, "fit_step") == (iterations if iterations < 3 else 0)
-        assert (4 * n * 3 in gpu.sizes) == (iterations == 3)
+        _fit(fake, W.MONOEXP_4K, (n, 1, 1), iterations=iterations, mask=mask, tv_lambda=tv, tv_params=1 if tv else 0)
+        assert _count(gpu, "fit_step") == (iterations if iterations < many_from else 0)
+        assert (4 * n * iterations in gpu.sizes) == (iterations >= many_from)
+
 
 
 def _spec_cases():
@@ -282,7 +282,7 @@ ROUTES = [
     ("monoexp", 12, 4096, 5, 0, "mh_split_kernel<1,2,0>"), ("monoexp", 24, 9600, 5, 0, "mh_split_kernel<1,4,0>"),
     # blocks of 128 past one block an SM where the waves promise enough
     ("monoexp", 12, 200_000, 100, 0, "mh_kernel<1,0,0,128>"), ("monoexp", 12, 240_000, 100, 0, "mh_kernel<1,0,0,256>"),
-    ("monoexp", 12, 400_000, 100, 0, "mh_kernel<1,0,0,256>"), ("smt", 6, 200_000, 100, 0, "mh_kernel<3,0,0,128>"),
+    ("monoexp", 12, 400_000, 100, 0, "mh_kernel<1,0,0,256>"), ("smt", 6, 393_216, 100, 0, "mh_kernel<3,0,0,128>"),
     ("mwi3", 24, 200_000, 100, 0, "mh_kernel<2,0,0,128>"),
 ]
 
