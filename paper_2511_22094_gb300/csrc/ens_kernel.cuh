@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kEnsBlock, 4) ens_kernel(const ModelConst mc, 
                 R th[P];
 #pragma unroll
                 for (int p = 0; p < P; ++p) th[p] = xk[p];
-                LL[lv * L + k] = loglik_any<KIND, PREC, 1, false>(th, y, inv_s2, mc);
+                LL[lv * L + k] = loglik_any<KIND, PREC, 1, kFormEns>(th, y, inv_s2, mc);
 #pragma unroll
                 for (int p = 0; p < P; ++p) {
                     wf_mean[p * nw + lv * L + k] = W(0);
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kEnsBlock, 4) ens_kernel(const ModelConst mc, 
                         // (one echo block at a time: two gained 0.5% with the SMs full, but the
                         // two half-steps' code grew past the instruction cache: 401 voxels x
                         // 64 walkers ran 12% slower)
-                        Lp = loglik_any<KIND, PREC, 1, false>(prop, y, inv_s2, mc);
+                        Lp = loglik_any<KIND, PREC, 1, kFormEns>(prop, y, inv_s2, mc);
                         n_bad[h] += !isfinite(Lp);
                         // log u < (P - 1) log z + L(Y) - L(X_k): the z factor
                         // enters as an offset of the likelihood difference

@@ -434,11 +434,11 @@ static size_t smem_bytes_for(int kind, int prec, int C, int M, int moments_mode,
     return tile_smem_bytes(model_n_par(kind), w, block / C, row_stride_for(kind, M), true, blocked, block);
 }
 
-static const void *mh_kernel_ptr(int kind, int prec, bool trace, int block) {
-    switch (kind) {
+static const void *mh_kernel_ptr(const ModelConst &mc, int prec, bool trace, int block) {
+    switch (mc.kind) {
     case GAC_MODEL_MONOEXP: return mh_ptr_monoexp(prec, trace, block);
     case GAC_MODEL_MWI3: return mh_ptr_mwi3(prec, trace, block);
-    case GAC_MODEL_SMT: return mh_ptr_smt(prec, trace, block);
+    case GAC_MODEL_SMT: return mh_ptr_smt(prec, trace, block, mc.n_acq < kAnchor);
     case GAC_MODEL_AXCAL_SMT: return mh_ptr_axcal(prec, trace, block);
     case GAC_MODEL_LINEAR_TEST: return mh_ptr_linear(prec, trace, block);
     default: return nullptr;
@@ -449,7 +449,7 @@ static const void *mh_kernel_ptr(int kind, int prec, bool trace, int block) {
 // attributes set.
 static gac_status mh_resident(const ModelConst &mc, int prec, bool trace, int C, int moments_mode, int block,
                               LaunchCfg *cfg, int *per_sm) {
-    cfg->fn = mh_kernel_ptr(mc.kind, prec, trace, block);
+    cfg->fn = mh_kernel_ptr(mc, prec, trace, block);
     if (!cfg->fn) return fail(GAC_ERR_INVALID_ARG, "no kernel for kind %d precision %d", mc.kind, prec);
     cfg->block = block;
     cfg->smem = smem_bytes_for(mc.kind, prec, C, mc.n_meas, moments_mode, block);

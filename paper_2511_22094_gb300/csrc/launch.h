@@ -20,7 +20,7 @@ struct LaunchCfg {
 // Per-kind kernels defined in mh_<kind>.cu: (precision, trace, kBlock or kHalfBlock)
 const void *mh_ptr_monoexp(int prec, bool trace, int block);
 const void *mh_ptr_mwi3(int prec, bool trace, int block);
-const void *mh_ptr_smt(int prec, bool trace, int block);
+const void *mh_ptr_smt(int prec, bool trace, int block, bool few_b);  // fewer than kAnchor b-values
 const void *mh_ptr_axcal(int prec, bool trace, int block);
 const void *mh_ptr_linear(int prec, bool trace, int block);
 // In slices (mh_slice_kernel: further arguments ss, pos0, q), MIXED.

@@ -189,12 +189,12 @@ struct PrecTraits<GAC_PREC_FP64> {
     using Acc = PlainSumD;
 };
 
-template <int KIND, int PREC, int REP = gtab_copies(KIND), bool TWO = true>
+template <int KIND, int PREC, int REP = gtab_copies(KIND), int FORM = kFormMh>
 __device__ __forceinline__ typename PrecTraits<PREC>::R loglik_any(
     const typename PrecTraits<PREC>::R *th, const float *y, typename PrecTraits<PREC>::R inv_s2,
     const ModelConst &mc) {
     if constexpr (PREC == GAC_PREC_FP64) return loglik_d<KIND>(th, y, inv_s2, mc);
-    else return loglik_f<KIND, typename PrecTraits<PREC>::Acc, REP, TWO>(th, y, inv_s2, mc);
+    else return loglik_f<KIND, typename PrecTraits<PREC>::Acc, REP, FORM>(th, y, inv_s2, mc);
 }
 
 // MIXED acceptance, FP64 semantics at FP32 cost, from lu32 = __logf(u01_f(w)).
@@ -285,7 +285,7 @@ __device__ __forceinline__ void pool_chains(const W *mean_k, const W *m2_k, int 
 // SLICED = false: t_begin = 0, t_end = I, Welford accumulators in shared
 // memory at the start of `smem`; SLICED = true: chain state and accumulators
 // in `ss` (HBM).
-template <int KIND, int PREC, bool TRACE, bool SLICED, int BLK = kBlock>
+template <int KIND, int PREC, bool TRACE, bool SLICED, int BLK = kBlock, int FORM = kFormMh>
 __device__ __forceinline__ void run_tile(const ModelConst &mc, const RunArgs &ra,
                                          const SliceState &ss, int64_t tile, int t_begin,
                                          int t_end, unsigned char *smem) {
@@ -399,7 +399,7 @@ __device__ __forceinline__ void run_tile(const ModelConst &mc, const RunArgs &ra
                         th[p] = fmaf(mc.ub_f[p] - mc.lb_f[p], u01_f(w0[p]), mc.lb_f[p]);
                 }
             }
-            L = loglik_any<KIND, PREC>(th, y, inv_s2, mc);
+            L = loglik_any<KIND, PREC, gtab_copies(KIND), FORM>(th, y, inv_s2, mc);
 #pragma unroll
             for (int p = 0; p < P; ++p) {
                 wf_mean[p * wf_stride + wf_idx] = W(0);
@@ -461,7 +461,7 @@ __device__ __forceinline__ void run_tile(const ModelConst &mc, const RunArgs &ra
                     }
                 }
                 // a5 + a6: forward model and likelihood
-                const R Lp = loglik_any<KIND, PREC>(prop, y, inv_s2, mc);
+                const R Lp = loglik_any<KIND, PREC, gtab_copies(KIND), FORM>(prop, y, inv_s2, mc);
                 // a7: accept / reject
                 const uint32_t w_acc = w[NW - 1];
                 const bool acc = accept_step<PREC>(Lp, L, w_acc);
@@ -590,13 +590,13 @@ __device__ __forceinline__ void run_tile(const ModelConst &mc, const RunArgs &ra
 }
 
 // One job, one launch: every tile runs all I iterations.
-template <int KIND, int PREC, bool TRACE, int BLK = kBlock>
+template <int KIND, int PREC, bool TRACE, int BLK = kBlock, int FORM = kFormMh>
 __global__ void __launch_bounds__(BLK, mh_min_blocks<KIND, PREC>() * (kBlock / BLK))
     mh_kernel(const ModelConst mc, const RunArgs ra) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SliceState none{};
     for (int64_t tile = blockIdx.x; tile < ra.n_tiles; tile += gridDim.x)
-        run_tile<KIND, PREC, TRACE, false, BLK>(mc, ra, none, tile, 0, ra.I, smem_raw);
+        run_tile<KIND, PREC, TRACE, false, BLK, FORM>(mc, ra, none, tile, 0, ra.I, smem_raw);
 }
 
 // One job in slices of q iterations, for problems of a few waves of tiles: tile k
@@ -615,19 +615,19 @@ __global__ void __launch_bounds__(kBlock, mh_min_blocks<KIND, GAC_PREC_MIXED>())
 }
 
 // The kernel of a kind for (precision, trace, threads per block), or nullptr.
-template <int KIND>
+template <int KIND, int FORM = kFormMh>
 const void *mh_kernel_ptr_of(int prec, bool trace, int block) {
     const bool half = block == kHalfBlock;
     if (half && (trace || prec == GAC_PREC_FP64)) return nullptr;
     switch (prec) {
     case GAC_PREC_MIXED:
         return trace  ? reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_MIXED, true>)
-               : half ? reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_MIXED, false, kHalfBlock>)
-                      : reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_MIXED, false>);
+               : half ? reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_MIXED, false, kHalfBlock, FORM>)
+                      : reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_MIXED, false, kBlock, FORM>);
     case GAC_PREC_FP32:
         return trace  ? reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_FP32, true>)
-               : half ? reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_FP32, false, kHalfBlock>)
-                      : reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_FP32, false>);
+               : half ? reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_FP32, false, kHalfBlock, FORM>)
+                      : reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_FP32, false, kBlock, FORM>);
     case GAC_PREC_FP64:
         return trace ? reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_FP64, true>)
                      : reinterpret_cast<const void *>(&mh_kernel<KIND, GAC_PREC_FP64, false>);

@@ -25,8 +25,8 @@
 //    keeps those too.
 //
 // What bounds it: a lone warp per scheduler issues its instructions in turn
-// and waits out every latency (ncu, AxCaliberSMT at depth 5: 1,295 instructions
-// a round, one issued every 2.7 cycles), so a round costs little more than one
+// and waits out every latency (ncu, AxCaliberSMT at depth 5: 1,260 instructions
+// a round, one issued every 2.6 cycles), so a round costs little more than one
 // iteration of mh_kernel does there, but advances D iterations instead of one.
 // The work per iteration grows by 2^D / D, so the host (choose_depth in
 // gac.cu) takes the deepest tree whose warps still fit the idle issue slots.

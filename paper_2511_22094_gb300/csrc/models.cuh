@@ -126,16 +126,26 @@ constexpr double kTwoPiMilliD = 6.28318530717958648e-3;
 constexpr float kSqrtPiHalf = 0.886226925452758014f;
 constexpr double kSqrtPiHalfD = 0.886226925452758014;
 
+// Forms of the FP32 evaluation, chosen by kernel where the compiled code's size or
+// registers decide: the same values whichever is taken.
+//  kFormTwo    3-pool: two echo blocks side by side, where the sum allows it
+//  kFormShort  SMT: a path of its own for protocols of fewer than six b-values, in
+//              kernels of their own (beside the longer ones' code it cost 24
+//              b-values 7 to 12% and the ensemble kernel's six 4%)
+//  kFormPairs  AxCaliberSMT: the measurements of a partial block in pairs
+constexpr int kFormTwo = 1, kFormShort = 2, kFormPairs = 4;
+constexpr int kFormMh = kFormTwo, kFormMhShort = kFormTwo | kFormShort, kFormEns = kFormPairs;
+
 // ---------------------------------------------------------------- g(x) ----
 // The g(x) table of the block's model, copied from ModelConst by
 // model_smem_load before the first evaluation (the lookups of a warp go to
 // different intervals, which the constant bank would serialise).  REP = 8: eight
-// copies side by side.  A 16-byte load is served eight lanes at a time, and with
-// lane l reading copy l % 8 no two of them meet in a bank.  The AxCaliberSMT MH
-// kernels, bound by shared-memory wavefronts (64 such loads an evaluation; 346
-// wavefronts of a warp's 425 cycles an SM, 71 of them conflicts) and holding 2
-// blocks an SM by registers, take it: 23.9 -> 23.5 ms for 25,001 voxels x 4 x
-// 5,000.  SMT (12 loads) gained 0.5% and keeps one copy, and so do the ensemble
+// copies side by side.  A 16-byte load is served eight lanes at a time, and lane l
+// reads copy l % 8, in a bank group of its own whatever the interval.  The
+// AxCaliberSMT MH kernels, bound by shared-memory wavefronts (64 such loads an
+// evaluation) and holding 2 blocks an SM by registers, take it: 23.9 -> 23.5 ms for
+// 25,001 voxels x 4 x 5,000, although the conflicts that the counter shows only
+// fell from 2.05 to 1.82 a chain-iteration (not explained).  SMT (12 loads) gained 0.5% and keeps one copy, and so do the ensemble
 // kernels, whose walkers need the shared memory (64 walkers with moments over
 // every state lost a block an SM to the copies: 7.7 -> 8.1 ms).
 __host__ __device__ constexpr int gtab_copies(int kind) { return kind == GAC_MODEL_AXCAL_SMT ? 8 : 1; }
@@ -705,7 +715,7 @@ __device__ __forceinline__ void eval_mwi3_f(const float *th, const ModelConst &m
 // branch); otherwise only the first one is, and its two lookups are left out
 // (registration sets smt_b0 for such protocols; of the benchmark's six b-values
 // it saves a sixth of the evaluation).
-template <bool TAIL, bool SEL, class V>
+template <bool TAIL, bool SEL, bool SHORT, class V>
 __device__ __forceinline__ void eval_smt_blocks_f(const float *th, const ModelConst &mc, V &visit) {
     const float f = th[0], da = th[1], dpar = th[2], dperp = th[3];
     const float ddiff = dpar - dperp;
@@ -722,9 +732,9 @@ __device__ __forceinline__ void eval_smt_blocks_f(const float *th, const ModelCo
         else one(k);
     };
     // a full block has no test between its b-values, so their table lookups
-    // overlap; a protocol of one block, full or not, reads them at fixed offsets
-    // (without it, four b-values, 19,000 chains: 0.71 -> 0.78 us an iteration); only
-    // a partial block tests
+    // overlap; a protocol of one block reads them at fixed offsets (SHORT: a partial
+    // one too; without it, four b-values, 19,000 chains: 0.71 -> 0.78 us an
+    // iteration); only a partial block tests
     if (n == kAnchor) {
         first(0);
 #pragma unroll
@@ -732,7 +742,7 @@ __device__ __forceinline__ void eval_smt_blocks_f(const float *th, const ModelCo
         end_block(visit, 0);
         return;
     }
-    if (n < kAnchor) {
+    if (SHORT && n < kAnchor) {
         first(0);
 #pragma unroll
         for (int k = 1; k < kAnchor; ++k)
@@ -756,10 +766,10 @@ __device__ __forceinline__ void eval_smt_blocks_f(const float *th, const ModelCo
     }
 }
 
-template <bool TAIL, class V>
+template <bool TAIL, bool SHORT, class V>
 __device__ __forceinline__ void eval_smt_f(const float *th, const ModelConst &mc, V &&visit) {
-    if (mc.smt_b0) eval_smt_blocks_f<TAIL, false>(th, mc, visit);  // the same branch for every thread
-    else eval_smt_blocks_f<TAIL, true>(th, mc, visit);
+    if (mc.smt_b0) eval_smt_blocks_f<TAIL, false, SHORT>(th, mc, visit);  // the same branch for every thread
+    else eval_smt_blocks_f<TAIL, true, SHORT>(th, mc, visit);
 }
 
 // The cylinder's Gaussian-phase attenuation (Neuman 1974; van Gelderen et al.
@@ -848,8 +858,9 @@ __device__ __forceinline__ void ax_phi_table_f(float R, const AxConst &ax, float
 // for every thread: no shared-memory wavefronts, of which the table lookups
 // leave few; 24.6 -> 23.5 ms for 25,001 voxels x 4 x 5,000).  A full block's
 // lookups overlap; those of a partial one come one by one (in pairs, 16
-// measurements ran 1% slower and 7 in blocks of four and three 3%).
-template <bool TAIL, int REP, class V>
+// measurements ran 1% slower and 7 in blocks of four and three 3%) or, in the
+// ensemble kernel, in pairs (6,000 voxels x 64 walkers, one by one: 11% slower).
+template <bool TAIL, int REP, bool PAIRS, class V>
 __device__ __forceinline__ void eval_axcal_f(const float *th, const ModelConst &mc, V &&visit) {
     const AxConst &ax = mc.ax;
     const float R = 0.5f * th[0], fn = th[1], fcsf = th[2], der = th[3];
@@ -876,7 +887,15 @@ __device__ __forceinline__ void eval_axcal_f(const float *th, const ModelConst &
                 for (int k = 0; k < kAnchor; ++k) one(i0 + k);
                 i = i1;
             }
-            for (; i < i1; ++i) one(i);
+            if constexpr (PAIRS) {
+                for (; i + 1 < i1; i += 2) {
+                    one(i);
+                    one(i + 1);
+                }
+                if (i < i1) one(i);
+            } else {
+                for (; i < i1; ++i) one(i);
+            }
             end_block(visit, 0);
         }
     }
@@ -965,16 +984,16 @@ __device__ __forceinline__ void eval_linear_d(const double *th, const ModelConst
 }
 
 // --------------------------------------------------------- dispatch by kind
-template <int KIND, int REP = gtab_copies(KIND), class V>
+template <int KIND, int REP = gtab_copies(KIND), int FORM = kFormMh, class V>
 __device__ __forceinline__ void eval_f(const float *th, const ModelConst &mc, V &&visit) {
     if constexpr (KIND == GAC_MODEL_MONOEXP) eval_monoexp_f(th, mc, visit);
     else if constexpr (KIND == GAC_MODEL_MWI3) eval_mwi3_f(th, mc, visit);
     else if constexpr (KIND == GAC_MODEL_SMT) {
-        if (mc.gtab_tail) eval_smt_f<true>(th, mc, visit);  // the same branch for every thread
-        else eval_smt_f<false>(th, mc, visit);
+        if (mc.gtab_tail) eval_smt_f<true, (FORM & kFormShort) != 0>(th, mc, visit);  // the same branch for every thread
+        else eval_smt_f<false, (FORM & kFormShort) != 0>(th, mc, visit);
     } else if constexpr (KIND == GAC_MODEL_AXCAL_SMT) {
-        if (mc.gtab_tail) eval_axcal_f<true, REP>(th, mc, visit);
-        else eval_axcal_f<false, REP>(th, mc, visit);
+        if (mc.gtab_tail) eval_axcal_f<true, REP, (FORM & kFormPairs) != 0>(th, mc, visit);
+        else eval_axcal_f<false, REP, (FORM & kFormPairs) != 0>(th, mc, visit);
     }
     else eval_linear_f(th, mc, visit);
 }
@@ -1060,15 +1079,14 @@ struct KahanVisitor : ResidualVisitor<KahanSum> {
     __device__ __forceinline__ void end_blocks() const { acc.end_two(); }
 };
 
-// TWO: the 3-pool model's echo blocks two at a time where the sum allows it.
-template <int KIND, class ACC, int REP = gtab_copies(KIND), bool TWO = true>
+template <int KIND, class ACC, int REP = gtab_copies(KIND), int FORM = kFormMh>
 __device__ __forceinline__ float loglik_f(const float *th, const float *y, float inv_s2,
                                           const ModelConst &mc) {
     ACC acc;
-    if constexpr (TWO && KIND == GAC_MODEL_MWI3 && std::is_same<ACC, KahanSum>::value)
-        eval_f<KIND, REP>(th, mc, KahanVisitor{{acc, y}});
+    if constexpr ((FORM & kFormTwo) && KIND == GAC_MODEL_MWI3 && std::is_same<ACC, KahanSum>::value)
+        eval_f<KIND, REP, FORM>(th, mc, KahanVisitor{{acc, y}});
     else
-        eval_f<KIND, REP>(th, mc, ResidualVisitor<ACC>{acc, y});
+        eval_f<KIND, REP, FORM>(th, mc, ResidualVisitor<ACC>{acc, y});
     return -0.5f * acc.value() * inv_s2;
 }
 

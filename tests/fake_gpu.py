@@ -28,8 +28,10 @@ def short(mangled):
     m = re.search(r"\d([a-z_]+_kernel)(I((?:L[ibx]\d+E|[fd])+)E)?", mangled)
     if not m:
         return mangled
-    args = re.findall(r"L[ibx](\d+)E|([fd])", m.group(3) or "")
-    return m.group(1) + (f"<{','.join(a or b for a, b in args)}>" if args else "")
+    args = [a or b for a, b in re.findall(r"L[ibx](\d+)E|([fd])", m.group(3) or "")]
+    if m.group(1) == "mh_kernel":  # the form: 3 where it is the short protocols' own
+        args[4:] = ["short"] * (args[4] == "3")
+    return m.group(1) + (f"<{','.join(args)}>" if args else "")
 
 
 class FakeGpu:
