@@ -496,10 +496,10 @@ static gac_status plan_launch(const ModelConst &mc, int prec, bool trace, int C,
         // of four warps load them evenly, while two blocks of eight with
         // some idle warps, or a last wave of few large blocks, leave
         // schedulers with twice the warps of others.  Full waves of half
-        // blocks measured up to 3% slower (1.03); where an SM holds more than two of
-        // kBlock, whose ends then spread of themselves, they have to promise 5.5%
-        // (mono-exponential, kBlock -> kHalfBlock: 240,000 chains, 2.2% promised,
-        // 2.39 -> 2.46; 200,000, 5.8%, 2.14 -> 2.02).  3-pool, us per iteration,
+        // blocks measured up to 3% slower (1.03); the mono-exponential ones have
+        // to promise 5.5% (kBlock -> kHalfBlock, us per iteration: 240,000
+        // chains, where they promise 2.2%, 2.39 -> 2.46; 200,000, 5.8%, 2.14 ->
+        // 2.02; SMT, 393,216 chains, 0.4%: 6.44 -> 6.14).  3-pool, us per iteration,
         // kBlock -> kHalfBlock: 14,400 chains 1.79 -> 1.31, 49,380 3.12 ->
         // 2.51, 120,000 6.09 -> 5.24, 200,000 9.01 -> 8.05.  Below one block
         // an SM, tiles shrink in whole warps of chains: each scheduler gets at
@@ -510,7 +510,7 @@ static gac_status plan_launch(const ModelConst &mc, int prec, bool trace, int C,
         half_per_sm = std::min(half_per_sm, 2 * per_sm);  // as many warps: 20 instead of 16 ran 2% slower (3-pool)
         const int vb1 = std::max(1, kBlock / C), vb2 = std::max(1, kHalfBlock / C);
         const double t1 = waves((n_vox + vb1 - 1) / vb1, per_sm);
-        const double t2 = (per_sm > 2 ? 1.055 : 1.03) * waves((n_vox + vb2 - 1) / vb2, half_per_sm);
+        const double t2 = (mc.kind == GAC_MODEL_MONOEXP ? 1.055 : 1.03) * waves((n_vox + vb2 - 1) / vb2, half_per_sm);
         const int64_t want = (chains + sm_count() - 1) / sm_count();  // chains an SM
         if (t2 < t1 || want <= kHalfBlock) {
             *cfg = half;
@@ -518,9 +518,18 @@ static gac_status plan_launch(const ModelConst &mc, int prec, bool trace, int C,
             threads = static_cast<int>(std::min<int64_t>(kHalfBlock, (want + 31) / 32 * 32));
         }
     }
-    if (cfg->block == kBlock && chains < resident * kBlock) {
-        // too few chains for a full tile per resident block: tiles shrink in
-        // whole warps of chains, so that the chains spread over all SMs
+    // Too few chains for a full tile per resident block: tiles shrink in whole
+    // warps of chains, so that the chains spread over all SMs.  Not where they lost
+    // to full tiles on fewer SMs, MIXED and FP32 without a trace: SMT (58,400 chains,
+    // 1.31 -> 1.35 us an iteration), the 3-pool model and AxCaliberSMT with thinned
+    // moments (3-pool, 20,000: 1.58 -> 1.63; over every state, 1.75 -> 1.65, and FP32,
+    // 1.66 -> 1.58, they gain) and the mono-exponential model once every SM has a tile
+    // (100,000: 1.13 -> 1.18; 20,000: 0.54 -> 0.53).
+    const bool two_blocks = mc.kind == GAC_MODEL_MWI3 || mc.kind == GAC_MODEL_AXCAL_SMT;
+    const bool spread = trace || prec == GAC_PREC_FP64 ||
+                        (two_blocks && (prec == GAC_PREC_FP32 || moments_mode == GAC_MOMENTS_ALL_POSTBURNIN)) ||
+                        (mc.kind == GAC_MODEL_MONOEXP && chains < static_cast<int64_t>(sm_count()) * kBlock);
+    if (spread && cfg->block == kBlock && chains < resident * kBlock) {
         const int64_t want = (chains + resident - 1) / resident;  // chains per block
         threads = static_cast<int>(std::min<int64_t>(kBlock, std::max<int64_t>(32, (want + 31) / 32 * 32)));
     }
@@ -778,7 +787,7 @@ static int choose_depth(const ModelConst &mc, const gac_mcmc_opts *o, int64_t n_
     const int64_t schedulers = static_cast<int64_t>(sm_count()) * 4;
     const bool mwi3 = mc.kind == GAC_MODEL_MWI3, mono = mc.kind == GAC_MODEL_MONOEXP;
     const bool all = o->moments_mode == GAC_MOMENTS_ALL_POSTBURNIN;
-    const bool mono4 = !mc.even || mc.n_acq == kAnchor || mc.n_acq >= 48 || (!all && o->thin <= 4);
+    const bool mono4 = !mc.even || mc.n_acq == kAnchor || mc.n_acq >= 48 || (!all && o->thin <= 7);
     for (int depth = 5; depth >= 2; --depth) {
         if (C << depth > kSpecBlock || n_vox * C > (schedulers * 32 * 4 >> depth)) continue;
         // warps a scheduler

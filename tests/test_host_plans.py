@@ -282,7 +282,7 @@ ROUTES = [
     ("monoexp", 12, 4096, 5, 0, "mh_split_kernel<1,2,0>"), ("monoexp", 24, 9600, 5, 0, "mh_split_kernel<1,4,0>"),
     # blocks of 128 past one block an SM where the waves promise enough
     ("monoexp", 12, 200_000, 100, 0, "mh_kernel<1,0,0,128>"), ("monoexp", 12, 240_000, 100, 0, "mh_kernel<1,0,0,256>"),
-    ("monoexp", 12, 400_000, 100, 0, "mh_kernel<1,0,0,256>"), ("smt", 6, 200_000, 100, 0, "mh_kernel<3,0,0,128>"),
+    ("monoexp", 12, 400_000, 100, 0, "mh_kernel<1,0,0,256>"), ("smt", 6, 393_216, 100, 0, "mh_kernel<3,0,0,128>"),
     ("mwi3", 24, 200_000, 100, 0, "mh_kernel<2,0,0,128>"),
     # SMT protocols of fewer than six b-values
     ("smt", 5, 40_000, 100, 0, "mh_kernel<3,0,0,128,short>"), ("smt", 6, 40_000, 100, 0, "mh_kernel<3,0,0,128>"),
