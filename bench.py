@@ -105,12 +105,12 @@ MEASURED = {
     # voxels, all iterations, so every term scales with the voxels) x 3.81;
     # the lines still in L2 when the small launch ends are not counted
     # (~1-3% of its writes).  warp_instr: smsp__inst_executed of small cases.
-    "mwi3_1m": dict(sources="9abb6a90ec58d117", traffic_bytes=(78.36e6 + 1697.09e6) * 1e6 / 262144, warp_instr=912.8),
-    "smt_1p5m": dict(sources="a55baf101b33f8b8", traffic_bytes=(27.15e6 + 1119.01e6) * 1.5e6 / 393216, warp_instr=415.2),
-    "axcal_250k": dict(sources="08a0242b2918f34f", traffic_bytes=(37.45e6 + 908.68e6) * 250000 / 65536, warp_instr=1154.0),
+    "mwi3_1m": dict(sources="2664ef4f4e4ffdaa", traffic_bytes=(77.79e6 + 1696.76e6) * 1e6 / 262144, warp_instr=912.8),
+    "smt_1p5m": dict(sources="6924f0ec4e8d14f6", traffic_bytes=(26.96e6 + 1119.11e6) * 1.5e6 / 393216, warp_instr=415.2),
+    "axcal_250k": dict(sources="4f7596b305ddf7e2", traffic_bytes=(32.74e6 + 907.43e6) * 250000 / 65536, warp_instr=1154.0),
     # the lane-split kernel (2 lanes a chain): the 4,096-voxel workload's data
     # and samples stay in L2, so no DRAM figure
-    "monoexp_4k": dict(sources="afb9ab015406985b", traffic_bytes=None, warp_instr=368.8),
+    "monoexp_4k": dict(sources="400b3b6195959a5e", traffic_bytes=None, warp_instr=368.8),
 }
 
 

@@ -677,7 +677,7 @@ __global__ void __launch_bounds__(kFitBlock, fit_min_blocks(PREC)) fit_step_kern
 // The same over the list of fitted voxels of a masked grid: parameters and
 // moments lie in the list's order, so that their accesses stay whole lines, and
 // the penalised maps once more over the grid, where the neighbours read them.
-// Tiles hold fitted voxels only: 552,960 voxels, 68% inside, 3-pool, 61 -> 49.5 us
+// Tiles hold fitted voxels only: 552,960 voxels, 68% inside, 3-pool, 61 -> 48 us
 // an update.
 template <int KIND, int PREC, bool L1>
 __global__ void __launch_bounds__(kFitBlock, fit_min_blocks(PREC)) fit_list_kernel(const ModelConst mc, const FitArgs<typename PrecTraits<PREC>::R> fa,
@@ -815,7 +815,7 @@ __device__ void fit_check(const FA &fa, int n_blocks, int t, double *red) {
 // a few hundred tiles, by the latency of one update) instead of by the 413 bytes
 // a voxel-update moves when every update is a launch.  Measured, whole calls on
 // a GB300, a launch per update -> this: mono-exponential, 37 x 41 x 9 voxels, 300
-// updates 1.70 -> 0.22 ms; 3-pool, 96 x 96 x 60, 100 updates 5.6 -> 3.3 ms, with
+// updates 1.70 -> 0.21 ms; 3-pool, 96 x 96 x 60, 100 updates 5.6 -> 3.3 ms, with
 // a mask of 68% of it 5.7 -> 2.4 ms.
 constexpr int kFitChunk = 128;
 constexpr int kFitLossThreads = 128;

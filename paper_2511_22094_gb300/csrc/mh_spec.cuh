@@ -31,7 +31,7 @@
 // The work per iteration grows by 2^D / D, so the host (choose_depth in
 // gac.cu) takes the deepest tree whose warps still fit the idle issue slots.
 // Measured on GB300, before -> with it: AxCaliberSMT, 100 voxels x 4 chains x
-// 25,000 iterations (depth 5): 41.4 -> 7.97 ms; 3-pool, 301 voxels x 4 x 5,000,
+// 25,000 iterations (depth 5): 41.4 -> 7.94 ms; 3-pool, 301 voxels x 4 x 5,000,
 // host arrays (depth 4): 5.59 -> 1.58 ms; SMT, 600 chains x 1,000 (depth 5): 0.59 ->
 // 0.15 ms.
 //
