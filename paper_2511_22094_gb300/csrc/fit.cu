@@ -1357,15 +1357,16 @@ static gac_status fit_run_prec(const ModelConst &mc, const gac_fit_opts *o, cons
     const bool rules = o->tol > 0 || o->convergence_value > 0;
     // Many updates a launch.  With stopping rules a launch of 32 runs up to 31
     // updates past the stop and then those before it again, while the grid's
-    // launches after a stop return at once.  In FP32, with at most three quarters of
-    // the persistent warps' lanes, that is never slower, wherever the fit stops (ms,
+    // launches after a stop return at once.  In FP32, with at most a voxel a lane of
+    // the persistent warps (three quarters of them for the 3-pool model, whose
+    // updates are the longest), that is never slower, wherever the fit stops (ms,
     // grid -> 32 a launch, stop at update 1, 33, 129 of 200: 3-pool, 51,200 voxels 0.36
-    // -> 0.24, 0.54 -> 0.38, 1.51 -> 0.83; SMT 0.35 -> 0.18, 0.55 -> 0.29, 1.59 -> 0.58;
-    // mono-exponential, 13,653 voxels 0.35 -> 0.12, 0.36 -> 0.17, 0.93 -> 0.32).  Not so
-    // beyond that (3-pool, 97,200 voxels, stop at 2: 0.35 -> 0.37; 552,960 0.53 -> 1.27)
-    // and in FP64 (3-pool, 13,653 voxels: 0.46 -> 6.4, at 33 7.4 -> 12.6).
+    // -> 0.24, 0.54 -> 0.38, 1.51 -> 0.83; SMT, 97,200 0.36 -> 0.25, 0.70 -> 0.39, 2.10 ->
+    // 0.83; mono-exponential, 97,200 0.36 -> 0.17, 0.48 -> 0.26, 1.25 -> 0.52).  Not so
+    // beyond that (3-pool, 97,200 voxels, stop at 2: 0.35 -> 0.37; SMT, 552,960 0.39 ->
+    // 0.68) and in FP64 (3-pool, 13,653 voxels: 0.46 -> 6.4, at 33 7.4 -> 12.6).
     const int64_t n_fit = d_mask ? n_mask : N;
-    bool many = !coupled && (!rules || (PREC == GAC_PREC_FP32 && 4 * n_fit <= 3 * one_round));
+    bool many = !coupled && (!rules || (PREC == GAC_PREC_FP32 && 4 * n_fit <= (P <= 4 ? 4 : 3) * one_round));
     // One update a launch, where the loss shares of two pass 64 MB, gains nothing
     // over the grid's kernel, which loads a tile while it computes another, unless
     // that visits voxels outside the mask (mono-exponential, 16.2 million voxels, 20

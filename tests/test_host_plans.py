@@ -192,16 +192,18 @@ def test_losses_of_few_updates_are_summed_by_the_whole_gpu(fake, n, updates):
         assert grid * count * block // 32 >= min(8 * 152, n)
 
 
-@pytest.mark.parametrize("precision,n,kernel", [(1, 72_960, "fit_many"), (1, 72_961, "fit_step"), (2, 100, "fit_step")])
-def test_stopping_rules_run_few_updates_past_the_stop(fake, precision, n, kernel):
+@pytest.mark.parametrize("w,precision,n,kernel", [
+    (W.MONOEXP_4K, 1, 97_280, "fit_many"), (W.MONOEXP_4K, 1, 97_281, "fit_step"), (W.MONOEXP_4K, 2, 100, "fit_step"),
+    (W.MWI3_1M, 1, 72_960, "fit_many"), (W.MWI3_1M, 1, 72_961, "fit_step")])
+def test_stopping_rules_run_few_updates_past_the_stop(fake, w, precision, n, kernel):
     """A launch of many updates runs past a stop: only where that costs less than the idle launches
-    it saves, in FP32 with a tile for at most three warps of four."""
+    it saves, in FP32 with at most one tile a warp (3-pool: a tile for three warps of four)."""
     _, gpu = fake
     for rules in (dict(tol=1e-300), dict(convergence_value=1e-300)):
         for extra in (0, 1000):  # voxels outside the mask
             mask = np.r_[np.ones(n, np.uint8), np.zeros(extra, np.uint8)]
             gpu.reset()
-            _fit(fake, W.MONOEXP_4K, (n + extra, 1, 1), mask=mask, iterations=33, precision=precision, **rules)
+            _fit(fake, w, (n + extra, 1, 1), mask=mask, iterations=33, precision=precision, **rules)
             fits = [x.split("_kernel")[0] for x in gpu.names() if x.startswith(("fit_many", "fit_step", "fit_list"))]
             assert fits == [kernel] * (2 if kernel == "fit_many" else 33)
 
